@@ -70,8 +70,6 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
             BOut out, int smem_vec)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ T red[BLOCK / 32];
-    __shared__ float redf[BLOCK / 32];
     __shared__ int s_sys;
     for (;;) {
         if (threadIdx.x == 0) s_sys = (int)atomicAdd(queue, 1u);
@@ -84,7 +82,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
         BlockRows<BLOCK> g((int)(row_off[s + 1] - ro));
         const SysOut o = solve_rows<T, BLOCK, SOLVER, MIXED>(
             g, rp_all + ro + s, col_all + nnz_off[s], val_all + nnz_off[s], MIXED ? val32_all + nnz_off[s] : nullptr,
-            b_all + ro, x_all + ro, work, nrows, ro, smem_vec ? smem : nullptr, red, redf, tol, maxit);
+            b_all + ro, x_all + ro, work, nrows, ro, smem_vec ? smem : nullptr, tol, maxit);
         if (threadIdx.x == 0) {
             out.status[s] = o.status;
             out.iters[s] = o.iters;
@@ -102,12 +100,14 @@ int launch_batch_t(spx_ctx *ctx, spx_batch *B, const T *b, T *x, double tol, int
 {
     auto kern = k_batch<T, BLOCK, SOLVER, MIXED>;
     int smem = (int)(B->max_n * (MIXED ? 8 : sizeof(T)));
-    const int smem_vec = smem <= ctx->max_smem_optin - 1024 ? 1 : 0;  // else the vector stays in global memory
+    // the opt-in is made once, to all that the kernel's static part leaves: the
+    // server's batch lanes launch this kernel from several threads with different
+    // sizes, and lowering the limit between another thread's opt-in and its launch
+    // got that launch refused
+    int smem_max = 0;
+    SPX_TRY(smem_optin(reinterpret_cast<const void *>(kern), -1, &smem_max));
+    const int smem_vec = smem <= smem_max ? 1 : 0;  // else the vector stays in global memory
     if (!smem_vec) smem = 0;
-    // the opt-in only ever grows (smem_optin): the server's batch lanes launch this
-    // kernel from several threads with different sizes, and lowering the limit
-    // between another thread's opt-in and its launch got that launch refused
-    SPX_TRY(smem_optin(reinterpret_cast<const void *>(kern), smem));
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BLOCK, smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;

@@ -17,17 +17,16 @@ __global__ void __launch_bounds__(kDotBlock)
     k_dot(int64_t n, const T *__restrict__ x, const T *__restrict__ y, T *partials, unsigned *ticket,
           T *result)
 {
-    __shared__ T red[kDotBlock / 32];
     T s = T(0);
     for (int64_t i = blockIdx.x * (int64_t)kDotBlock + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * kDotBlock)
         s = fma(x[i], y[i], s);
-    s = block_sum<T, kDotBlock>(s, red);
+    s = block_sum<T, kDotBlock>(s);
     if (threadIdx.x == 0) partials[blockIdx.x] = s;
     if (!last_block(ticket, gridDim.x)) return;
     T t = T(0);
     for (unsigned b = threadIdx.x; b < gridDim.x; b += kDotBlock) t += ldcg(partials + b);
-    t = block_sum<T, kDotBlock>(t, red);
+    t = block_sum<T, kDotBlock>(t);
     if (threadIdx.x == 0) *result = t;
 }
 

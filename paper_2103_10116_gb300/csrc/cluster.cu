@@ -52,10 +52,10 @@ struct ClOut {
 // in k_cluster_cg.  bc is rewritten by the next sum only after its block
 // barriers, which every thread reaches after reading it.
 template <class T, int CL, int BLOCK>
-__device__ __forceinline__ T cluster_sum(cg::cluster_group &cl, T v, T *red, T *part, int slot)
+__device__ __forceinline__ T cluster_sum(cg::cluster_group &cl, T v, T *part, int slot)
 {
     __shared__ T bc;
-    v = block_sum<T, BLOCK>(v, red);
+    v = block_sum<T, BLOCK>(v);
     if (threadIdx.x == 0) part[slot] = v;
     cl.sync();
     if (threadIdx.x < 32) {
@@ -100,7 +100,6 @@ __global__ void __launch_bounds__(BLOCK, 1)  // one block per SM: no register ca
     T *rs = ps + R;
     T *xs = rs + R;
     T *qs = xs + R;
-    __shared__ T red[BLOCK / 32];
     __shared__ T part[4];
     __shared__ T sc[2];  // alpha and beta, computed by thread 0 (a division is many FP64 instructions)
     const int tid = threadIdx.x;
@@ -111,7 +110,7 @@ __global__ void __launch_bounds__(BLOCK, 1)  // one block per SM: no register ca
         bb = fma(bi, bi, bb);
         xs[i] = x[r0 + i];
     }
-    bb = cluster_sum<T, CL, BLOCK>(cl, bb, red, part, 2);
+    bb = cluster_sum<T, CL, BLOCK>(cl, bb, part, 2);
     ClOut res{SPX_MAX_ITER, 0, 0, 0.0};
     if (bb == T(0)) {
         for (int i = tid; i < nr; i += BLOCK) xs[i] = T(0);
@@ -129,7 +128,7 @@ __global__ void __launch_bounds__(BLOCK, 1)  // one block per SM: no register ca
                 rs[i] = ri;
                 rho = fma(ri, ri, rho);
             }
-            rho = cluster_sum<T, CL, BLOCK>(cl, rho, red, part, 3);  // every block is past its reads of ps
+            rho = cluster_sum<T, CL, BLOCK>(cl, rho, part, 3);  // every block is past its reads of ps
             for (int i = tid; i < nr; i += BLOCK) ps[i] = rs[i];
             cl.sync();
             T last = rho;  // the last recurrence residual, squared
@@ -146,7 +145,7 @@ __global__ void __launch_bounds__(BLOCK, 1)  // one block per SM: no register ca
                     qs[i] = qi;
                     pq = fma(ps[i], qi, pq);
                 }
-                pq = cluster_sum<T, CL, BLOCK>(cl, pq, red, part, 0);
+                pq = cluster_sum<T, CL, BLOCK>(cl, pq, part, 0);
                 if (pq == T(0)) {
                     status = SPX_BREAKDOWN;
                     break;
@@ -161,7 +160,7 @@ __global__ void __launch_bounds__(BLOCK, 1)  // one block per SM: no register ca
                     rs[i] = ri;
                     rr = fma(ri, ri, rr);
                 }
-                rr = cluster_sum<T, CL, BLOCK>(cl, rr, red, part, 1);
+                rr = cluster_sum<T, CL, BLOCK>(cl, rr, part, 1);
                 ++iters;
                 last = rr;
                 if (rr <= tol2) {
@@ -189,7 +188,7 @@ __global__ void __launch_bounds__(BLOCK, 1)  // one block per SM: no register ca
                 const T ri = b[r0 + i] - dist_row_dot<T>(cl, rp, col, val, ps, lg, r0 + i);
                 rt = fma(ri, ri, rt);
             }
-            rt = cluster_sum<T, CL, BLOCK>(cl, rt, red, part, 2);
+            rt = cluster_sum<T, CL, BLOCK>(cl, rt, part, 2);
             res.relres = (double)sqrt(rt / bb);
             if (rt <= tol2) break;
             if (restart == 3) {
@@ -340,8 +339,6 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
                     const float *__restrict__ val32, const T *__restrict__ b, T *__restrict__ x, T *__restrict__ work,
                     T tol, long long maxit, SysOut *out)
 {
-    __shared__ T red[BLOCK / 32];
-    __shared__ float redf[BLOCK / 32];
     __shared__ double part[8];
     __shared__ double bc[2];
     const int rank = (int)cg::this_cluster().block_rank();
@@ -351,8 +348,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
     g.hi = min(n, g.lo + R);
     g.part = part;
     g.bc = bc;
-    const SysOut o = solve_rows<T, BLOCK, SOLVER, MIXED>(g, rp, col, val, val32, b, x, work, n, 0, nullptr, red,
-                                                         redf, tol, maxit);
+    const SysOut o = solve_rows<T, BLOCK, SOLVER, MIXED>(g, rp, col, val, val32, b, x, work, n, 0, nullptr, tol, maxit);
     if (rank == 0 && threadIdx.x == 0) *out = o;
     cg::this_cluster().sync();  // no block exits while another may still read its shared memory
 }

@@ -8,7 +8,7 @@
 // cluster, block k owning a contiguous slice of rows (the single-launch solve
 // of a mid-size system, cluster.cu).  A group provides
 //   lo, hi       the rows of this block;
-//   sum(v, red)  the sum of v over the group's threads, the same bits in every
+//   sum(v)       the sum of v over the group's threads, the same bits in every
 //                thread of every block (fixed reduction order);
 //   sum2(a, b)   two such sums at the cost of one group barrier;
 //   sync()       a barrier after which every block sees the others' writes of
@@ -36,11 +36,18 @@ template <int BLOCK> struct BlockRows {
     int lo, hi;
     __device__ explicit BlockRows(int n) : lo(0), hi(n) {}
     __device__ __forceinline__ void sync() { __syncthreads(); }
-    template <class T> __device__ __forceinline__ T sum(T v, T *red) { return block_sum<T, BLOCK>(v, red); }
-    template <class T> __device__ __forceinline__ void sum2(T &a, T &b, T *red)
+    template <class T> __device__ __forceinline__ T sum(T v) { return block_sum<T, BLOCK>(v); }
+    template <class T> __device__ __forceinline__ void sum2(T &a, T &b)
     {
-        a = block_sum<T, BLOCK>(a, red);
-        b = block_sum<T, BLOCK>(b, red);
+        if constexpr (BLOCK < 1024) {
+            T v[2] = {a, b};
+            block_sums<T, BLOCK, 2>(v);
+            a = v[0];
+            b = v[1];
+        } else {  // one sum's buffer: the batched kernel keeps its shared memory for the gathered vector
+            a = block_sum<T, BLOCK>(a);
+            b = block_sum<T, BLOCK>(b);
+        }
     }
     template <class T> __device__ __forceinline__ T gather(const T *v, int c) const { return v[c]; }
 };
@@ -73,9 +80,9 @@ template <int CL, int BLOCK, int UROWS = 2> struct ClusterRows {
             if (threadIdx.x == 0) bc[which] = (double)p;
         }
     }
-    template <class T> __device__ __forceinline__ T sum(T v, T *red)
+    template <class T> __device__ __forceinline__ T sum(T v)
     {
-        v = block_sum<T, BLOCK>(v, red);
+        v = block_sum<T, BLOCK>(v);
         if (threadIdx.x == 0) part[slot] = (double)v;  // exact for float and double
         sync();
         combine<T>(0);
@@ -84,10 +91,17 @@ template <int CL, int BLOCK, int UROWS = 2> struct ClusterRows {
         slot = (slot + 1) & 3;
         return s;
     }
-    template <class T> __device__ __forceinline__ void sum2(T &a, T &b, T *red)
+    template <class T> __device__ __forceinline__ void sum2(T &a, T &b)
     {
-        a = block_sum<T, BLOCK>(a, red);
-        b = block_sum<T, BLOCK>(b, red);
+        if constexpr (BLOCK < 1024) {
+            T v[2] = {a, b};
+            block_sums<T, BLOCK, 2>(v);
+            a = v[0];
+            b = v[1];
+        } else {  // one sum's buffer: the batched kernel keeps its shared memory for the gathered vector
+            a = block_sum<T, BLOCK>(a);
+            b = block_sum<T, BLOCK>(b);
+        }
         if (threadIdx.x == 0) {
             part[slot] = (double)a;
             part[4 + slot] = (double)b;
@@ -173,12 +187,12 @@ template <class T> __device__ __forceinline__ T share_scalar(T v, T *slot)
 template <class T, class V, int BLOCK, class G>
 __device__ int cg_rows(G &g, const int *__restrict__ rp, const int *__restrict__ col, const V *__restrict__ val,
                        const T *__restrict__ b, T *__restrict__ x, T *__restrict__ r, T *__restrict__ q, T *ps,
-                       T *red, T tol, long long maxit, bool zero_x0, bool check_true, long long &iters, T &relres)
+                       T tol, long long maxit, bool zero_x0, bool check_true, long long &iters, T &relres)
 {
     __shared__ T sc[2];
     T bb = T(0);
     SPX_OWN_ROWS(i) bb = fma(b[i], b[i], bb);
-    bb = g.sum(bb, red);
+    bb = g.sum(bb);
     if (bb == T(0)) {
         SPX_OWN_ROWS(i) x[i] = T(0);
         relres = T(0);
@@ -197,7 +211,7 @@ __device__ int cg_rows(G &g, const int *__restrict__ rp, const int *__restrict__
             r[i] = ri;
             rho = fma(ri, ri, rho);
         });
-        rho = g.sum(rho, red);  // every gather of ps is done
+        rho = g.sum(rho);  // every gather of ps is done
         SPX_OWN_ROWS(i) ps[i] = r[i];
         g.sync();
         T last = rho;  // the last recurrence residual, squared
@@ -208,7 +222,7 @@ __device__ int cg_rows(G &g, const int *__restrict__ rp, const int *__restrict__
                 q[i] = qi;
                 pq = fma(ps[i], qi, pq);
             });
-            pq = g.sum(pq, red);
+            pq = g.sum(pq);
             if (pq == T(0)) {
                 status = SPX_BREAKDOWN;
                 break;
@@ -222,7 +236,7 @@ __device__ int cg_rows(G &g, const int *__restrict__ rp, const int *__restrict__
                 r[i] = ri;
                 rr = fma(ri, ri, rr);
             }
-            rr = g.sum(rr, red);
+            rr = g.sum(rr);
             ++iters;
             last = rr;
             if (rr <= tol2) {
@@ -245,7 +259,7 @@ __device__ int cg_rows(G &g, const int *__restrict__ rp, const int *__restrict__
             const T ri = b[i] - t;
             rt = fma(ri, ri, rt);
         });
-        rt = g.sum(rt, red);
+        rt = g.sum(rt);
         relres = sqrt(rt / bb);
         if (rt <= tol2) break;
         if (restart == kGroupMaxRestarts) {
@@ -262,14 +276,14 @@ __device__ int cg_rows(G &g, const int *__restrict__ rp, const int *__restrict__
 template <class T, class V, int BLOCK, class G>
 __device__ int bicgstab_rows(G &g, const int *__restrict__ rp, const int *__restrict__ col,
                              const V *__restrict__ val, const T *__restrict__ b, T *__restrict__ x, T *const *w, T *ps,
-                             T *red, T tol, long long maxit, bool zero_x0, bool check_true, long long &iters,
+                             T tol, long long maxit, bool zero_x0, bool check_true, long long &iters,
                              T &relres)
 {
     __shared__ T sc[3];
     T *r = w[0], *rh = w[1], *p = w[2], *v = w[3], *s = w[4], *t = w[5];
     T bb = T(0);
     SPX_OWN_ROWS(i) bb = fma(b[i], b[i], bb);
-    bb = g.sum(bb, red);
+    bb = g.sum(bb);
     if (bb == T(0)) {
         SPX_OWN_ROWS(i) x[i] = T(0);
         relres = T(0);
@@ -290,7 +304,7 @@ __device__ int bicgstab_rows(G &g, const int *__restrict__ rp, const int *__rest
             v[i] = T(0);
             rr0 = fma(ri, ri, rr0);
         });
-        rr0 = g.sum(rr0, red);
+        rr0 = g.sum(rr0);
         T rho = T(1), alpha = T(1), omega = T(1), rho1 = rr0;
         T last = rr0;  // the last recurrence residual, squared
         status = rr0 <= tol2 ? SPX_CONVERGED : SPX_MAX_ITER;
@@ -312,7 +326,7 @@ __device__ int bicgstab_rows(G &g, const int *__restrict__ rp, const int *__rest
                 v[i] = vi;
                 rv = fma(rh[i], vi, rv);
             });
-            rv = g.sum(rv, red);
+            rv = g.sum(rv);
             if (rv == T(0)) {
                 status = SPX_BREAKDOWN;
                 break;
@@ -326,7 +340,7 @@ __device__ int bicgstab_rows(G &g, const int *__restrict__ rp, const int *__rest
                 ps[i] = si;
                 ss = fma(si, si, ss);
             }
-            ss = g.sum(ss, red);  // its group barrier also publishes ps
+            ss = g.sum(ss);  // its group barrier also publishes ps
             ++iters;
             if (ss <= tol2) {
                 SPX_OWN_ROWS(i)
@@ -345,7 +359,7 @@ __device__ int bicgstab_rows(G &g, const int *__restrict__ rp, const int *__rest
                 ts = fma(ti, s[i], ts);
                 tt = fma(ti, ti, tt);
             });
-            g.sum2(ts, tt, red);
+            g.sum2(ts, tt);
             if (tt == T(0)) {
                 status = SPX_BREAKDOWN;
                 break;
@@ -360,7 +374,7 @@ __device__ int bicgstab_rows(G &g, const int *__restrict__ rp, const int *__rest
                 rr = fma(ri, ri, rr);
                 rhr = fma(rh[i], ri, rhr);
             }
-            g.sum2(rr, rhr, red);
+            g.sum2(rr, rhr);
             last = rr;
             if (rr <= tol2) {
                 status = SPX_CONVERGED;
@@ -383,7 +397,7 @@ __device__ int bicgstab_rows(G &g, const int *__restrict__ rp, const int *__rest
             const T ri = b[i] - t;
             rt = fma(ri, ri, rt);
         });
-        rt = g.sum(rt, red);
+        rt = g.sum(rt);
         relres = sqrt(rt / bb);
         if (rt <= tol2) break;
         if (restart == kGroupMaxRestarts) {
@@ -401,7 +415,7 @@ __device__ int bicgstab_rows(G &g, const int *__restrict__ rp, const int *__rest
 // iterations without halving.
 template <class T, class V, int BLOCK, class G>
 __device__ int cgs_rows(G &g, const int *__restrict__ rp, const int *__restrict__ col, const V *__restrict__ val,
-                        const T *__restrict__ b, T *__restrict__ x, T *const *w, T *ps, T *red, T tol,
+                        const T *__restrict__ b, T *__restrict__ x, T *const *w, T *ps, T tol,
                         long long maxit, bool zero_x0, bool check_true, long long &iters, T &relres, int stall = 0)
 {
     T mark2 = T(1);  // the squared relative residual the stall test measures against
@@ -410,7 +424,7 @@ __device__ int cgs_rows(G &g, const int *__restrict__ rp, const int *__restrict_
     T *r = w[0], *rh = w[1], *p = w[2], *u = w[3], *q = w[4], *v = w[5];
     T bb = T(0);
     SPX_OWN_ROWS(i) bb = fma(b[i], b[i], bb);
-    bb = g.sum(bb, red);
+    bb = g.sum(bb);
     if (bb == T(0)) {
         SPX_OWN_ROWS(i) x[i] = T(0);
         relres = T(0);
@@ -431,7 +445,7 @@ __device__ int cgs_rows(G &g, const int *__restrict__ rp, const int *__restrict_
             u[i] = ri;
             rr0 = fma(ri, ri, rr0);
         });
-        rr0 = g.sum(rr0, red);  // (its barrier also ends every gather of ps)
+        rr0 = g.sum(rr0);  // (its barrier also ends every gather of ps)
         SPX_OWN_ROWS(i) ps[i] = p[i];
         g.sync();
         T rho = rr0;
@@ -447,7 +461,7 @@ __device__ int cgs_rows(G &g, const int *__restrict__ rp, const int *__restrict_
                 v[i] = vi;
                 rv = fma(rh[i], vi, rv);
             });
-            rv = g.sum(rv, red);
+            rv = g.sum(rv);
             if (rv == T(0)) {
                 status = SPX_BREAKDOWN;
                 break;
@@ -469,7 +483,7 @@ __device__ int cgs_rows(G &g, const int *__restrict__ rp, const int *__restrict_
                 rr = fma(ri, ri, rr);
                 rhr = fma(rh[i], ri, rhr);
             });
-            g.sum2(rr, rhr, red);
+            g.sum2(rr, rhr);
             ++iters;
             last = rr;
             if (rr <= tol2) {
@@ -507,7 +521,7 @@ __device__ int cgs_rows(G &g, const int *__restrict__ rp, const int *__restrict_
             const T ri = b[i] - t;
             rt = fma(ri, ri, rt);
         });
-        rt = g.sum(rt, red);
+        rt = g.sum(rt);
         relres = sqrt(rt / bb);
         if (rt <= tol2) break;
         if (restart == kGroupMaxRestarts) {
@@ -536,13 +550,13 @@ __device__ int cg_reliable_rows(G &g, const int *__restrict__ rp, const int *__r
                                 const double *__restrict__ val, const float *__restrict__ v32,
                                 const double *__restrict__ b, double *__restrict__ x, double *__restrict__ r64,
                                 float *__restrict__ r32, float *__restrict__ y, float *__restrict__ q, float *p,
-                                double *red, float *redf, double tol, long long maxit, long long &iters,
+                                double tol, long long maxit, long long &iters,
                                 double &relres, int &updates)
 {
     __shared__ float sc[2];
     double bb = 0.0;
     SPX_OWN_ROWS(i) bb = fma(b[i], b[i], bb);
-    bb = g.sum(bb, red);
+    bb = g.sum(bb);
     if (bb == 0.0) {
         SPX_OWN_ROWS(i) x[i] = 0.0;
         relres = 0.0;
@@ -559,7 +573,7 @@ __device__ int cg_reliable_rows(G &g, const int *__restrict__ rp, const int *__r
             r64[i] = ri;
             rr = fma(ri, ri, rr);
         });
-        return g.sum(rr, red);
+        return g.sum(rr);
     };
     double rr64 = fp64_residual();
     relres = sqrt(rr64 / bb);
@@ -573,7 +587,7 @@ __device__ int cg_reliable_rows(G &g, const int *__restrict__ rp, const int *__r
         y[i] = 0.f;
         rho = fmaf(ri, ri, rho);
     }
-    rho = g.sum(rho, redf);  // its group barrier also publishes p
+    rho = g.sum(rho);  // its group barrier also publishes p
     float maxr2 = rho;
     int status = SPX_MAX_ITER;
     while (iters < maxit) {
@@ -582,7 +596,7 @@ __device__ int cg_reliable_rows(G &g, const int *__restrict__ rp, const int *__r
             q[i] = qi;
             pq = fmaf(p[i], qi, pq);
         });
-        pq = g.sum(pq, redf);
+        pq = g.sum(pq);
         if (pq == 0.f) {
             status = SPX_BREAKDOWN;
             break;
@@ -596,7 +610,7 @@ __device__ int cg_reliable_rows(G &g, const int *__restrict__ rp, const int *__r
             r32[i] = ri;
             rr = fmaf(ri, ri, rr);
         }
-        rr = g.sum(rr, redf);
+        rr = g.sum(rr);
         ++iters;
         if (rr > maxr2) maxr2 = rr;
         if (rr <= tol2 || iters >= maxit || rr < kRuDelta2 * maxr2) {  // reliable update
@@ -620,7 +634,7 @@ __device__ int cg_reliable_rows(G &g, const int *__restrict__ rp, const int *__r
                 r32[i] = ri;
                 r2 = fmaf(ri, ri, r2);
             }
-            rr = g.sum(r2, redf);
+            rr = g.sum(r2);
             maxr2 = rr;
         }
         const float beta = share_scalar(threadIdx.x == 0 ? rr / rho : 0.f, &sc[1]);
@@ -659,7 +673,7 @@ template <class T, int BLOCK, int SOLVER, bool MIXED, class G>
 __device__ SysOut solve_rows(G &g, const int *__restrict__ rp, const int *__restrict__ col,
                              const T *__restrict__ val_all, const float *__restrict__ v32, const T *__restrict__ b,
                              T *__restrict__ x, T *__restrict__ work, int64_t nrows, int64_t ro, void *smem_vec,
-                             T *red, float *redf, T tol, long long maxit)
+                             T tol, long long maxit)
 {
     long long iters = 0;
     T relres = T(0);
@@ -670,13 +684,13 @@ __device__ SysOut solve_rows(G &g, const int *__restrict__ rp, const int *__rest
         T *w[6];
         for (int k = 0; k < 6; ++k) w[k] = work + (int64_t)k * nrows + ro;
         if constexpr (SOLVER == SPX_CG)
-            status = cg_rows<T, T, BLOCK>(g, rp, col, val_all, b, x, w[0], w[1], ps, red, tol, maxit, false, true,
+            status = cg_rows<T, T, BLOCK>(g, rp, col, val_all, b, x, w[0], w[1], ps, tol, maxit, false, true,
                                           iters, relres);
         else if constexpr (SOLVER == SPX_CGS)
-            status = cgs_rows<T, T, BLOCK>(g, rp, col, val_all, b, x, w, ps, red, tol, maxit, false, true, iters,
+            status = cgs_rows<T, T, BLOCK>(g, rp, col, val_all, b, x, w, ps, tol, maxit, false, true, iters,
                                            relres);
         else
-            status = bicgstab_rows<T, T, BLOCK>(g, rp, col, val_all, b, x, w, ps, red, tol, maxit, false, true,
+            status = bicgstab_rows<T, T, BLOCK>(g, rp, col, val_all, b, x, w, ps, tol, maxit, false, true,
                                                 iters, relres);
     } else {
         static_assert(sizeof(T) == 8, "refinement runs on FP64 systems");
@@ -691,16 +705,15 @@ __device__ SysOut solve_rows(G &g, const int *__restrict__ rp, const int *__rest
         float *ps32 = smem_vec ? reinterpret_cast<float *>(smem_vec) : reinterpret_cast<float *>(wd + 7 * nrows) + ro;
         const double *bd = reinterpret_cast<const double *>(b);
         double *xd = reinterpret_cast<double *>(x);
-        double *redd = reinterpret_cast<double *>(red);
         if constexpr (SOLVER == SPX_CG) {  // reliable updates instead of restarted refinement cycles
             double rel = 0.0;
-            status = cg_reliable_rows<BLOCK>(g, rp, col, val, v32, bd, xd, r64, r32, d32, fv[0], ps32, redd, redf,
+            status = cg_reliable_rows<BLOCK>(g, rp, col, val, v32, bd, xd, r64, r32, d32, fv[0], ps32,
                                              (double)tol, maxit, iters, rel, outer);
             return SysOut{status, outer, iters, rel};
         }
         double bb = 0.0;
         SPX_OWN_ROWS(i) bb = fma(bd[i], bd[i], bb);
-        bb = g.sum(bb, redd);
+        bb = g.sum(bb);
         status = SPX_MAX_ITER;
         if (bb == 0.0) {
             SPX_OWN_ROWS(i) xd[i] = 0.0;
@@ -715,7 +728,7 @@ __device__ SysOut solve_rows(G &g, const int *__restrict__ rp, const int *__rest
                 r64[i] = ri;
                 rr = fma(ri, ri, rr);
             });
-            rr = g.sum(rr, redd);
+            rr = g.sum(rr);
             relres = (T)sqrt(rr / bb);
             if (rr <= (double)tol * (double)tol * bb) {
                 status = SPX_CONVERGED;
@@ -729,13 +742,13 @@ __device__ SysOut solve_rows(G &g, const int *__restrict__ rp, const int *__rest
             // at most kIrInnerCap inner iterations per refinement cycle
             const long long cyc_max = min(maxit, iters + (long long)kIrInnerCap);
             if constexpr (SOLVER == SPX_CG)
-                cg_rows<float, float, BLOCK>(g, rp, col, v32, r32, d32, fv[0], fv[1], ps32, redf, 1e-4f, cyc_max,
+                cg_rows<float, float, BLOCK>(g, rp, col, v32, r32, d32, fv[0], fv[1], ps32, 1e-4f, cyc_max,
                                              true, false, iters, rel32);
             else if constexpr (SOLVER == SPX_CGS)
-                cgs_rows<float, float, BLOCK>(g, rp, col, v32, r32, d32, fv, ps32, redf, 1e-4f, cyc_max, true, false,
+                cgs_rows<float, float, BLOCK>(g, rp, col, v32, r32, d32, fv, ps32, 1e-4f, cyc_max, true, false,
                                               iters, rel32, kIrCgsStall);
             else
-                bicgstab_rows<float, float, BLOCK>(g, rp, col, v32, r32, d32, fv, ps32, redf, 1e-4f, cyc_max, true,
+                bicgstab_rows<float, float, BLOCK>(g, rp, col, v32, r32, d32, fv, ps32, 1e-4f, cyc_max, true,
                                                    false, iters, rel32);
             SPX_OWN_ROWS(i) xd[i] = fma(rn, (double)d32[i], xd[i]);
             __syncthreads();

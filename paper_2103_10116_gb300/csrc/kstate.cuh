@@ -221,31 +221,43 @@ template <class T> __device__ __forceinline__ void run_fin(int fin, void *state,
 // Grid-wide finish of up to two dot products: block partials, then the last
 // block to arrive sums them in block order (deterministic), stores dots[0..1]
 // (if dots != null) and runs the scalar update.  Every block must call it.
-template <class T, int BLOCK>
+// WHICH: bit 0, d0 is used; bit 1, d1 is used (an unused sum is 0 and costs
+// nothing).  EXT: the FP64 block sums use the caller's shared memory ext
+// (fin_smem<T, BLOCK, WHICH> bytes) instead of an array of their own.
+template <class T, int BLOCK, int WHICH> constexpr int fin_smem = sizeof(T) == 8 ? (WHICH == 3 ? 2 : 1) * BLOCK * 8 : 0;
+
+template <class T, int BLOCK, int WHICH = 3, bool EXT = false>
 __device__ __forceinline__ void grid_dots_finish(T d0, T d1, T *dots, int fin, void *fst, T *partials,
-                                                 unsigned *ticket)
+                                                 unsigned *ticket, T *ext = nullptr)
 {
-    __shared__ T red[BLOCK / 32];
-    const T b0 = block_sum<T, BLOCK>(d0, red);
-    const T b1 = block_sum<T, BLOCK>(d1, red);
+    static_assert(WHICH >= 1 && WHICH <= 3, "which dots");
+    constexpr int NV = WHICH == 3 ? 2 : 1;
+    auto sums = [&](T(&a)[NV]) {
+        if constexpr (EXT) block_sums_in<T, BLOCK, NV>(a, ext);
+        else block_sums<T, BLOCK, NV>(a);
+    };
+    T v[NV];
+    v[0] = WHICH == 2 ? d1 : d0;
+    if constexpr (NV == 2) v[1] = d1;
+    sums(v);
     if (threadIdx.x == 0) {
-        partials[2 * blockIdx.x] = b0;
-        partials[2 * blockIdx.x + 1] = b1;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) partials[NV * blockIdx.x + q] = v[q];
     }
     if (!last_block(ticket, gridDim.x)) return;
-    T s0 = T(0), s1 = T(0);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = T(0);
     for (unsigned b = threadIdx.x; b < gridDim.x; b += BLOCK) {
-        s0 += ldcg(partials + 2 * b);
-        s1 += ldcg(partials + 2 * b + 1);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) v[q] += ldcg(partials + NV * b + q);
     }
-    s0 = block_sum<T, BLOCK>(s0, red);
-    s1 = block_sum<T, BLOCK>(s1, red);
+    sums(v);
     if (threadIdx.x == 0) {
+        const T dd[2] = {WHICH == 2 ? T(0) : v[0], WHICH == 1 ? T(0) : v[NV - 1]};
         if (dots) {
-            dots[0] = s0;
-            dots[1] = s1;
+            dots[0] = dd[0];
+            dots[1] = dd[1];
         }
-        const T dd[2] = {s0, s1};
         run_fin<T>(fin, fst, dd);
     }
 }

@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kVB)
     T d0 = T(0);
     T av[kU], bv[kU];
     SPX_ROWS_LOOP(av[u] = a[i]; bv[u] = b[i];, d0 = fma(av[u], bv[u], d0);)
-    grid_dots_finish<T, kVB>(d0, T(0), (T *)nullptr, fin, st, partials, ticket);
+    grid_dots_finish<T, kVB, 1>(d0, T(0), (T *)nullptr, fin, st, partials, ticket);
 }
 
 // CG: x += alpha p; r -= alpha q; rho' = r.r.  PRE 1 (Jacobi): also r.z with
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kVB)
     SPX_ROWS_LOOP(xv[u] = x[i]; rv[u] = r[i]; pv[u] = p[i]; qv[u] = q[i]; if (PRE == 1) dv[u] = dinv[i];,
                   x[i] = fma(alpha, pv[u], xv[u]); const T ri = fma(-alpha, qv[u], rv[u]); r[i] = ri;
                   d0 = fma(ri, ri, d0); if (PRE == 1) d1 = fma(ri, dv[u] * ri, d1);)
-    grid_dots_finish<T, kVB>(d0, d1, (T *)nullptr, PRE == 1 ? FIN_PCG_R : PRE == 2 ? FIN_CG_RR : FIN_CG_RHO, st,
+    grid_dots_finish<T, kVB, PRE == 1 ? 3 : 1>(d0, d1, (T *)nullptr, PRE == 1 ? FIN_PCG_R : PRE == 2 ? FIN_CG_RR : FIN_CG_RHO, st,
                              partials, ticket);
 }
 
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(kVB)
     T d0 = T(0);
     T rv[kU], dv[kU];
     SPX_ROWS_LOOP(rv[u] = r[i]; dv[u] = dinv[i];, const T zi = dv[u] * rv[u]; p[i] = zi; d0 = fma(rv[u], zi, d0);)
-    grid_dots_finish<T, kVB>(d0, T(0), (T *)nullptr, FIN_PCG_RHO0, st, partials, ticket);
+    grid_dots_finish<T, kVB, 1>(d0, T(0), (T *)nullptr, FIN_PCG_RHO0, st, partials, ticket);
 }
 
 // out = dinv in (M^-1 applied to a vector)
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(kVB)
     SPX_ROWS_LOOP(rv[u] = r[i]; vv[u] = v[i]; if (PRE) dv[u] = dinv[i];,
                   const T si = fma(-alpha, vv[u], rv[u]); s[i] = si; if (PRE) sh[i] = dv[u] * si;
                   d0 = fma(si, si, d0);)
-    grid_dots_finish<T, kVB>(d0, T(0), (T *)nullptr, FIN_BI_S, st, partials, ticket);
+    grid_dots_finish<T, kVB, 1>(d0, T(0), (T *)nullptr, FIN_BI_S, st, partials, ticket);
 }
 
 // BiCGSTAB: x += alpha p + omega s; r = s - omega t  (or, converged on s:
@@ -816,7 +816,7 @@ __global__ void __launch_bounds__(kVB)
             }
         }
     }
-    if constexpr (MODE == BJ_DOT) grid_dots_finish<T, kVB>(d0, T(0), (T *)nullptr, fin, st, partials, ticket);
+    if constexpr (MODE == BJ_DOT) grid_dots_finish<T, kVB, 1>(d0, T(0), (T *)nullptr, fin, st, partials, ticket);
 }
 
 // ------------------------------------------------------------------ GMRES kernels
@@ -1020,7 +1020,6 @@ __global__ void __launch_bounds__(kVB)
     if (gs->skip) return;
     T *w = V + (int64_t)(j + 1) * ld;
     __shared__ T hs[kGmKmax];
-    __shared__ T red[kVB / 32];
     const int jn = j + 1;
     if (threadIdx.x < kGmKmax) hs[threadIdx.x] = threadIdx.x < jn ? ldcg(sm.h1 + threadIdx.x) : T(0);
     __syncthreads();
@@ -1042,12 +1041,12 @@ __global__ void __launch_bounds__(kVB)
             ww = fma(wr[u], wr[u], ww);  // zero for rows past the end
         }
     }
-    const T bsum = block_sum<T, kVB>(ww, red);
+    const T bsum = block_sum<T, kVB>(ww);
     if (threadIdx.x == 0) partials[blockIdx.x] = bsum;
     if (!last_block(ticket, gridDim.x)) return;
     T s = T(0);
     for (unsigned b = threadIdx.x; b < gridDim.x; b += kVB) s += ldcg(partials + b);
-    s = block_sum<T, kVB>(s, red);
+    s = block_sum<T, kVB>(s);
     const bool again = s < T(kGmReorthKeep2) * ldcg(wa + 1);
     if (!again && threadIdx.x < jn) sm.h2[threadIdx.x] = T(0);
     __syncthreads();
@@ -1066,7 +1065,6 @@ __global__ void __launch_bounds__(kVB)
     if (gs->skip || !gs->reorth) return;
     T *w = V + (int64_t)(j + 1) * ld;
     __shared__ T hs[kGmKmax];
-    __shared__ T red[kVB / 32];
     const int jn = j + 1;
     if (threadIdx.x < kGmKmax) hs[threadIdx.x] = threadIdx.x < jn ? ldcg(sm.h2 + threadIdx.x) : T(0);
     __syncthreads();
@@ -1081,12 +1079,12 @@ __global__ void __launch_bounds__(kVB)
         ww = fma(wr[0], wr[0], ww);
         ww = fma(wr[1], wr[1], ww);
     }
-    const T bsum = block_sum<T, kVB>(ww, red);
+    const T bsum = block_sum<T, kVB>(ww);
     if (threadIdx.x == 0) partials[blockIdx.x] = bsum;
     if (!last_block(ticket, gridDim.x)) return;
     T s = T(0);
     for (unsigned b = threadIdx.x; b < gridDim.x; b += kVB) s += ldcg(partials + b);
-    s = block_sum<T, kVB>(s, red);
+    s = block_sum<T, kVB>(s);
     if (threadIdx.x == 0) gm_finish_column<T>(gs, sm, j, s);
 }
 
@@ -1870,7 +1868,7 @@ __global__ void __launch_bounds__(kVB)
     float d0 = 0.f;
     double rv[kU];
     SPX_ROWS_LOOP(rv[u] = r64[i];, const float ri = (float)rv[u]; r32[i] = ri; d0 = fmaf(ri, ri, d0);)
-    grid_dots_finish<float, kVB>(d0, 0.f, (float *)nullptr, fin, st, partials, ticket);
+    grid_dots_finish<float, kVB, 1>(d0, 0.f, (float *)nullptr, fin, st, partials, ticket);
 }
 
 // Mixed-precision CG with reliable updates (the residual replacement of

@@ -121,11 +121,23 @@ __device__ __forceinline__ void out_row_pre(const Epi<T> &e, int64_t r, T t, con
 
 // Reduce (d0, d1) over the grid; the last block stores dots and runs the
 // scalar update.  Every block must call it.
-template <class T, int BLOCK>
+template <int MODE> constexpr int mode_dots = MODE == 4 ? 1 : MODE == 6 || MODE == 7 ? 2 : 3;  // the sums it forms
+
+template <class T, int BLOCK, int MODE = 0>
 __device__ __forceinline__ void finish_dots(T d0, T d1, const Epi<T> &e, T *partials,
                                             unsigned *ticket)
 {
-    grid_dots_finish<T, BLOCK>(d0, d1, e.dots, e.fin, e.fin_state, partials, ticket);
+    grid_dots_finish<T, BLOCK, mode_dots<MODE>>(d0, d1, e.dots, e.fin, e.fin_state, partials, ticket);
+}
+
+// The same in a kernel whose dynamic shared memory is free by then (the tile
+// stages): the sums go there, so that the largest tile that fits stays as it is.
+template <class T, int BLOCK, int MODE>
+__device__ __forceinline__ void finish_dots_in(T d0, T d1, const Epi<T> &e, T *partials, unsigned *ticket,
+                                               unsigned char *smem)
+{
+    grid_dots_finish<T, BLOCK, mode_dots<MODE>, true>(d0, d1, e.dots, e.fin, e.fin_state, partials, ticket,
+                                                      reinterpret_cast<T *>(smem));
 }
 
 // ------------------------------------------------------------------ cross-tile carries
@@ -700,7 +712,7 @@ __global__ void __launch_bounds__(ROWS * TPR)
         mbar_wait(&bar[(it + 1) & 1], (uint32_t)(((it + 1) >> 1) & 1), err, 200000000LL);
     }
     if constexpr (MODE == 0 || MODE >= 4)
-        if (e.dots) finish_dots<T, ROWS * TPR>(d0, d1, e, partials, ticket);
+        if (e.dots) finish_dots_in<T, ROWS * TPR, MODE>(d0, d1, e, partials, ticket, smem);
 }
 
 // ------------------------------------------------------------------ row-block COO (regular rows)
@@ -847,7 +859,7 @@ __global__ void __launch_bounds__(ROWS)
     }
     if (!ok && pending_prefetch) mbar_wait(&bar[(it + 1) & 1], (uint32_t)(((it + 1) >> 1) & 1), err, 200000000LL);
     if constexpr (MODE == 0 || MODE >= 4)
-        if (e.dots) finish_dots<T, ROWS>(d0, d1, e, partials, ticket);
+        if (e.dots) finish_dots_in<T, ROWS, MODE>(d0, d1, e, partials, ticket, smem);
 }
 
 // tiles[t] = first COO entry of row t * rows (entries are row-sorted), t = 0..ntiles
@@ -1059,7 +1071,7 @@ __global__ void __launch_bounds__(256)
         out_row<MODE>(e, first_row, tot, d0, d1);
     }
     if constexpr (MODE == 0 || MODE >= 4)
-        if (e.dots) finish_dots<T, 256>(d0, d1, e, partials, ticket);
+        if (e.dots) finish_dots<T, 256, MODE>(d0, d1, e, partials, ticket);
 #undef SPX_SPLIT_EMIT
 }
 
@@ -1242,7 +1254,7 @@ __global__ void __launch_bounds__(256)
         out_row<MODE>(e, first_row, tot, d0, d1);
     }
     if constexpr (MODE == 0 || MODE >= 4)
-        if (e.dots) finish_dots<T, 256>(d0, d1, e, partials, ticket);
+        if (e.dots) finish_dots<T, 256, MODE>(d0, d1, e, partials, ticket);
 }
 
 // Tiled copy of the nonzeros: source entry k (thread k) goes to its slot in
@@ -1487,7 +1499,7 @@ __global__ void __launch_bounds__(256)
         SPX_COO_OUT(first_row, tot);
     }
     if constexpr (MODE == 0 || MODE >= 4)
-        if (e.dots) finish_dots<T, 256>(d0, d1, e, partials, ticket);
+        if (e.dots) finish_dots<T, 256, MODE>(d0, d1, e, partials, ticket);
 #undef SPX_COO_OUT
 }
 
@@ -1685,7 +1697,7 @@ __global__ void __launch_bounds__(256, 4)
         out_row<MODE>(e, first_row, tot, d0, d1);
     }
     if constexpr (MODE == 0 || MODE >= 4)
-        if (e.dots) finish_dots<T, 256>(d0, d1, e, partials, ticket);
+        if (e.dots) finish_dots<T, 256, MODE>(d0, d1, e, partials, ticket);
 }
 
 // hint[g] = the row holding nonzero g*ipt: first r with rp[r+1] > g*ipt
@@ -1776,7 +1788,7 @@ __global__ void __launch_bounds__(BLOCK)
             if (i + q < n) out_row<MODE>(e, i + q, s[q], d0, d1);
     }
     if constexpr (MODE == 0 || MODE >= 4)
-        if (e.dots) finish_dots<T, BLOCK>(d0, d1, e, partials, ticket);
+        if (e.dots) finish_dots<T, BLOCK, MODE>(d0, d1, e, partials, ticket);
 }
 
 // ------------------------------------------------------------------ COO segmented reduction
@@ -2247,7 +2259,8 @@ int launch_rows_m(spx_ctx *ctx, spx_matrix *A, const T *val, const T *x, const E
     // the dynamic shared memory may reach the opt-in limit less the static part
     int dyn_max = 0;
     SPX_TRY(smem_optin(reinterpret_cast<const void *>(kern), -1, &dyn_max));
-    const int64_t smem = rows_smem<T>(A, STAGES);
+    // (the dots' block sums reuse the stages)
+    const int64_t smem = std::max<int64_t>(rows_smem<T>(A, STAGES), MODE == 1 ? 0 : fin_smem<T, block, mode_dots<MODE>>);
     if (smem > dyn_max)
         return fail(SPX_ERR_TOO_LARGE, "row-block CSR: a tile of 128 rows does not fit in shared memory");
     const int64_t ntiles = ceil_div(A->n, kRowsTile);
@@ -2330,7 +2343,8 @@ int launch_coo_rows_m(spx_ctx *ctx, spx_matrix *A, const T *cval, const T *x, co
     SPX_TRY(ensure_coo_rowtiles(ctx, A));
     int dyn_max = 0;
     SPX_TRY(smem_optin(reinterpret_cast<const void *>(kern), -1, &dyn_max));
-    const int64_t smem = coo_rows_smem<T>(A);
+    // (the dots' block sums reuse the stages)
+    const int64_t smem = std::max<int64_t>(coo_rows_smem<T>(A), MODE == 1 ? 0 : fin_smem<T, kRowsTile, mode_dots<MODE>>);
     if (smem > dyn_max)
         return fail(SPX_ERR_TOO_LARGE, "row-block COO: a tile of 128 rows does not fit in shared memory");
     const int64_t ntiles = ceil_div(A->n, kRowsTile);
