@@ -1,0 +1,6 @@
+// grid_f64.cu -- the one-launch solves over the device (grid_solve.cuh), b and x in double, products on double values.
+#include "grid_solve.cuh"
+
+namespace spx {
+template int grid_launch<double, double>(spx_ctx *, const GridArgs &, int, int, int, int);
+}

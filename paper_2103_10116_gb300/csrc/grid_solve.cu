@@ -1,0 +1,104 @@
+// grid_solve.cu -- host side of the one-launch solves over the device
+// (grid_solve.cuh): partition, workspace, launch, result.
+#include "grid_solve.cuh"
+
+#include <algorithm>
+
+namespace spx {
+
+template <class T, class V>
+int grid_launch(spx_ctx *ctx, const GridArgs &A, int solver, int blocks, int threads, int r);
+extern template int grid_launch<double, double>(spx_ctx *, const GridArgs &, int, int, int, int);
+extern template int grid_launch<float, float>(spx_ctx *, const GridArgs &, int, int, int, int);
+extern template int grid_launch<double, float>(spx_ctx *, const GridArgs &, int, int, int, int);
+
+namespace {
+
+// Rows per block from which a further block is taken.  Fewer blocks make each sum
+// cheaper (grid_solve.cuh), more blocks share the FP64 work: FP64 BiCGSTAB on 12 000
+// rows of 20 random columns 0.77 ms at 128, 0.90 at 256, 1.25 at 512; mixed CG on 8100
+// 5-point rows 1.51 / 1.40 / 1.42 ms, mixed BiCGSTAB on 30 001 random rows 0.64 / 0.63
+// / 0.72 ms.
+constexpr int kGridMinRows64 = 128;
+constexpr int kGridMinRows32 = 256;
+// Systems from which this route is faster than one cluster (CG in one precision,
+// cluster.cu) or one SM (the others, the batched kernel as a batch of one), measured
+// in ms, the other route first.  CG FP64: 8100 rows 1.90 / 2.05, 15 625 rows 1.11 /
+// 0.88; FP32: 8100 rows 0.23 / 0.27.  Mixed CG: 900 rows 0.41 / 0.52, 2025 rows 1.02 /
+// 0.74.  BiCGSTAB FP64: 256 rows 0.25 / 0.32, 512 rows 0.50 / 0.40; FP32 the same
+// at 512 rows (0.14).
+constexpr int64_t kGridCgRows64 = 12288;
+constexpr int64_t kGridCgRows32 = 16384;
+constexpr int64_t kGridCgRowsMixed = 1280;
+constexpr int64_t kGridRows = 512;
+constexpr size_t kGridWordBytes = grid_words(kGridMaxBlocks) * 8;
+
+}  // namespace
+
+// See spx_internal.cuh.
+int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, double tol, int64_t maxit,
+               int precision, spx_solve_info *info)
+{
+    if (A->format != SPX_CSR || !A->rp.p || A->n < 1 || A->nnz < 1) return SPX_ERR_UNSUPPORTED;
+    if (solver != SPX_CG && solver != SPX_BICGSTAB && solver != SPX_CGS) return SPX_ERR_UNSUPPORTED;
+    const bool mixed = precision == SPX_PREC_MIXED;
+    if (mixed ? A->dtype != SPX_F64 || !A->val32.p : (precision == SPX_PREC_F64 ? SPX_F64 : SPX_F32) != A->dtype)
+        return SPX_ERR_UNSUPPORTED;  // the general path reports the mismatch
+    // one thread per row: rows of similar length only (the row-block SpMV's rule)
+    if ((double)A->max_len > 2.0 * A->mean_len + 8.0) return SPX_ERR_UNSUPPORTED;
+    const int64_t sms = std::min<int64_t>(ctx->grid_sms, kGridMaxBlocks);
+    const int64_t from = solver != SPX_CG ? kGridRows : mixed ? kGridCgRowsMixed
+                         : precision == SPX_PREC_F64 ? kGridCgRows64 : kGridCgRows32;
+    if (A->n < from) return SPX_ERR_UNSUPPORTED;
+    const int64_t min_rows = precision == SPX_PREC_F64 ? kGridMinRows64 : kGridMinRows32;
+    const int64_t want = std::min<int64_t>(sms, ceil_div(A->n, min_rows));
+    const int64_t rows = (int64_t)round_up((size_t)ceil_div(A->n, want), 32);
+    if (rows > 4 * kGridBlockMax) return SPX_ERR_UNSUPPORTED;
+    const int r = rows <= kGridBlockMax ? 1 : rows <= 2 * kGridBlockMax ? 2 : 4;
+    const int threads = (int)round_up((size_t)ceil_div(rows, (int64_t)r), 32);
+    const int blocks = (int)ceil_div(A->n, rows);
+    const int64_t cap = std::min<int64_t>(A->max_len * rows, A->nnz);
+    const size_t smem = A->dtype == SPX_F64 && !mixed ? grid_smem<double>((int)std::min<int64_t>(cap, 1 << 20))
+                                                      : grid_smem<float>((int)std::min<int64_t>(cap, 1 << 20));
+    if (smem > (size_t)ctx->max_smem_optin - 1024) return SPX_ERR_UNSUPPORTED;
+    // workspace: slots and result | gathered vector | gathered FP64 x
+    const size_t head = kGridWordBytes + 256, vec = round_up((size_t)A->n * 8, 256);
+    if (!A->grid_work.p) SPX_TRY(dbuf_alloc(ctx, A->grid_work, head + 2 * vec));  // stream-ordered with its use
+    char *w = A->grid_work.as<char>();
+    GridArgs g;
+    g.n = (int)A->n;
+    g.rows = (int)rows;
+    g.cap = (int)cap;
+    g.rp = A->rp.as<int>();
+    g.col = A->col.as<int>();
+    g.val = mixed ? A->val32.p : A->val.p;
+    g.val64 = A->val.p;
+    g.b = b;
+    g.x = x;
+    g.ps = w + head;
+    g.xs = reinterpret_cast<double *>(w + head + vec);
+    g.words = reinterpret_cast<unsigned long long *>(w);
+    g.out = reinterpret_cast<GridOut *>(w + kGridWordBytes);
+    g.err = ctx->dev_err;
+    g.tol = tol;
+    g.maxit = (long long)maxit;
+    SPX_CUDA(cudaMemsetAsync(w, 0, grid_words(blocks) * 8, ctx->stream));
+    SPX_CUDA(cudaMemsetAsync(g.out, 0, sizeof(GridOut), ctx->stream));
+    const int st = mixed ? grid_launch<double, float>(ctx, g, solver, blocks, threads, r)
+                   : A->dtype == SPX_F64 ? grid_launch<double, double>(ctx, g, solver, blocks, threads, r)
+                                         : grid_launch<float, float>(ctx, g, solver, blocks, threads, r);
+    if (st != SPX_OK) return st;
+    GridOut h;
+    SPX_CUDA(cudaMemcpyAsync(&h, g.out, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
+    SPX_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (!h.done) return check_dev_err(ctx) != SPX_OK ? SPX_ERR_TIMEOUT : fail(SPX_ERR_CUDA, "the solve did not finish");
+    info->status = h.status;
+    info->iterations = h.iters;
+    info->restarts = h.restarts;
+    info->relres_recurrence = h.relres;
+    info->relres_true = h.relres_true;
+    if (mixed) info->inner_iterations = h.iters;
+    return SPX_OK;
+}
+
+}  // namespace spx

@@ -1225,6 +1225,18 @@ int parse_solver_code(int code, int *solver, bool *jacobi, int *bs, bool *adapti
     return SPX_OK;
 }
 
+int check_dev_err(spx_ctx *ctx)
+{
+    unsigned h = 0;
+    SPX_CUDA(cudaMemcpyAsync(&h, ctx->dev_err, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
+    SPX_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (h) {
+        cudaMemsetAsync(ctx->dev_err, 0, sizeof(unsigned), ctx->stream);
+        return fail(SPX_ERR_TIMEOUT, "a bounded device-side wait gave up (error word " + std::to_string(h) + ")");
+    }
+    return SPX_OK;
+}
+
 // ------------------------------------------------------------------ host drivers
 namespace {
 
@@ -1645,18 +1657,6 @@ template <class T> int read_dots(spx_ctx *ctx, SolverWork *w, T out[2])
 {
     SPX_CUDA(cudaMemcpyAsync(out, w->dots.p, 2 * sizeof(T), cudaMemcpyDeviceToHost, ctx->stream));
     SPX_CUDA(cudaStreamSynchronize(ctx->stream));
-    return SPX_OK;
-}
-
-int check_dev_err(spx_ctx *ctx)
-{
-    unsigned h = 0;
-    SPX_CUDA(cudaMemcpyAsync(&h, ctx->dev_err, sizeof(unsigned), cudaMemcpyDeviceToHost, ctx->stream));
-    SPX_CUDA(cudaStreamSynchronize(ctx->stream));
-    if (h) {
-        cudaMemsetAsync(ctx->dev_err, 0, sizeof(unsigned), ctx->stream);
-        return fail(SPX_ERR_TIMEOUT, "a bounded device-side wait gave up (error word " + std::to_string(h) + ")");
-    }
     return SPX_OK;
 }
 
@@ -2081,18 +2081,20 @@ int solve_typed(spx_ctx *ctx, spx_matrix *A, const T *b, T *x, int solver, doubl
     return run_short<T>(ctx, A, A->work, solver, b, x, tol, maxit, use32, false, fixed, info);
 }
 
-// ------------------------------------------------------------------ single-launch route for small systems
-// Small systems are solved by one launch that runs every iteration, where the
-// general path pays three launches and a device-wide reduction per iteration
-// (the 2D Laplacian on a 64 x 64 grid, n = 4096: 23 us per CG iteration
-// there).  CG in FP64 or FP32 on up to kSmallSolveRows rows runs on one
-// cluster of 16 (or 8) SMs (cluster.cu); BiCGSTAB, CGS and FP32-inner
-// refinement on up to kSmallBatchRows rows run in the persistent batched
-// kernel as a batch of one (one SM, whose two FP64 lanes bound it, so larger
-// systems take the general path).  CSR matrices whose SpMV kernel is left to
-// the library, no preconditioner, run to a tolerance.  The batch (the matrix's
-// own copy of the CSR arrays, from its creating context) is built on first use
-// and kept with the matrix.
+// ------------------------------------------------------------------ single-launch routes
+// Small and mid-size systems are solved by one launch that runs every iteration,
+// where the general path pays three launches and a device-wide reduction per
+// iteration (the 2D Laplacian on a 64 x 64 grid, n = 4096: 23 us per CG iteration
+// there).  CSR matrices whose SpMV kernel is left to the library, no
+// preconditioner, run to a tolerance:
+//   * from the sizes at which it measured fastest (grid_solve.cu), and up to what
+//     the SMs' shared memory and registers hold, over the whole device;
+//   * below, CG in FP64 or FP32 on one cluster of 16 (or 8) SMs (cluster.cu; up to
+//     kSmallSolveRows rows where the first route does not take the system), and
+//     BiCGSTAB, CGS and mixed precision on up to kSmallBatchRows rows in the
+//     persistent batched kernel as a batch of one (one SM, whose two FP64 lanes
+//     bound it).  The batch (the matrix's own copy of the CSR arrays, from its
+//     creating context) is built on first use and kept with the matrix.
 constexpr int64_t kSmallSolveRows = 32768;   // CG on a cluster
 constexpr int64_t kSmallBatchRows = 4096;    // the other solvers on one SM
 
@@ -2150,6 +2152,13 @@ int solve_entry(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver,
         st = cluster_solve(ctx, A, b, x, solver, tol, maxit, precision, info);
         info->time_ms = tm.ms();
         return st;
+    }
+    if (fixed == 0 && !pre && bs == 0 && A->kernel == SPX_KERNEL_AUTO) {  // a pinned SpMV kernel keeps the general path
+        st = grid_solve(ctx, A, b, x, solver, tol, maxit, precision, info);
+        if (st != SPX_ERR_UNSUPPORTED) {
+            info->time_ms = tm.ms();
+            return st;
+        }
     }
     if (fixed == 0 && !pre && bs == 0 && solver != SPX_GMRES && A->format == SPX_CSR && A->n <= kSmallSolveRows &&
         A->rp.p && A->kernel == SPX_KERNEL_AUTO) {  // a pinned SpMV kernel keeps the general path

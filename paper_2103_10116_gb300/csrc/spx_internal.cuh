@@ -145,6 +145,7 @@ struct spx_matrix {
     bool batch1_shadow = false;
     spx::DBuf small_out;  // result record of the cluster solves (cluster.cu)
     spx::DBuf cl_work;    // workspace of the one-cluster solve of a mid-size system (cluster.cu)
+    spx::DBuf grid_work;  // workspace of the one-launch solve over the device (grid_solve.cu)
     int64_t solves = 0;   // spx_solve calls made on this matrix (solvers.cu: when to capture graphs)
 };
 
@@ -211,5 +212,16 @@ int cluster_cg_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, double
 // synchronous.  SPX_ERR_UNSUPPORTED when no cluster fits the device.
 int cluster_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, double tol, int64_t maxit,
                   int precision, spx_solve_info *info);
+
+// A whole solve (CG, BiCGSTAB or CGS; F64, F32 or MIXED) of a CSR system of rows of
+// similar length in one cooperative launch over the device, the matrix in the
+// SMs' shared memory (grid_solve.cu); synchronous.  SPX_ERR_UNSUPPORTED (no error
+// message) when the system does not qualify or fit.
+int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, double tol, int64_t maxit,
+               int precision, spx_solve_info *info);
+
+// SPX_ERR_TIMEOUT (with a message; the word is cleared) when a bounded device wait has
+// given up on this context; synchronises the stream (solvers.cu).
+int check_dev_err(spx_ctx *ctx);
 
 }  // namespace spx
