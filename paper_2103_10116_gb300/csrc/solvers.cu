@@ -49,6 +49,7 @@ template <class T> struct GState {
     T bnorm;     // ||b||
     T tol;       // relative tolerance
     T beta;      // ||r|| at the start of the cycle
+    T rinv;      // 1 / rho: the cycle runs on A / rho (k_gm_dots)
     T relres;    // residual estimate |g_{j+1}| / ||b||, or the true one after a restart
     int done;    // solve finished
     int skip;    // Arnoldi kernels return at once (done or cycle stopped)
@@ -62,9 +63,10 @@ template <class T> struct GState {
     long long iters, maxit;
 };
 
-// small per-solve arrays of GMRES (device): H[(m+1) x m] row-major, cs, sn, g, y, h1, h2
+// small per-solve arrays of GMRES (device): H[(m+1) x m] row-major, cs, sn, g, y, h1, h2,
+// s (the basis vectors' scale factors)
 template <class T> struct GSmall {
-    T *H, *cs, *sn, *g, *y, *h1, *h2;
+    T *H, *cs, *sn, *g, *y, *h1, *h2, *s;
 };
 
 // ------------------------------------------------------------------ workspace
@@ -155,7 +157,7 @@ static int work_prepare(spx_ctx *ctx, SolverWork *&wk, int64_t n, int solver, in
     SPX_TRY(dbuf_alloc(ctx, wk->red, (size_t)wk->red_grid * (kGmKmax + 2) * 8));
     SPX_TRY(dbuf_alloc(ctx, wk->ticket, 64));
     SPX_CUDA(cudaMemsetAsync(wk->ticket.p, 0, 64, ctx->stream));
-    SPX_TRY(dbuf_alloc(ctx, wk->small, (size_t)((m + 1) * m + 4 * (m + 2) + 2 * (kGmKmax + 2) + 16) * 8));
+    SPX_TRY(dbuf_alloc(ctx, wk->small, (size_t)((m + 1) * m + 5 * (m + 2) + 2 * (kGmKmax + 2) + 16) * 8));
     if (!wk->host) SPX_CUDA(cudaMallocHost(&wk->host, 512));
     return SPX_OK;
 }
@@ -820,345 +822,397 @@ __global__ void __launch_bounds__(kVB)
 }
 
 // ------------------------------------------------------------------ GMRES kernels
-// Basis V[k] = base + k*ld, k = 0..m.  The Arnoldi step j forms w = A v_j in
-// V[j+1] (with ||w||^2 from the SpMV epilogue), then classical Gram-Schmidt
-// with selective reorthogonalisation: h1 = V_j^T w; w -= V_j h1; and only if
-// that pass cancelled nearly all of w (||w_new|| < ||w_old|| / 8) a second
-// pass h2 = V_j^T w; w -= V_j h2.  h = h1 + h2; H(j+1, j) = ||w||;
-// v_{j+1} = w / ||w||.  One pass leaves w_new orthogonal to V_j up to about
-// eps ||w_old|| / ||w_new||, so the threshold bounds that loss at 8 eps per
-// step.  (The classic criterion of Daniel, Gragg, Kaufman and Stewart, 1976,
+// Basis V[k] = base + k*ld, k = 0..m, stored unnormalised past V[0]: v_k = s_k V[k]
+// with s_k = 1 / ||V[k]|| kept beside the Hessenberg matrix, so that no pass over a
+// vector only scales it.  The cycle runs on A / rho, rho = ||A v_0||, so that the
+// stored vectors' norms stay near 1 however A is scaled.  The Arnoldi step j forms
+// u = A V[j] in V[j+1], then, with t_j = s_j / rho, classical Gram-Schmidt with
+// selective reorthogonalisation: h1_k = v_k . (t_j u); w = t_j u - V_j h1; and only
+// if that pass cancelled nearly all of the vector (||w|| < ||t_j u|| / 8) a second
+// pass h2 = V_j^T w; w -= V_j h2.  h = h1 + h2; H(j+1, j) = ||w||; V[j+1] = w.  One
+// pass leaves w orthogonal to V_j up to about eps ||t_j u|| / ||w||, so the
+// threshold bounds that loss at 8 eps per step; ||t_j u||^2 = ||w||^2 + ||h1||^2 to
+// the same accuracy.
+// (The classic criterion of Daniel, Gragg, Kaufman and Stewart, 1976,
 // reorthogonalises below 1/sqrt 2: on diagonally dominant matrices such as the
 // upwind convection-diffusion operator, A v_j is mostly v_j and one pass keeps
 // 26-42% of the norm, so that criterion asks for the second pass at every step,
 // doubling the FP64 work of the orthogonalisation for an orthogonality gain
 // from about 4 eps to eps.)
-constexpr double kGmReorthKeep2 = 1.0 / 64.0;  // (||w_new|| / ||w_old||)^2 below which the second pass runs
+constexpr double kGmReorthKeep2 = 1.0 / 64.0;  // (||w|| / ||t_j u||)^2 below which the second pass runs
 
-// Gram-Schmidt kernels.  Rows are processed in chunks of kGmRows (grid-stride
-// over a fixed grid).  Dots: the chunk of w sits in shared memory; warp wp
-// owns basis vectors k = wp, wp+8, wp+16, wp+24 and each lane takes four
-// rows at a time, so up to 16 independent loads per lane are in flight.
-// Block partials [k][block] are summed by the last block in block order
-// (deterministic).  Updates: a thread owns rows, two basis vectors per step.
-constexpr int kGmRows = 1024;
+// Gram-Schmidt passes.  A pass is (j+1) n FMAs: at GB300's FP64 rate 3.35 us per
+// vector of 2.1 M rows against 2.5 us for its bytes, so what counts is that every
+// SM has the same share and its FP64 pipe never waits.  A warp takes tiles of U
+// 16-byte vectors per lane (64 or 128 rows in FP64), tile t on warp t mod the
+// grid's warps, block index fastest, so that the last round's tiles spread over the
+// SMs; the grid is what is resident at once; the tiles of eight basis vectors are in
+// flight together.  The dots keep all their sums in registers and the blocks add
+// them once at the end.  The update walks the tiles backwards: the part of the
+// basis that the dots read last is still in L2.
+//   FP64, 128^3 (us, at 1 / 8 / 16 / 30 vectors): dots 14 / 42 / 73 / 132, update
+// 22 / 50 / 78 / 127, that is 3.6 to 4.0 per vector; with warps owning vectors over
+// chunks of rows and grids of 1.6 waves the passes took 101 and 98 on average over a
+// cycle.  U = 2 at three or four groups of vectors leaves room for one block per SM
+// only (146 at 30 vectors); the update with U = 2 and two blocks per SM took 133.
+constexpr int kGmB = 8;  // basis vectors in flight together
+constexpr int kGmDotsBlocks = 2, kGmUpdBlocks = 3, kGmUpdU = 1;  // blocks per SM; U of the update
+template <int KB> constexpr int gm_dots_u = KB == 1 ? 2 : 1;  // U of the dots
 
-// acc[q] += sum over the chunk's rows of V[wp + 8q][r0 + i] * ws[i]
-template <class T>
-__device__ __forceinline__ void gm_chunk_dots(const T *__restrict__ V, int64_t ld, int64_t r0, int nr, const T *ws,
-                                              int j, int lane, int wp, T acc[4])
+template <class T> struct GmVec;
+template <> struct GmVec<double> { using V = double2; };
+template <> struct GmVec<float> { using V = float4; };
+
+template <class T, int U> struct GmTile {
+    static constexpr int VEC = 16 / (int)sizeof(T), E = U * VEC;  // elements per 16 bytes; per lane
+    static constexpr int ROWS = 32 * E;
+};
+
+// this lane's E elements of the tile at p (U vectors, 32 VEC rows apart); full: the tile has all its rows
+template <class T, int U>
+__device__ __forceinline__ void gm_load(const T *__restrict__ p, int lane, bool full, int64_t left,
+                                        T (&o)[GmTile<T, U>::E])
 {
-    if constexpr (sizeof(T) == 8) {
-        // FP64: one owned vector at a time (four loads in flight), so no FP64
-        // instruction is issued for a vector the warp does not own
-        for (int i0 = lane; i0 < nr; i0 += 128) {
-            T wi[4];
+    using S = GmTile<T, U>;
+    using V = typename GmVec<T>::V;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) wi[u] = i0 + 32 * u < nr ? ws[i0 + 32 * u] : T(0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int k = wp + 8 * q;
-                if (k > j) break;  // warp-uniform
-                const T *vk = V + (int64_t)k * ld + r0;
-                T v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = i0 + 32 * u < nr ? vk[i0 + 32 * u] : T(0);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) acc[q] = fma(v[u], wi[u], acc[q]);
+    for (int h = 0; h < U; ++h) {
+        const int i = (h * 32 + lane) * S::VEC;
+        if (full) {
+            const V v = *reinterpret_cast<const V *>(p + i);
+            o[h * S::VEC] = v.x;
+            o[h * S::VEC + 1] = v.y;
+            if constexpr (S::VEC == 4) {
+                o[h * S::VEC + 2] = v.z;
+                o[h * S::VEC + 3] = v.w;
             }
+        } else {
+#pragma unroll
+            for (int e = 0; e < S::VEC; ++e) o[h * S::VEC + e] = i + e < left ? p[i + e] : T(0);
         }
-        return;
-    }
-    // FP32: every owned vector's rows are loaded before any FMA (up to 16 loads in flight)
-    const int nq = wp > j ? 0 : min(4, (j - wp) / 8 + 1);  // vectors this warp owns (warp-uniform)
-    if (nq == 0) return;
-    for (int i0 = lane; i0 < nr; i0 += 128) {
-        T wi[4], v[4][4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) wi[u] = i0 + 32 * u < nr ? ws[i0 + 32 * u] : T(0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const T *vk = V + (int64_t)(wp + 8 * q) * ld + r0;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[q][u] = q < nq && i0 + 32 * u < nr ? vk[i0 + 32 * u] : T(0);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (q < nq) {  // warp-uniform
-#pragma unroll
-                for (int u = 0; u < 4; ++u) acc[q] = fma(v[q][u], wi[u], acc[q]);
-            }
     }
 }
 
-// The last block of a dots pass: hout[k] = sum of the block partials of k.
-template <class T>
-__device__ __forceinline__ void gm_store_dots(const T acc[4], int j, int lane, int wp, T *partials, T *hout,
-                                              unsigned *ticket, bool &last)
+template <class T, int U>
+__device__ __forceinline__ void gm_store(T *__restrict__ p, int lane, bool full, int64_t left,
+                                         const T (&o)[GmTile<T, U>::E])
 {
+    using S = GmTile<T, U>;
+    using V = typename GmVec<T>::V;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int k = wp + 8 * q;
-        const T s = warp_sum(acc[q]);
-        if (lane == 0 && k <= j) partials[(int64_t)k * gridDim.x + blockIdx.x] = s;
+    for (int h = 0; h < U; ++h) {
+        const int i = (h * 32 + lane) * S::VEC;
+        if (full) {
+            V v;
+            v.x = o[h * S::VEC];
+            v.y = o[h * S::VEC + 1];
+            if constexpr (S::VEC == 4) {
+                v.z = o[h * S::VEC + 2];
+                v.w = o[h * S::VEC + 3];
+            }
+            *reinterpret_cast<V *>(p + i) = v;
+        } else {
+#pragma unroll
+            for (int e = 0; e < S::VEC; ++e)
+                if (i + e < left) p[i + e] = o[h * S::VEC + e];
+        }
     }
-    last = last_block(ticket, gridDim.x);
-    if (!last) return;
+}
+
+// calls f(q) for q < cnt (cnt <= kGmB, the same in all lanes) by a jump, not by
+// predicates: a predicated-off FP64 instruction still takes its issue slots
+template <class F> __device__ __forceinline__ void gm_first(int cnt, F f)
+{
+    switch (cnt) {
+    case 8: f(7); [[fallthrough]];
+    case 7: f(6); [[fallthrough]];
+    case 6: f(5); [[fallthrough]];
+    case 5: f(4); [[fallthrough]];
+    case 4: f(3); [[fallthrough]];
+    case 3: f(2); [[fallthrough]];
+    case 2: f(1); [[fallthrough]];
+    case 1: f(0); break;
+    default: break;
+    }
+}
+
+// A dots pass over V[0..j] and w = V[j+1], KB = ceil((j+1) / kGmB).  The first pass
+// always runs: h1_k = s_k t_j V[k].u; the second (h2_k = s_k V[k].w) only when the
+// first update asked for it.  wa (j = 0): wa[1] = ||u||^2, which sets rho.
+template <class T, int KB>
+__global__ void __launch_bounds__(kVB, kGmDotsBlocks)
+    k_gm_dots(int64_t n, int64_t ld, const T *__restrict__ V, int j, GState<T> *gs, GSmall<T> sm, const T *wa,
+              T *partials, unsigned *ticket, bool second)
+{
+    constexpr int U = gm_dots_u<KB>;
+    using S = GmTile<T, U>;
+    if (gs->skip || (second && !gs->reorth)) return;
+    const T *w = V + (int64_t)(j + 1) * ld;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int last = j + 1 - kGmB * (KB - 1);  // vectors in the last group: 1 .. kGmB
+    T acc[KB][kGmB];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int k = wp + 8 * q;
+    for (int g = 0; g < KB; ++g)
+#pragma unroll
+        for (int q = 0; q < kGmB; ++q) acc[g][q] = T(0);
+    const int64_t ntiles = (n + S::ROWS - 1) / S::ROWS, nw = (int64_t)gridDim.x * (kVB / 32);
+    for (int64_t t = (int64_t)wp * gridDim.x + blockIdx.x; t < ntiles; t += nw) {
+        const int64_t r0 = t * S::ROWS, left = n - r0;
+        const bool full = left >= S::ROWS;
+        T wv[S::E];
+        gm_load<T, U>(w + r0, lane, full, left, wv);
+#pragma unroll
+        for (int g = 0; g < KB; ++g) {
+            T v[kGmB][S::E];
+#pragma unroll
+            for (int q = 0; q < kGmB; ++q)
+                if (g < KB - 1 || q < last) gm_load<T, U>(V + (int64_t)(g * kGmB + q) * ld + r0, lane, full, left, v[q]);
+            auto add = [&](int q) {
+#pragma unroll
+                for (int e = 0; e < S::E; ++e) acc[g][q] = fma(v[q][e], wv[e], acc[g][q]);
+            };
+            if (g < KB - 1) {
+#pragma unroll
+                for (int q = 0; q < kGmB; ++q) add(q);
+            } else {
+                gm_first(last, add);
+            }
+        }
+    }
+    // block sums, eight vectors at a time: warp q adds the block's sums of vector q
+    __shared__ T buf[kGmB][kVB];
+    static_assert(kGmB == kVB / 32, "a warp per vector of a group");
+#pragma unroll
+    for (int g = 0; g < KB; ++g) {
+#pragma unroll
+        for (int q = 0; q < kGmB; ++q) buf[q][threadIdx.x] = acc[g][q];
+        __syncthreads();
+        const int k = g * kGmB + wp;
+        if (k <= j) {
+            const T s = strided_sum<T, kVB / 32>(buf[wp], lane);
+            if (lane == 0) partials[(int64_t)k * gridDim.x + blockIdx.x] = s;
+        }
+        __syncthreads();
+    }
+    if (!last_block(ticket, gridDim.x)) return;
+    T *hout = second ? sm.h2 : sm.h1;
+    T rinv;
+    if (j == 0 && !second) {
+        const T uu = ldcg(wa + 1);
+        rinv = uu > T(0) && !isinf(uu) ? T(1) / sqrt(uu) : T(1);
+        if (threadIdx.x == 0) gs->rinv = rinv;
+    } else {
+        rinv = gs->rinv;
+    }
+    const T tj = second ? T(1) : sm.s[j] * rinv;
+#pragma unroll
+    for (int g = 0; g < KB; ++g) {
+        const int k = g * kGmB + wp;
         if (k > j) continue;
         T s = T(0);
         for (unsigned b = lane; b < gridDim.x; b += 32) s += ldcg(partials + (int64_t)k * gridDim.x + b);
         s = warp_sum(s);
-        if (lane == 0) hout[k] = s;
+        if (lane == 0) hout[k] = s * tj * sm.s[k];
     }
 }
 
-// w_i -= sum_{k<=j} hs[k] V[k][i] for R rows i = i0 + stride * u (those with
-// ok[u]); two basis vectors per step, so 2R loads are in flight together.
-template <class T, int R>
-__device__ __forceinline__ void gm_rows_update(const T *__restrict__ V, int64_t ld, int64_t i0, int64_t stride,
-                                               const bool ok[R], int jn, const T *hs, T wr[R])
+// o_e += sum_{k < jn} c[k] V[k][tile rows] for the lane's E elements
+template <class T, int U>
+__device__ __forceinline__ void gm_tile_axpy(const T *__restrict__ V, int64_t ld, int64_t r0, int lane, bool full,
+                                             int64_t left, int jn, const T *c, T (&o)[GmTile<T, U>::E])
 {
-    int k = 0;
-    for (; k + 2 <= jn; k += 2) {
-        const T *v0 = V + (int64_t)k * ld + i0, *v1 = v0 + ld;
-        T a[R], c[R];
+    using S = GmTile<T, U>;
+    for (int k0 = 0; k0 < jn; k0 += kGmB) {
+        const int cnt = min(kGmB, jn - k0);
+        T v[kGmB][S::E];
 #pragma unroll
-        for (int u = 0; u < R; ++u) {
-            a[u] = ok[u] ? v0[stride * u] : T(0);
-            c[u] = ok[u] ? v1[stride * u] : T(0);
-        }
-        const T h0 = hs[k], h1 = hs[k + 1];
+        for (int q = 0; q < kGmB; ++q)
+            if (q < cnt) gm_load<T, U>(V + (int64_t)(k0 + q) * ld + r0, lane, full, left, v[q]);
+        gm_first(cnt, [&](int q) {
+            const T cq = c[k0 + q];
 #pragma unroll
-        for (int u = 0; u < R; ++u) {
-            wr[u] = fma(-h0, a[u], wr[u]);
-            wr[u] = fma(-h1, c[u], wr[u]);
-        }
+            for (int e = 0; e < S::E; ++e) o[e] = fma(cq, v[q][e], o[e]);
+        });
     }
-    if (k < jn) {
-        const T *v0 = V + (int64_t)k * ld + i0;
-        T a[R];
-#pragma unroll
-        for (int u = 0; u < R; ++u) a[u] = ok[u] ? v0[stride * u] : T(0);
-#pragma unroll
-        for (int u = 0; u < R; ++u) wr[u] = fma(-hs[k], a[u], wr[u]);
-    }
-}
-
-// A dots pass: h = V_j^T w.  The first pass always runs (h1); the second
-// (h2, second = true) only when the first update asked for it.
-template <class T>
-__global__ void __launch_bounds__(kVB)
-    k_gm_dots(int64_t n, int64_t ld, const T *__restrict__ V, int j, const GState<T> *gs, T *hout, T *partials,
-              unsigned *ticket, bool second)
-{
-    if (gs->skip || (second && !gs->reorth)) return;
-    const T *w = V + (int64_t)(j + 1) * ld;
-    __shared__ T ws[kGmRows];
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    T acc[4] = {T(0), T(0), T(0), T(0)};
-    for (int64_t r0 = (int64_t)blockIdx.x * kGmRows; r0 < n; r0 += (int64_t)gridDim.x * kGmRows) {
-        const int nr = (int)min((int64_t)kGmRows, n - r0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < nr; i += kVB) ws[i] = w[r0 + i];
-        __syncthreads();
-        gm_chunk_dots<T>(V, ld, r0, nr, ws, j, lane, wp, acc);
-    }
-    bool last;
-    gm_store_dots<T>(acc, j, lane, wp, partials, hout, ticket, last);
 }
 
 // Column j of the Hessenberg matrix from h1 + h2 and ||w|| = sqrt(ww): the
 // earlier Givens rotations, a new rotation, the residual estimate and the
-// stopping decision (one thread).
-template <class T> __device__ void gm_finish_column(GState<T> *gs, GSmall<T> sm, int j, T ww)
+// stopping decision (the first warp of the last block: its lanes load the column
+// and the rotations, one thread runs the chain).
+template <class T> __device__ void gm_finish_column(GState<T> *gs, GSmall<T> sm, int j, T ww, bool second)
 {
+    __shared__ T col[kGmKmax], cs[kGmKmax], sn[kGmKmax];
+    const int l = threadIdx.x;
+    if (l >= 32) return;
     const int m = gs->m;
+    if (l <= j) col[l] = ldcg(sm.h1 + l) + (second ? ldcg(sm.h2 + l) : T(0));
+    if (l < j) {
+        cs[l] = ldcg(sm.cs + l);
+        sn[l] = ldcg(sm.sn + l);
+    }
+    __syncwarp();
     T *H = sm.H;
-    const T hn = sqrt(ww);
-    for (int k = 0; k <= j; ++k) H[k * m + j] = ldcg(sm.h1 + k) + ldcg(sm.h2 + k);
-    H[(j + 1) * m + j] = hn;
-    for (int k = 0; k < j; ++k) {  // earlier rotations on column j
-        const T a = H[k * m + j], c = H[(k + 1) * m + j];
-        H[k * m + j] = sm.cs[k] * a + sm.sn[k] * c;
-        H[(k + 1) * m + j] = -sm.sn[k] * a + sm.cs[k] * c;
+    if (l == 0) {
+        const T hn = sqrt(ww);
+        T a = col[0];
+        for (int k = 0; k < j; ++k) {  // earlier rotations on column j
+            const T c = col[k + 1];
+            col[k] = cs[k] * a + sn[k] * c;
+            a = -sn[k] * a + cs[k] * c;
+        }
+        const T d = hypot(a, hn);
+        const T cj = d == T(0) ? T(1) : a / d, sj = d == T(0) ? T(0) : hn / d;
+        col[j] = d;
+        sm.cs[j] = cj;
+        sm.sn[j] = sj;
+        const T gj = sm.g[j];
+        sm.g[j + 1] = -sj * gj;
+        sm.g[j] = cj * gj;
+        sm.s[j + 1] = T(1) / hn;  // (not used when hn = 0: the cycle ends)
+        gs->iters += 1;
+        gs->jdone = j + 1;
+        gs->relres = fabs(sm.g[j + 1]) / gs->bnorm;
+        const bool conv = gs->relres <= gs->tol;
+        if (conv || hn == T(0) || gs->iters >= gs->maxit || j + 1 >= m) {
+            gs->cyc_stop = 1;
+            gs->est_conv = conv || hn == T(0);
+            if (conv || hn == T(0) || gs->iters >= gs->maxit) gs->skip = 1;
+        }
     }
-    const T a = H[j * m + j], c = H[(j + 1) * m + j];
-    const T d = hypot(a, c);
-    sm.cs[j] = d == T(0) ? T(1) : a / d;
-    sm.sn[j] = d == T(0) ? T(0) : c / d;
-    H[j * m + j] = d;
-    H[(j + 1) * m + j] = T(0);
-    const T gj = sm.g[j];
-    sm.g[j + 1] = -sm.sn[j] * gj;
-    sm.g[j] = sm.cs[j] * gj;
-    gs->iters += 1;
-    gs->jdone = j + 1;
-    gs->relres = fabs(sm.g[j + 1]) / gs->bnorm;
-    sm.h1[kGmKmax] = hn;  // the norm for the normalisation kernel
-    const bool conv = gs->relres <= gs->tol;
-    if (conv || hn == T(0) || gs->iters >= gs->maxit || j + 1 >= m) {
-        gs->cyc_stop = 1;
-        gs->est_conv = conv || hn == T(0);
-        if (conv || hn == T(0) || gs->iters >= gs->maxit) gs->skip = 1;
-    }
+    __syncwarp();
+    if (l <= j) H[l * m + j] = col[l];
 }
 
-// First update: w -= V_j h1 with ||w||^2 of the result accumulated on the way.
-// The last block compares it with ||A v_j||^2 (wa[1], from the SpMV): if the
-// pass kept more than 1/8 of the norm, the column is finished with h2 = 0;
-// otherwise the reorthogonalisation runs (second dots pass, second update).
-// The common case thus costs one dots pass and one update over the basis:
-// 2 (j+1) n FMAs per Arnoldi step.
+// An update pass.  First: w = t_j u - V_j h1 with ||w||^2 accumulated on the way;
+// the last block compares it with ||t_j u||^2 = ||w||^2 + ||h1||^2: if the pass kept
+// more than 1/8 of the norm the column is finished, otherwise the
+// reorthogonalisation runs (second dots pass, second update: w -= V_j h2).  The
+// common case thus costs one dots pass and one update over the basis: 2 (j+1) n
+// FMAs per Arnoldi step.  Jacobi, right: also z = dinv w, the next SpMV's input.
 template <class T>
-__global__ void __launch_bounds__(kVB)
-    k_gm_upd1(int64_t n, int64_t ld, T *__restrict__ V, int j, GState<T> *gs, GSmall<T> sm, const T *wa,
-              T *partials, unsigned *ticket)
+__global__ void __launch_bounds__(kVB, kGmUpdBlocks)
+    k_gm_upd(int64_t n, int64_t ld, T *__restrict__ V, int j, GState<T> *gs, GSmall<T> sm, const T *__restrict__ dinv,
+             T *__restrict__ z, T *partials, unsigned *ticket, bool second)
 {
-    if (gs->skip) return;
+    constexpr int U = kGmUpdU;
+    using S = GmTile<T, U>;
+    if (gs->skip || (second && !gs->reorth)) return;
     T *w = V + (int64_t)(j + 1) * ld;
-    __shared__ T hs[kGmKmax];
-    const int jn = j + 1;
-    if (threadIdx.x < kGmKmax) hs[threadIdx.x] = threadIdx.x < jn ? ldcg(sm.h1 + threadIdx.x) : T(0);
+    __shared__ T c[kGmKmax];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, jn = j + 1;
+    if (threadIdx.x < kGmKmax)
+        c[threadIdx.x] = (int)threadIdx.x < jn
+                             ? -ldcg((second ? sm.h2 : sm.h1) + threadIdx.x) * ldcg(sm.s + threadIdx.x)
+                             : T(0);
     __syncthreads();
-    constexpr int R = 4;
+    const T tj = second ? T(1) : ldcg(sm.s + j) * gs->rinv;
     T ww = T(0);
-    const int64_t stride = (int64_t)gridDim.x * kVB;
-    for (int64_t i = blockIdx.x * (int64_t)kVB + threadIdx.x; i < n; i += R * stride) {
-        bool ok[R];
-        T wr[R];
+    const int64_t ntiles = (n + S::ROWS - 1) / S::ROWS, nw = (int64_t)gridDim.x * (kVB / 32);
+    for (int64_t t = (int64_t)wp * gridDim.x + blockIdx.x; t < ntiles; t += nw) {
+        const int64_t r0 = (ntiles - 1 - t) * S::ROWS, left = n - r0;
+        const bool full = left >= S::ROWS;
+        T o[S::E];
+        gm_load<T, U>(w + r0, lane, full, left, o);
+        if (!second) {
 #pragma unroll
-        for (int u = 0; u < R; ++u) {
-            ok[u] = i + u * stride < n;
-            wr[u] = ok[u] ? w[i + u * stride] : T(0);
+            for (int e = 0; e < S::E; ++e) o[e] *= tj;
         }
-        gm_rows_update<T, R>(V, ld, i, stride, ok, jn, hs, wr);
+        gm_tile_axpy<T, U>(V, ld, r0, lane, full, left, jn, c, o);
 #pragma unroll
-        for (int u = 0; u < R; ++u) {
-            if (ok[u]) w[i + u * stride] = wr[u];
-            ww = fma(wr[u], wr[u], ww);  // zero for rows past the end
+        for (int e = 0; e < S::E; ++e) ww = fma(o[e], o[e], ww);  // zero for rows past the end
+        gm_store<T, U>(w + r0, lane, full, left, o);
+        if (dinv) {
+            T d[S::E];
+            gm_load<T, U>(dinv + r0, lane, full, left, d);
+#pragma unroll
+            for (int e = 0; e < S::E; ++e) d[e] *= o[e];
+            gm_store<T, U>(z + r0, lane, full, left, d);
         }
     }
     const T bsum = block_sum<T, kVB>(ww);
     if (threadIdx.x == 0) partials[blockIdx.x] = bsum;
     if (!last_block(ticket, gridDim.x)) return;
-    T s = T(0);
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += kVB) s += ldcg(partials + b);
-    s = block_sum<T, kVB>(s);
-    const bool again = s < T(kGmReorthKeep2) * ldcg(wa + 1);
-    if (!again && threadIdx.x < jn) sm.h2[threadIdx.x] = T(0);
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    gs->reorth = again ? 1 : 0;
-    if (!again) gm_finish_column<T>(gs, sm, j, s);
-}
-
-// Second update (only when asked for): w -= V_j h2, ||w||^2; the last block
-// finishes the column.
-template <class T>
-__global__ void __launch_bounds__(kVB)
-    k_gm_upd2(int64_t n, int64_t ld, T *__restrict__ V, int j, GState<T> *gs, GSmall<T> sm, T *partials,
-              unsigned *ticket)
-{
-    if (gs->skip || !gs->reorth) return;
-    T *w = V + (int64_t)(j + 1) * ld;
-    __shared__ T hs[kGmKmax];
-    const int jn = j + 1;
-    if (threadIdx.x < kGmKmax) hs[threadIdx.x] = threadIdx.x < jn ? ldcg(sm.h2 + threadIdx.x) : T(0);
-    __syncthreads();
-    T ww = T(0);
-    const int64_t stride = (int64_t)gridDim.x * kVB;
-    for (int64_t i = blockIdx.x * (int64_t)kVB + threadIdx.x; i < n; i += 2 * stride) {
-        const bool ok[2] = {true, i + stride < n};
-        T wr[2] = {w[i], ok[1] ? w[i + stride] : T(0)};
-        gm_rows_update<T, 2>(V, ld, i, stride, ok, jn, hs, wr);
-        w[i] = wr[0];
-        if (ok[1]) w[i + stride] = wr[1];
-        ww = fma(wr[0], wr[0], ww);
-        ww = fma(wr[1], wr[1], ww);
+    T v[2] = {T(0), T(0)};  // ||w||^2, ||h1||^2
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += kVB) v[0] += ldcg(partials + b);
+    if (!second && (int)threadIdx.x < jn) {
+        const T h = ldcg(sm.h1 + threadIdx.x);
+        v[1] = h * h;
     }
-    const T bsum = block_sum<T, kVB>(ww);
-    if (threadIdx.x == 0) partials[blockIdx.x] = bsum;
-    if (!last_block(ticket, gridDim.x)) return;
-    T s = T(0);
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += kVB) s += ldcg(partials + b);
-    s = block_sum<T, kVB>(s);
-    if (threadIdx.x == 0) gm_finish_column<T>(gs, sm, j, s);
+    block_sums<T, kVB, 2>(v);
+    const bool again = !second && v[0] < T(kGmReorthKeep2) * (v[0] + v[1]);
+    if (threadIdx.x == 0) gs->reorth = again ? 1 : 0;
+    if (!again) gm_finish_column<T>(gs, sm, j, v[0], second);
 }
 
-// v_{j+1} = w / ||w||  (Jacobi, right: also z = dinv v_{j+1}, the next SpMV's input)
-template <class T>
-__global__ void __launch_bounds__(kVB) k_gm_scale(int64_t n, int64_t ld, T *__restrict__ V, int j, const GState<T> *gs,
-                                                  GSmall<T> sm, const T *__restrict__ dinv, T *__restrict__ z)
-{
-    // v_{j+1} is needed only while the cycle goes on
-    if (gs->skip || gs->cyc_stop || gs->jdone != j + 1) return;
-    const T inv = T(1) / ldcg(sm.h1 + kGmKmax);
-    T *w = V + (int64_t)(j + 1) * ld;
-    if (dinv) {
-        for (int64_t i = blockIdx.x * (int64_t)kVB + threadIdx.x; i < n; i += (int64_t)gridDim.x * kVB) {
-            const T vi = w[i] * inv;
-            w[i] = vi;
-            z[i] = dinv[i] * vi;
-        }
-    } else {
-        for (int64_t i = blockIdx.x * (int64_t)kVB + threadIdx.x; i < n; i += (int64_t)gridDim.x * kVB) w[i] *= inv;
-    }
-}
-
-// End of a cycle: y = H^{-1} g by back substitution (one thread; m <= 32)
+// End of a cycle: y = H^{-1} g by back substitution, then scaled by s / rho (H is that of
+// A / rho, and x += sum y_k v_k = sum (y_k s_k) V[k]); one warp, column by column from shared memory (m <= 31)
 template <class T> __global__ void k_gm_solve(GState<T> *gs, GSmall<T> sm)
 {
-    if (gs->done || threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int jn = gs->jdone, m = gs->m;
+    __shared__ T Hs[kGmKmax * kGmKmax], ys[kGmKmax];
+    if (gs->done) return;
+    const int jn = gs->jdone, m = gs->m, l = threadIdx.x;
+    for (int e = l; e < jn * jn; e += 32) Hs[e] = sm.H[(e / jn) * m + e % jn];
+    T g = l < jn ? sm.g[l] : T(0);
+    __syncwarp();
     for (int i = jn - 1; i >= 0; --i) {
-        T s = sm.g[i];
-        for (int k = i + 1; k < jn; ++k) s -= sm.H[i * m + k] * sm.y[k];
-        sm.y[i] = s / sm.H[i * m + i];
+        if (l == i) ys[i] = g / Hs[i * jn + i];
+        __syncwarp();
+        if (l < i) g -= Hs[l * jn + i] * ys[i];
     }
+    __syncwarp();
+    if (l < jn) sm.y[l] = ys[l] * gs->rinv * sm.s[l];
 }
 
-// x += sum_k y_k v_k  (Jacobi, right: x += dinv sum_k y_k v_k; uout != null
-// (block-Jacobi): u = sum_k y_k v_k goes to uout and x is left to the block
-// apply, which adds M^-1 u)
+// x += sum_k y_k V[k], y scaled (Jacobi, right: x += dinv sum; uout != null
+// (block-Jacobi): the sum goes to uout and x is left to the block apply, which
+// adds M^-1 u)
 template <class T>
-__global__ void __launch_bounds__(kVB)
+__global__ void __launch_bounds__(kVB, kGmUpdBlocks)
     k_gm_update(int64_t n, int64_t ld, const T *__restrict__ V, T *__restrict__ x, const GState<T> *gs, GSmall<T> sm,
                 const T *__restrict__ dinv, T *__restrict__ uout)
 {
+    constexpr int U = kGmUpdU;
+    using S = GmTile<T, U>;
     if (gs->done) return;
     const int jn = gs->jdone;
-    if (jn == 0) {
-        if (uout)
-            for (int64_t i = blockIdx.x * (int64_t)kVB + threadIdx.x; i < n; i += (int64_t)gridDim.x * kVB)
-                uout[i] = T(0);
-        return;
-    }
-    __shared__ T ys[kGmKmax];
-    if (threadIdx.x < kGmKmax) ys[threadIdx.x] = threadIdx.x < jn ? ldcg(sm.y + threadIdx.x) : T(0);
+    if (jn == 0 && !uout) return;
+    __shared__ T c[kGmKmax];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    if (threadIdx.x < kGmKmax) c[threadIdx.x] = (int)threadIdx.x < jn ? ldcg(sm.y + threadIdx.x) : T(0);
     __syncthreads();
-    for (int64_t i = blockIdx.x * (int64_t)kVB + threadIdx.x; i < n; i += (int64_t)gridDim.x * kVB) {
-        if (dinv || uout) {
-            T ui = T(0);
+    // (x comes from the caller: 16-byte loads only where it is so aligned)
+    const bool vx = ((uintptr_t)x & 15u) == 0;
+    const int64_t ntiles = (n + S::ROWS - 1) / S::ROWS, nw = (int64_t)gridDim.x * (kVB / 32);
+    for (int64_t t = (int64_t)wp * gridDim.x + blockIdx.x; t < ntiles; t += nw) {
+        const int64_t r0 = t * S::ROWS, left = n - r0;
+        const bool full = left >= S::ROWS;
+        T o[S::E], xo[S::E];
 #pragma unroll
-            for (int k = 0; k < kGmKmax; ++k)
-                if (k < jn) ui = fma(ys[k], V[(int64_t)k * ld + i], ui);
-            if (uout) uout[i] = ui;
-            else x[i] = fma(dinv[i], ui, x[i]);
-        } else {
-            T xi = x[i];
+        for (int e = 0; e < S::E; ++e) o[e] = T(0);
+        if (!uout) gm_load<T, U>(x + r0, lane, full && vx, left, xo);
+        if (!uout && !dinv) {
 #pragma unroll
-            for (int k = 0; k < kGmKmax; ++k)
-                if (k < jn) xi = fma(ys[k], V[(int64_t)k * ld + i], xi);
-            x[i] = xi;
+            for (int e = 0; e < S::E; ++e) o[e] = xo[e];
         }
+        gm_tile_axpy<T, U>(V, ld, r0, lane, full, left, jn, c, o);
+        if (uout) {
+            gm_store<T, U>(uout + r0, lane, full, left, o);
+            continue;
+        }
+        if (dinv) {
+            T d[S::E];
+            gm_load<T, U>(dinv + r0, lane, full, left, d);
+#pragma unroll
+            for (int e = 0; e < S::E; ++e) o[e] = fma(d[e], o[e], xo[e]);
+        }
+        gm_store<T, U>(x + r0, lane, full && vx, left, o);
     }
 }
 
 // Start of a cycle: V[0] holds r = b - A x and dots[1] = r.r (SpMV epilogue).
-// Decide convergence on the TRUE residual, else v_0 = r / ||r||, g = ||r|| e_1.
+// Decide convergence on the TRUE residual, else v_0 = r / ||r||, g = ||r|| e_1
+// (Jacobi, right: also z = dinv v_0).
 template <class T>
 __global__ void __launch_bounds__(kVB) k_gm_start(int64_t n, T *__restrict__ v0, const T *dots, GState<T> *gs, GSmall<T> sm,
                                                   const T *__restrict__ dinv, T *__restrict__ z)
@@ -1193,6 +1247,7 @@ __global__ void __launch_bounds__(kVB) k_gm_start(int64_t n, T *__restrict__ v0,
         gs->est_conv = 0;
         gs->jdone = 0;
         gs->skip = 0;
+        sm.s[0] = T(1);
         sm.g[0] = beta;
         for (int k = 1; k <= gs->m; ++k) sm.g[k] = T(0);
     }
@@ -1751,6 +1806,7 @@ int run_gmres(spx_ctx *ctx, spx_matrix *A, SolverWork *w, const T *b, T *x, doub
     sm.y = sm.g + m + 2;
     sm.h1 = sm.y + m + 1;
     sm.h2 = sm.h1 + kGmKmax + 2;
+    sm.s = sm.h2 + kGmKmax + 2;
     T *dots = w->dots.as<T>();
     T *part = w->red.as<T>();
     unsigned *tk = w->ticket.as<unsigned>();
@@ -1779,10 +1835,21 @@ int run_gmres(spx_ctx *ctx, spx_matrix *A, SolverWork *w, const T *b, T *x, doub
     hs.status = SPX_MAX_ITER;
     SPX_CUDA(cudaMemcpyAsync(gs, &hs, sizeof(hs), cudaMemcpyHostToDevice, ctx->stream));
     const int g = vgrid(ctx, n, 2);
-    int gd = (int)ceil_div(n, kGmRows);  // dots passes: persistent grid, at most 4 blocks per SM
-    if (gd > 4 * ctx->grid_sms) gd = 4 * ctx->grid_sms;
-    if (gd < 1) gd = 1;
-    const int gu = vgrid(ctx, n, 8);
+    auto gm_grid = [&](int per_sm, int u) {
+        const int64_t need = ceil_div(ceil_div(n, (int64_t)u * GmTile<T, 1>::ROWS), kVB / 32);
+        return (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)per_sm * ctx->grid_sms));
+    };
+    auto dots_pass = [&](int j, bool second) {
+#define SPX_GM_DOTS(KB_) \
+    k_gm_dots<T, KB_><<<gm_grid(kGmDotsBlocks, gm_dots_u<KB_>), kVB, 0, ctx->stream>>>(n, ld, V, j, gs, sm, dots, part, tk, second)
+        switch (j / kGmB) {
+        case 0: SPX_GM_DOTS(1); break;
+        case 1: SPX_GM_DOTS(2); break;
+        case 2: SPX_GM_DOTS(3); break;
+        default: SPX_GM_DOTS(4); break;
+        }
+#undef SPX_GM_DOTS
+    };
     auto cycle = [&]() -> int {
         // restart: V[0] = b - A x, r.r
         Epi<T> e;
@@ -1799,20 +1866,22 @@ int run_gmres(spx_ctx *ctx, spx_matrix *A, SolverWork *w, const T *b, T *x, doub
         for (int j = 0; j < m; ++j) {
             Epi<T> ea = epi_plain(V + (int64_t)(j + 1) * ld);
             ea.skip = &gs->skip;
-            ea.want_yy = true;  // ||A v_j||^2 -> dots[1], for the reorthogonalisation test
-            ea.dots = dots;
-            SPX_TRY(spmv_launch<T>(ctx, A, Z ? Z : V + (int64_t)j * ld, ea, use32));  // A v_j or A M^-1 v_j
-            k_gm_dots<T><<<gd, kVB, 0, ctx->stream>>>(n, ld, V, j, gs, sm.h1, part, tk, false);
-            k_gm_upd1<T><<<gu, kVB, 0, ctx->stream>>>(n, ld, V, j, gs, sm, dots, part, tk);
-            k_gm_dots<T><<<gd, kVB, 0, ctx->stream>>>(n, ld, V, j, gs, sm.h2, part, tk, true);
-            k_gm_upd2<T><<<gu, kVB, 0, ctx->stream>>>(n, ld, V, j, gs, sm, part, tk);
-            k_gm_scale<T><<<g, kVB, 0, ctx->stream>>>(n, ld, V, j, gs, sm, dinv, Z);
+            if (j == 0) {  // ||A v_0||^2 -> dots[1]: the scale of the cycle
+                ea.want_yy = true;
+                ea.dots = dots;
+            }
+            SPX_TRY(spmv_launch<T>(ctx, A, Z ? Z : V + (int64_t)j * ld, ea, use32));  // A V[j] or A M^-1 V[j]
+            for (int pass = 0; pass < 2; ++pass) {
+                dots_pass(j, pass == 1);
+                k_gm_upd<T><<<gm_grid(kGmUpdBlocks, kGmUpdU), kVB, 0, ctx->stream>>>(n, ld, V, j, gs, sm, dinv, Z, part,
+                                                                                    tk, pass == 1);
+            }
             // (when this step ended the cycle, the apply's Z is never read: the next
             // cycle's start recomputes it)
             if (bj) SPX_TRY(bj_apply<T>(ctx, w, n, V + (int64_t)(j + 1) * ld, Z, BJ_PLAIN, &gs->skip));
         }
         k_gm_solve<T><<<1, 32, 0, ctx->stream>>>(gs, sm);
-        k_gm_update<T><<<g, kVB, 0, ctx->stream>>>(n, ld, V, x, gs, sm, dinv, bj ? Z : nullptr);
+        k_gm_update<T><<<gm_grid(kGmUpdBlocks, kGmUpdU), kVB, 0, ctx->stream>>>(n, ld, V, x, gs, sm, dinv, bj ? Z : nullptr);
         if (bj) SPX_TRY(bj_apply<T>(ctx, w, n, Z, (T *)nullptr, BJ_ADDX, &gs->done, x));
         SPX_CUDA(cudaGetLastError());
         return SPX_OK;

@@ -1,0 +1,121 @@
+"""GMRES's Gram-Schmidt passes where they can go wrong: every number of basis
+vector groups (1, 8, 9, 16, 17, 24, 25 and 31 vectors), systems of less than a
+tile, whole tiles and ragged last tiles, a solution vector that is not 16-byte
+aligned, a matrix whose first pass cancels nearly all of the new vector (the
+second pass runs), and matrices scaled far from 1.
+
+The reference is the definition: after k steps of one cycle x minimises
+||b - A x|| over the Krylov space span(b, A b, ..., A^(k-1) b), computed here in
+numpy with a twice-orthogonalised basis and a dense least-squares solve."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2103_10116_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def spx():
+    from paper_2103_10116_gb300 import spx as s
+    s.load()
+    return s
+
+
+@pytest.fixture(scope="module")
+def ctx(spx):
+    c = spx.spx_ctx_create(0)
+    yield c
+    torch.cuda.synchronize()
+    spx.spx_ctx_destroy(c)
+
+
+def _t(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+
+
+def _optimum(mat, b, k):
+    """min ||b - A x|| over the k-dimensional Krylov space of b, relative to ||b||."""
+    V = [b / np.linalg.norm(b)]
+    AV = []
+    for _ in range(k):
+        w = oracle.spmv_csr(*mat, V[-1])
+        AV.append(w.copy())
+        Q = np.array(V)
+        for _ in range(2):
+            w = w - Q.T @ (Q @ w)
+        if np.linalg.norm(w) <= 1e-13 * np.linalg.norm(AV[-1]):
+            break  # the space is invariant
+        V.append(w / np.linalg.norm(w))
+    M = np.array(AV).T
+    y = np.linalg.lstsq(M, b, rcond=None)[0]
+    return np.linalg.norm(b - M @ y) / np.linalg.norm(b)
+
+
+def _relres(spx, ctx, mat, b, k, dt, offset=0):
+    rp, col, val = mat
+    A = spx.spx_matrix_create(ctx, "csr", _t(rp), _t(col), _t(val).to(dt))
+    n = b.shape[0]
+    x = torch.zeros(n + offset, dtype=dt, device=DEV)[offset:]
+    bt = _t(b).to(dt)
+    info = spx.spx_solve_fixed(ctx, A, bt, x, "gmres", k, restart=k, precision="f64" if dt == torch.float64 else "f32")
+    spx.spx_matrix_destroy(A)
+    assert info.iterations <= k
+    return np.linalg.norm(b - oracle.spmv_csr(rp, col, val, x.double().cpu().numpy())) / np.linalg.norm(b)
+
+
+def _problem(n):
+    """n x n leading block of an upwind convection-diffusion matrix (nonsymmetric)."""
+    rp, col, val = synth.convdiff3d_upwind(int(np.ceil(n ** (1 / 3))) + 1)
+    keep_rows = np.repeat(np.arange(rp.shape[0] - 1), np.diff(rp))
+    keep = (keep_rows < n) & (col < n)
+    rows, col, val = keep_rows[keep], col[keep], val[keep]
+    out = np.zeros(n + 1, np.int32)
+    out[1:] = np.cumsum(np.bincount(rows, minlength=n))
+    return out, col.astype(np.int32), val
+
+
+# FP64 tiles of 64 and 128 rows, FP32 of 128 and 256: below one, exactly whole tiles, ragged
+@pytest.mark.parametrize("k", [1, 8, 9, 16, 17, 24, 25, 31])
+@pytest.mark.parametrize("n", [50, 1024, 20011])
+@pytest.mark.parametrize("dt", [torch.float64, torch.float32])
+def test_residual_is_the_minimum(spx, ctx, n, k, dt):
+    mat = _problem(n)
+    b = synth.uniform_vector(n, seed=n + k)
+    best = _optimum(mat, b, k)
+    got = _relres(spx, ctx, mat, b, k, dt)
+    # (FP32 also rounds A, b and x: k + 8 roundings of ||A|| ||x||, ||A|| <= 14 and ||x|| a few ||b||)
+    eps = 2.0 ** -53 if dt == torch.float64 else 2.0 ** -24
+    assert got <= best * (1 + 1e3 * eps * k) + 200 * (k + 8) * eps, (got, best)
+    if dt == torch.float64 and k in (9, 31):  # x at an odd 8-byte address
+        off = _relres(spx, ctx, mat, b, k, dt, offset=1)
+        assert abs(off - got) <= 1e-12
+
+
+@pytest.mark.parametrize("dt", [torch.float64, torch.float32])
+def test_second_pass(spx, ctx, dt):
+    """A = I + E with ||E|| small: A v_j is v_j up to a fraction of 1e-3, so one pass leaves less than 1/8."""
+    n, k = 5000, 12
+    rp, col, val = synth.laplace2d_5pt(50, 100)
+    rows = np.repeat(np.arange(n), np.diff(rp))
+    val = np.where(col == rows, 1.0 + 1e-3 * (rows % 7), 1e-3 * val)
+    mat = (rp, col, val)
+    b = synth.uniform_vector(n, seed=1)
+    best = _optimum(mat, b, k)
+    got = _relres(spx, ctx, mat, b, k, dt)
+    eps = 2.0 ** -53 if dt == torch.float64 else 2.0 ** -24
+    assert got <= 1.01 * best + 100 * (k + 8) * eps, (got, best)
+
+
+@pytest.mark.parametrize("scale", [1e-13, 1e13])
+def test_scaled_fp32(spx, ctx, scale):
+    """Products of entries of the unnormalised basis stay in FP32's range however A is scaled."""
+    n, k = 4097, 17
+    rp, col, val = _problem(n)
+    b = synth.uniform_vector(n, seed=9)
+    a = _relres(spx, ctx, (rp, col, val), b, k, torch.float32)
+    c = _relres(spx, ctx, (rp, col, val * scale), b, k, torch.float32)
+    assert abs(a - c) <= 200 * (k + 8) * 2.0 ** -24, (a, c)
