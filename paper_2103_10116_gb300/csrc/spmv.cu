@@ -580,6 +580,7 @@ __global__ void __launch_bounds__(ROWS * TPR)
     }
     __syncthreads();
 
+    const uint64_t once = policy_evict_first();
     // thread 0 only: copy the tile with rows [r0, r1) and nonzeros [j0, j1) into `stage`
     auto issue = [&](int r0, int r1, int j0, int j1, int stage) {
         unsigned char *base = smem + stage * stage_bytes;
@@ -596,8 +597,8 @@ __global__ void __launch_bounds__(ROWS * TPR)
         mbar_arrive_expect_tx(&bar[stage], (uint32_t)(rbytes + cbytes + vbytes));
         bulk_g2s(base, rp + ra, (uint32_t)rbytes, &bar[stage]);
         if (cbytes) {
-            bulk_g2s(base + S::RP_BYTES, col + ca, (uint32_t)cbytes, &bar[stage]);
-            bulk_g2s(base + S::RP_BYTES + S::col_bytes(cap), val + va, (uint32_t)vbytes, &bar[stage]);
+            bulk_g2s_once(base + S::RP_BYTES, col + ca, (uint32_t)cbytes, &bar[stage], once);
+            bulk_g2s_once(base + S::RP_BYTES + S::col_bytes(cap), val + va, (uint32_t)vbytes, &bar[stage], once);
         }
     };
 
