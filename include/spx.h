@@ -292,7 +292,8 @@ int spx_spmv_host(spx_ctx *ctx, const spx_matrix *A, const void *x_host, void *y
  *     device address (cudaGetSymbolAddress) and opts the kernel in to its
  *     shared memory; make that first call before any stream capture.
  *   - Every call shares the one array, which keeps the previous call's
- *     contents; each call clears what must start at zero.  Calls whose kernels
+ *     contents; calls on one stream leave it ready for the next, and a call on
+ *     another stream or under capture clears what it needs.  Calls whose kernels
  *     overlap on the GPU (different streams with no ordering between them)
  *     race on the array and give wrong results; order them on one stream.
  *   - The return code reports argument and launch errors only; the work runs

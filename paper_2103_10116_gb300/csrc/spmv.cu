@@ -2980,16 +2980,20 @@ constexpr size_t kNoAllocBytes = 1u << 20;  // 1 MiB
 
 // scratch layout: tiles int2[max+1] | carry_val 8B[max] | carry_row int[max] | flags int[max] |
 // arrivals, call number; the error word of the bounded waits in the last 64 bytes.  All zero at
-// load, and kept so that no call clears anything: flags hold call numbers, the last block of a
-// call leaves arrivals and error word at zero.
+// load.  Calls that follow one another on a stream clear nothing: flags hold call numbers, and
+// the last block of a call leaves arrivals and error word at zero.  A call on another stream
+// than the last one, and a captured one, clear what they need at zero first, so that calls
+// that overlapped by mistake spoil no later one.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 static_assert((kNoAllocMaxTiles + 1) * 8 + kNoAllocMaxTiles * (8 + 4 + 4) + 256 <= (int64_t)kNoAllocBytes,
               "no-alloc scratch too small for its tile limit");
 
 std::mutex g_noalloc_mu;
 void *g_noalloc_ptr[256];  // device address of the scratch per device, set once
+cudaStream_t g_noalloc_last[256];  // the stream of the device's last call
 
-int noalloc_scratch(int dev, void **out)
+// *clear: the call follows work of another stream, or is captured
+int noalloc_scratch(int dev, cudaStream_t st, void **out, bool *clear)
 {
     if (dev < 0 || dev >= 256) return fail(SPX_ERR_INVALID, "device ordinal out of range");
     std::lock_guard<std::mutex> lk(g_noalloc_mu);
@@ -2999,8 +3003,13 @@ int noalloc_scratch(int dev, void **out)
         cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(no-alloc scratch)");
         g_noalloc_ptr[dev] = p;
+        g_noalloc_last[dev] = st;  // the array is zero: the first call clears nothing
     }
     *out = g_noalloc_ptr[dev];
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+    *clear = cap != cudaStreamCaptureStatusNone || g_noalloc_last[dev] != st;
+    if (cap == cudaStreamCaptureStatusNone) g_noalloc_last[dev] = st;
     return SPX_OK;
 }
 
@@ -3015,7 +3024,7 @@ template <class K> int64_t noalloc_capacity(K kernel, int smem, int sm_count)
 
 template <class T>
 int spmv_noalloc(cudaStream_t st, void *scratch, int64_t n, int64_t nnz, const int *rp, const int *col, const T *val,
-                 const T *x, T *y, int sm_count, unsigned *err)
+                 const T *x, T *y, int sm_count, unsigned *err, bool clear)
 {
     char *base = static_cast<char *>(scratch);
     int2 *tiles = reinterpret_cast<int2 *>(base);
@@ -3025,25 +3034,26 @@ int spmv_noalloc(cudaStream_t st, void *scratch, int64_t n, int64_t nnz, const i
     unsigned *counters = reinterpret_cast<unsigned *>(flags + kNoAllocMaxTiles);  // arrivals, call number
     Epi<T> e;
     e.y = y;
-    // the split count is not read back (no synchronisation): always launch cooperatively
-    {
-        using S = MergeShape<T, kMergeBlock, kNoAllocIptOne>;
-        auto kern = k_csr_merge<T, kMergeBlock, kNoAllocIptOne, 2>;
-        constexpr int smem = S::SMEM;
-        const int64_t ntiles = ceil_div(n + nnz, S::TILE);
-        SPX_TRY(set_smem(kern, smem));
-        if (ntiles <= noalloc_capacity(kern, smem, sm_count))
-            return launch_k(kern, (int)ntiles, kMergeBlock, smem, st, true, (int)n, rp, col, val, x, (const int2 *)nullptr,
-                            (int)ntiles, carry_row, carry_val, flags, (T *)nullptr, counters, err, e, counters + 1,
-                            (int)nnz);
-    }
     using S = MergeShape<T, kMergeBlock, kNoAllocIpt>;
+    using S1 = MergeShape<T, kMergeBlock, kNoAllocIptOne>;
     auto kern = k_csr_merge<T, kMergeBlock, kNoAllocIpt, 1>;
-    const int64_t ntiles = ceil_div(n + nnz, S::TILE);
+    auto one = k_csr_merge<T, kMergeBlock, kNoAllocIptOne, 2>;
+    SPX_TRY(set_smem(kern, S::SMEM));  // both at the first call, which comes before any capture
+    SPX_TRY(set_smem(one, S1::SMEM));
+    const int64_t ntiles = ceil_div(n + nnz, S::TILE), ntiles1 = ceil_div(n + nnz, S1::TILE);
+    const bool map = ntiles1 > noalloc_capacity(one, S1::SMEM, sm_count);
+    if (clear) {
+        SPX_CUDA(cudaMemsetAsync(flags, 0, (size_t)(map ? ntiles : ntiles1) * 4, st));
+        SPX_CUDA(cudaMemsetAsync(counters, 0, 4, st));  // (the call number goes on: other flags hold earlier ones)
+        SPX_CUDA(cudaMemsetAsync(err, 0, sizeof(unsigned), st));
+    }
+    // the split count is not read back (no synchronisation): always launch cooperatively
+    if (!map)
+        return launch_k(one, (int)ntiles1, kMergeBlock, S1::SMEM, st, true, (int)n, rp, col, val, x, (const int2 *)nullptr,
+                        (int)ntiles1, carry_row, carry_val, flags, (T *)nullptr, counters, err, e, counters + 1, (int)nnz);
     k_merge_tiles<<<(int)ceil_div(ntiles + 1, 256), 256, 0, st>>>((int)n, (int)nnz, rp, S::TILE, S::SLACK, (int)ntiles,
                                                                  tiles, (unsigned *)nullptr);
     SPX_CUDA(cudaGetLastError());
-    SPX_TRY(set_smem(kern, S::SMEM));
     const int64_t grid = std::min<int64_t>(ntiles, noalloc_capacity(kern, S::SMEM, sm_count));
     return launch_k(kern, (int)grid, kMergeBlock, S::SMEM, st, true, (int)n, rp, col, val, x, (const int2 *)tiles,
                     (int)ntiles, carry_row, carry_val, flags, (T *)nullptr, counters, err, e, counters + 1, (int)nnz);
@@ -3073,10 +3083,11 @@ extern "C" int spx_spmv_csr_noalloc(void *stream, int dtype, int64_t nrows, int6
     int dev = 0;
     SPX_CUDA(cudaGetDevice(&dev));
     void *scratch = nullptr;
-    SPX_TRY(noalloc_scratch(dev, &scratch));
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    bool clear = false;
+    SPX_TRY(noalloc_scratch(dev, st, &scratch, &clear));
     int sms = 0;
     SPX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned *err = reinterpret_cast<unsigned *>(static_cast<char *>(scratch) + kNoAllocBytes - 64);
     if (nnz == 0) {  // y = 0
         const cudaError_t e = cudaMemsetAsync(y, 0, (size_t)nrows * (dtype == SPX_F64 ? 8 : 4), st);
@@ -3084,9 +3095,9 @@ extern "C" int spx_spmv_csr_noalloc(void *stream, int dtype, int64_t nrows, int6
     }
     if (dtype == SPX_F64)
         return spmv_noalloc<double>(st, scratch, nrows, nnz, row_ptr, col_idx, static_cast<const double *>(values),
-                                    static_cast<const double *>(x), static_cast<double *>(y), sms, err);
+                                    static_cast<const double *>(x), static_cast<double *>(y), sms, err, clear);
     return spmv_noalloc<float>(st, scratch, nrows, nnz, row_ptr, col_idx, static_cast<const float *>(values),
-                               static_cast<const float *>(x), static_cast<float *>(y), sms, err);
+                               static_cast<const float *>(x), static_cast<float *>(y), sms, err, clear);
 }
 
 // ------------------------------------------------------------------ gather probe

@@ -76,6 +76,11 @@ def test_calls_in_a_row(spx):
              ("long_rows", torch.float32), ("one_entry", torch.float64), ("long_rows", torch.float64)]
     out = [(n, dt) + _call(spx, n, dt, k) for k, (n, dt) in enumerate(order)]
     torch.cuda.synchronize()
+    side = torch.cuda.Stream()  # then on two streams in turn, each call ordered after the one before
+    for k, (n, dt) in enumerate(order):
+        with torch.cuda.stream(side if k % 2 else torch.cuda.default_stream()):
+            out.append((n, dt) + _call(spx, n, dt, k))
+            torch.cuda.current_stream().synchronize()
     for n, dt, _, y, xh in out:
         _check(n, dt, xh, y)
 
@@ -95,3 +100,6 @@ def test_captured(spx, name):
         g.replay()
         torch.cuda.synchronize()
         _check(name, torch.float64, x2, y)
+        _, y2, xh2 = _call(spx, "map_route", torch.float64, seed)  # a direct call of another size after a replay
+        torch.cuda.synchronize()
+        _check("map_route", torch.float64, xh2, y2)
