@@ -22,8 +22,10 @@
 // (23 us per iteration).
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
+#include <tuple>
 
 #include "dev_common.cuh"
 #include "krylov_rows.cuh"
@@ -203,42 +205,339 @@ __global__ void __launch_bounds__(BLOCK, 1)  // one block per SM: no register ca
     cl.sync();  // no block leaves while another may still read its shared memory
 }
 
+
+// ------------------------------------------------------------------ the same, matrix and vectors on chip
+// For systems of at most 16 * 1024 rows whose slices fit, block k also keeps its slice
+// of the matrix in shared memory, each column index already turned into the shared-memory
+// address of that entry of p in the cluster, and its slices of x, r, p, q in registers
+// (RPT rows per thread; p in shared memory as well, for the other blocks).  A sum needs no
+// cluster barrier: every block's first warp pushes its partial into a slot of every block
+// (st.async, counted by an mbarrier there) and adds the slots that arrived in its own, in
+// rank order.  Only the new p is published by a cluster barrier.
+//
+// What bounds an iteration is latency: 64 clocks for each dependent FP64 addition, 560 for
+// a division, some hundred for a remote access.  us per iteration, this kernel against
+// k_cluster_cg: 5-point 64 x 64 FP64 4.1 / 5.5, FP32 2.65 / 3.7; 90 x 90 FP64 4.9 / 6.9,
+// FP32 3.0 / 4.7; 7-point 25^3 FP64 8.2 / 10.5.  k_cluster_cg remains for slices that do not
+// fit and for more rows.
+
+// Sums over the cluster by pushed partials.  Two mbarriers and slot sets in turn: a block
+// pushes sum k + 1 only after it has every block's partial k, so no push is two ahead of a
+// block that still waits.
+template <int CL> struct PushSum {
+    uint64_t *bar;        // shared: 2
+    double *slots;        // shared: [2][CL]
+    double *out;          // shared: 2
+    double *buf;          // shared: one value per thread
+    unsigned *err;
+    int *dead;            // shared
+    unsigned count = 0;
+
+    static __device__ __forceinline__ uint32_t remote(uint32_t addr, uint32_t rank)
+    {
+        uint32_t r;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+        return r;
+    }
+    // v = the cluster's sum, e = f(v), the same bits in every thread of every block; false once a
+    // wait gave up
+    template <class T, int BLOCK, class F> __device__ __forceinline__ bool sum(T &v, T &e, F f)
+    {
+        const int tid = threadIdx.x, l = tid & 31;
+        const int set = (int)(count & 1u);
+        const uint32_t parity = (count >> 1) & 1u;
+        ++count;
+        T *bt = reinterpret_cast<T *>(buf);
+        if constexpr (sizeof(T) == 8) {
+            bt[tid] = v;
+        } else {
+            const T s = warp_sum(v);
+            if (l == 0) bt[tid >> 5] = s;
+        }
+        __syncthreads();
+        if (tid < 32) {
+            T s;
+            if constexpr (sizeof(T) == 8) s = strided_sum<T, BLOCK / 32>(bt, l);
+            else s = warp_sum(l < BLOCK / 32 ? bt[l] : T(0));
+            double *mine = slots + set * CL;
+            if (l == 0) mbar_arrive_expect_tx(&bar[set], CL * 8);
+            if (l < CL) {
+                const uint32_t dst = remote(smem_addr(mine + cg::this_cluster().block_rank()), (uint32_t)l);
+                const uint32_t rb = remote(smem_addr(&bar[set]), (uint32_t)l);
+                asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(dst),
+                             "l"(__double_as_longlong((double)s)), "r"(rb)
+                             : "memory");
+            }
+            bool ok;
+            const long long t0 = clock64();
+            do {
+                uint32_t done;
+                asm volatile(
+                    "{\n\t.reg .pred p;\n\t"
+                    "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                    "selp.u32 %0, 1, 0, p;\n\t}"
+                    : "=r"(done)
+                    : "r"(smem_addr(&bar[set])), "r"(parity)
+                    : "memory");
+                ok = done != 0u;
+            } while (!ok && clock64() - t0 < 2000000000LL);
+            if (!ok && l == 0) {
+                atomicOr(err, DEVERR_MBAR_TIMEOUT);
+                *dead = 1;
+            }
+            __syncwarp();
+            T t = l < CL ? (T)*(volatile double *)(mine + l) : T(0);
+#pragma unroll
+            for (int o = CL / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            const T q = f(t);
+            if (l == 0) {
+                out[0] = (double)t;
+                out[1] = (double)q;
+            }
+        }
+        __syncthreads();
+        v = (T)out[0];
+        e = (T)out[1];  // rewritten past the next sum's first barrier
+        return *dead == 0;
+    }
+    template <class T, int BLOCK> __device__ __forceinline__ bool sum(T &v)
+    {
+        T none;
+        return sum<T, BLOCK>(v, none, [](T s) { return s; });
+    }
+};
+
+// the entry at a cluster shared-memory address, 0 where !take
+template <class T> __device__ __forceinline__ T ld_cluster(uint32_t addr, bool take)
+{
+    T v = T(0);
+    if constexpr (sizeof(T) == 8)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p ld.shared::cluster.f64 %0, [%1];\n\t}"
+                     : "+d"(v)
+                     : "r"(addr), "r"((int)take)
+                     : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p ld.shared::cluster.f32 %0, [%1];\n\t}"
+                     : "+f"(v)
+                     : "r"(addr), "r"((int)take)
+                     : "memory");
+    return v;
+}
+
+// sum of val[k] p[k] over a row's entries, p[k] at cluster address adr[k]: index order, up to
+// eight remote loads in flight, FMAs only for the row's entries
+template <class T> __device__ __forceinline__ T push_row_dot(const uint32_t *adr, const T *val, int len)
+{
+    T s = T(0);
+    int k = 0;
+    for (; k + 8 <= len; k += 8) {
+        T g[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) g[u] = ld_cluster<T>(adr[k + u], true);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s = fma(val[k + u], g[u], s);
+    }
+    const int rem = len - k;
+    if (rem > 0) {
+        T g[7], v[7];
+#pragma unroll
+        for (int u = 0; u < 7; ++u) {
+            const bool take = u < rem;
+            g[u] = ld_cluster<T>(take ? adr[k + u] : 0u, take);
+            v[u] = take ? val[k + u] : T(0);
+        }
+        if (rem & 4) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s = fma(v[u], g[u], s);
+            v[0] = v[4]; v[1] = v[5]; v[2] = v[6];
+            g[0] = g[4]; g[1] = g[5]; g[2] = g[6];
+        }
+        if (rem & 2) {
+            s = fma(v[0], g[0], s);
+            s = fma(v[1], g[1], s);
+            v[0] = v[2];
+            g[0] = g[2];
+        }
+        if (rem & 1) s = fma(v[0], g[0], s);
+    }
+    return s;
+}
+
+template <class T, int CL, int BLOCK, int RPT>
+__global__ void __launch_bounds__(BLOCK, 1)
+    k_cluster_cg_push(int n, int lg, int cap, const int *__restrict__ rp, const int *__restrict__ col,
+                      const T *__restrict__ val, const T *__restrict__ b, T *__restrict__ x, T tol, long long maxit,
+                      ClOut *out, unsigned *err)
+{
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x;
+    const int R = 1 << lg;
+    const int r0 = min(n, rank * R), r1 = min(n, r0 + R);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *ps = reinterpret_cast<T *>(smem_raw);            // R entries of p
+    T *sv = ps + R;                                     // cap values
+    uint32_t *sa = reinterpret_cast<uint32_t *>(sv + cap);  // cap addresses
+    __shared__ uint64_t bar[2];
+    __shared__ double slots[2 * CL], buf[BLOCK], tot[2];
+    __shared__ int dead;
+    PushSum<CL> ps_sum{bar, slots, tot, buf, err, &dead};
+    if (tid == 0) {
+        mbar_init(&bar[0], 1);
+        mbar_init(&bar[1], 1);
+        fence_barrier_init();
+        dead = 0;
+    }
+    const int j0 = rp[r0], nz = rp[r1] - j0;
+    const uint32_t pbase = smem_addr(ps);
+    for (int k = tid; k < min(nz, cap); k += BLOCK) {
+        const int c = col[j0 + k];
+        sa[k] = PushSum<CL>::remote(pbase + (uint32_t)((c & (R - 1)) * (int)sizeof(T)), (uint32_t)(c >> lg));
+        sv[k] = val[j0 + k];
+    }
+    int at[RPT], len[RPT];
+    T xr[RPT], rr[RPT], pr[RPT], qr[RPT];
+    T bb = T(0);
+#pragma unroll
+    for (int u = 0; u < RPT; ++u) {
+        const int i = r0 + tid + u * BLOCK;
+        const bool live = i < r1;
+        at[u] = live ? rp[i] - j0 : 0;
+        len[u] = live && nz <= cap ? rp[i + 1] - j0 - at[u] : live ? 0 : -1;  // -1: no row
+        xr[u] = live ? x[i] : T(0);
+        const T bi = live ? b[i] : T(0);
+        bb = fma(bi, bi, bb);
+        if (live) ps[tid + u * BLOCK] = xr[u];
+    }
+    if (nz > cap && tid == 0) atomicOr(err, DEVERR_BOUNDS);  // never, for the matrix the slice was sized for
+#define SPX_EACH(u) _Pragma("unroll") for (int u = 0; u < RPT; ++u) if (len[u] >= 0)
+    cl.sync();  // mbarriers and x are in place
+    bool ok = ps_sum.template sum<T, BLOCK>(bb);
+    ClOut res{SPX_MAX_ITER, 0, 0, 0.0};
+    if (ok && bb == T(0)) {
+        SPX_EACH(u) xr[u] = T(0);
+        res.status = SPX_CONVERGED;
+    } else if (ok) {
+        const T tol2 = tol * tol * bb;
+        // r = b - A x (x in ps, published), ||r||^2
+        auto residual = [&](T &s) -> bool {
+            s = T(0);
+            SPX_EACH(u)
+            {
+                rr[u] = b[r0 + tid + u * BLOCK] - push_row_dot<T>(sa + at[u], sv + at[u], len[u]);
+                s = fma(rr[u], rr[u], s);
+            }
+            return ps_sum.template sum<T, BLOCK>(s);
+        };
+        T rho;
+        ok = residual(rho);
+        for (int restart = 0; ok; ++restart) {
+            SPX_EACH(u)
+            {
+                pr[u] = rr[u];
+                ps[tid + u * BLOCK] = pr[u];
+            }
+            cl.sync();
+            T last = rho;  // the last recurrence residual, squared
+            int status = rho <= tol2 ? SPX_CONVERGED : SPX_MAX_ITER;
+            // Per iteration: A p reads the cluster's p; the p.q sum (its partials follow those
+            // reads); x, r updates; the r.r sum; the p update; a cluster barrier.
+            while (status == SPX_MAX_ITER && res.iters < maxit) {
+                T pq = T(0), alpha, beta;
+                SPX_EACH(u)
+                {
+                    qr[u] = push_row_dot<T>(sa + at[u], sv + at[u], len[u]);
+                    pq = fma(pr[u], qr[u], pq);
+                }
+                if (!(ok = ps_sum.template sum<T, BLOCK>(pq, alpha, [=](T s) { return rho / s; }))) break;
+                if (pq == T(0)) {
+                    status = SPX_BREAKDOWN;
+                    break;
+                }
+                T s = T(0);
+                SPX_EACH(u)
+                {
+                    rr[u] = fma(-alpha, qr[u], rr[u]);
+                    s = fma(rr[u], rr[u], s);
+                    xr[u] = fma(alpha, pr[u], xr[u]);
+                }
+                if (!(ok = ps_sum.template sum<T, BLOCK>(s, beta, [=](T t) { return t / rho; }))) break;
+                ++res.iters;
+                last = s;
+                if (s <= tol2) {
+                    status = SPX_CONVERGED;
+                    break;
+                }
+                rho = s;
+                SPX_EACH(u)
+                {
+                    pr[u] = fma(beta, pr[u], rr[u]);
+                    ps[tid + u * BLOCK] = pr[u];
+                }
+                cl.sync();
+            }
+            if (!ok) break;
+            res.status = status;
+            res.relres = (double)sqrt(last / bb);
+            res.restarts = restart;
+            if (status != SPX_CONVERGED) break;
+            // the true residual ||b - A x|| / ||b||
+            cl.sync();  // every block is past its reads of ps
+            SPX_EACH(u) ps[tid + u * BLOCK] = xr[u];
+            cl.sync();
+            if (!(ok = residual(rho))) break;
+            res.relres = (double)sqrt(rho / bb);
+            if (rho <= tol2) break;
+            if (restart == 3) {
+                res.status = SPX_STAGNATED;
+                break;
+            }
+            cl.sync();
+        }
+    }
+    SPX_EACH(u) x[r0 + tid + u * BLOCK] = xr[u];
+#undef SPX_EACH
+    if (rank == 0 && tid == 0) {
+        if (!ok) res.status = -1;
+        *out = res;
+    }
+    cl.sync();  // no block leaves while another may still read its shared memory
+}
+
 }  // namespace
 
 int cluster_cg_max_rows() { return 16 * kClMaxRowsPerBlock; }
 
 namespace {
 
-// The largest cluster (16 blocks, a non-portable size, else the portable 8)
-// this device can run for the kernel's shared memory; 0 if none.
-// Asked once per (device, shared-memory size).
-template <class T, int CL, int BLOCK> int cluster_fits(int smem)
+// Clusters of CL blocks of this kernel and shared-memory size the device runs at once (0:
+// none); asked once per (kernel, device, size).
+template <class K> int cluster_count(K kern, int cl, int block, int smem)
 {
-    auto kern = k_cluster_cg<T, CL, BLOCK>;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     static std::mutex mu;
-    static std::map<std::pair<int, int>, int> known;  // (device, smem) -> clusters
+    static std::map<std::tuple<const void *, int, int>, int> known;  // (kernel, device, smem) -> clusters
     std::lock_guard<std::mutex> lk(mu);
-    auto it = known.find({dev, smem});
+    const auto key = std::make_tuple(reinterpret_cast<const void *>(kern), dev, smem);
+    auto it = known.find(key);
     if (it != known.end()) return it->second;
-    int &nc = known[{dev, smem}];
+    int &nc = known[key];
     nc = 0;
     if (smem_optin(reinterpret_cast<const void *>(kern), smem) != SPX_OK) return 0;
-    if (CL > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    if (cl > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(CL);
-    cfg.blockDim = dim3(BLOCK);
+    cfg.gridDim = dim3((unsigned)cl);
+    cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = (size_t)smem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.x = (unsigned)cl;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
@@ -248,6 +547,13 @@ template <class T, int CL, int BLOCK> int cluster_fits(int smem)
         nc = 0;
     }
     return nc;
+}
+
+// The largest cluster (16 blocks, a non-portable size, else the portable 8)
+// this device can run for the kernel's shared memory; 0 if none.
+template <class T, int CL, int BLOCK> int cluster_fits(int smem)
+{
+    return cluster_count(k_cluster_cg<T, CL, BLOCK>, CL, BLOCK, smem);
 }
 
 template <class T, int CL, int BLOCK>
@@ -273,13 +579,64 @@ int launch_cluster_cg(spx_ctx *ctx, spx_matrix *A, int lg, const T *b, T *x, dou
     return SPX_OK;
 }
 
+// Shared memory of k_cluster_cg_push
+template <class T> size_t push_smem(int lg, int64_t cap) { return (((size_t)1 << lg) + (size_t)cap) * sizeof(T) + (size_t)cap * 4; }
+
+// The kernel that keeps the matrix on chip, where the slices fit; SPX_ERR_UNSUPPORTED otherwise.
+template <class T, int RPT>
+int launch_cluster_push(spx_ctx *ctx, spx_matrix *A, int lg, int cap, const T *b, T *x, double tol, int64_t maxit, ClOut *out)
+{
+    constexpr int CL = 16, BLOCK = 256;
+    auto kern = k_cluster_cg_push<T, CL, BLOCK, RPT>;
+    const int smem = (int)push_smem<T>(lg, cap);
+    int lim = 0;
+    SPX_TRY(smem_optin(reinterpret_cast<const void *>(kern), -1, &lim));
+    if (smem > lim || cluster_count(kern, CL, BLOCK, smem) < 1) return SPX_ERR_UNSUPPORTED;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(CL);
+    cfg.blockDim = dim3(BLOCK);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    SPX_CUDA(cudaLaunchKernelEx(&cfg, kern, (int)A->n, lg, cap, (const int *)A->rp.as<int>(),
+                                (const int *)A->col.as<int>(), (const T *)A->val.as<T>(), b, x, (T)tol,
+                                (long long)maxit, out, ctx->dev_err));
+    return SPX_OK;
+}
+
+// log2 of the rows per block of a 16-block cluster, and whether k_cluster_cg_push takes A
+int push_lg(int64_t n)
+{
+    int lg = 0;
+    while ((int64_t)16 << lg < n) ++lg;
+    return lg;
+}
+template <class T> bool push_takes(const spx_ctx *ctx, const spx_matrix *A)
+{
+    const int lg = push_lg(A->n);
+    return lg <= 10 && push_smem<T>(lg, std::min<int64_t>(A->max_len << lg, A->nnz)) <= (size_t)ctx->max_smem_optin - 4096;
+}
+
 template <class T>
 int cluster_cg_typed(spx_ctx *ctx, spx_matrix *A, const T *b, T *x, double tol, int64_t maxit, ClOut *out)
 {
     // 16 blocks of 256 threads where the device runs such a cluster, else 8 of 512
-    int lg16 = 0, lg8 = 0;
-    while ((int64_t)16 << lg16 < A->n) ++lg16;
+    const int lg16 = push_lg(A->n);
+    int lg8 = 0;
     while ((int64_t)8 << lg8 < A->n) ++lg8;
+    if (push_takes<T>(ctx, A)) {
+        const int cap = (int)std::min<int64_t>(A->max_len << lg16, A->nnz);
+        const int st = lg16 <= 8   ? launch_cluster_push<T, 1>(ctx, A, lg16, cap, b, x, tol, maxit, out)
+                       : lg16 == 9 ? launch_cluster_push<T, 2>(ctx, A, lg16, cap, b, x, tol, maxit, out)
+                                   : launch_cluster_push<T, 4>(ctx, A, lg16, cap, b, x, tol, maxit, out);
+        if (st != SPX_ERR_UNSUPPORTED) return st;
+    }
     if ((1 << lg16) <= kClMaxRowsPerBlock && cluster_fits<T, 16, 256>((int)(4 * ((size_t)1 << lg16) * sizeof(T))) > 0)
         return launch_cluster_cg<T, 16, 256>(ctx, A, lg16, b, x, tol, maxit, out);
     if ((1 << lg8) <= kClMaxRowsPerBlock && cluster_fits<T, 8, 512>((int)(4 * ((size_t)1 << lg8) * sizeof(T))) > 0)
@@ -288,6 +645,12 @@ int cluster_cg_typed(spx_ctx *ctx, spx_matrix *A, const T *b, T *x, double tol, 
 }
 
 }  // namespace
+
+// Whether CG on A keeps matrix and vectors on the cluster's SMs (k_cluster_cg_push).
+bool cluster_cg_on_chip(const spx_ctx *ctx, const spx_matrix *A)
+{
+    return A->dtype == SPX_F64 ? push_takes<double>(ctx, A) : push_takes<float>(ctx, A);
+}
 
 // CG on one cluster (see the file comment); synchronous.  b, x: device, dtype
 // of A (FP64 or FP32); x holds the initial guess.  SPX_ERR_UNSUPPORTED when
@@ -308,6 +671,7 @@ int cluster_cg_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, double
     ClOut h;
     SPX_CUDA(cudaMemcpyAsync(&h, out, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
     SPX_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (h.status < 0) return check_dev_err(ctx) != SPX_OK ? SPX_ERR_TIMEOUT : fail(SPX_ERR_CUDA, "the solve did not finish");
     info->status = h.status;
     info->iterations = h.iters;
     info->restarts = h.restarts;

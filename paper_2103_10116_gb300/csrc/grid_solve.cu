@@ -23,12 +23,13 @@ constexpr int kGridMinRows64 = 128;
 constexpr int kGridMinRows32 = 256;
 // Systems from which this route is faster than one cluster (CG in one precision,
 // cluster.cu) or one SM (the others, the batched kernel as a batch of one), measured
-// in ms, the other route first.  CG FP64: 8100 rows 1.90 / 2.05, 15 625 rows 1.11 /
-// 0.88; FP32: 8100 rows 0.23 / 0.27.  Mixed CG: 900 rows 0.41 / 0.52, 2025 rows 1.02 /
-// 0.74.  BiCGSTAB FP64: 256 rows 0.25 / 0.32, 512 rows 0.50 / 0.40; FP32 the same
-// at 512 rows (0.14).
-constexpr int64_t kGridCgRows64 = 12288;
-constexpr int64_t kGridCgRows32 = 16384;
+// in ms, the other route first.  CG FP64: 8100 rows 1.36 / 2.05, 15 625 rows 0.86 / 0.88;
+// 27-point 10 648 rows, whose slices do not fit one cluster, 1.10 / 0.55; FP32: 8100 rows
+// 0.14 / 0.27.  Mixed CG: 900 rows 0.41 / 0.52, 2025 rows 1.02 / 0.74.  BiCGSTAB FP64:
+// 256 rows 0.25 / 0.32, 512 rows 0.50 / 0.40; FP32 the same at 512 rows (0.14).
+constexpr int64_t kGridCgRows64 = 14336;
+constexpr int64_t kGridCgRows32 = 16385;
+constexpr int64_t kGridCgRowsOff = 4096;  // ... where the cluster does not keep the matrix on chip
 constexpr int64_t kGridCgRowsMixed = 1280;
 constexpr int64_t kGridRows = 512;
 constexpr size_t kGridWordBytes = grid_words(kGridMaxBlocks) * 8;
@@ -47,8 +48,11 @@ int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, 
     // one thread per row: rows of similar length only (the row-block SpMV's rule)
     if ((double)A->max_len > 2.0 * A->mean_len + 8.0) return SPX_ERR_UNSUPPORTED;
     const int64_t sms = std::min<int64_t>(ctx->grid_sms, kGridMaxBlocks);
-    const int64_t from = solver != SPX_CG ? kGridRows : mixed ? kGridCgRowsMixed
-                         : precision == SPX_PREC_F64 ? kGridCgRows64 : kGridCgRows32;
+    const int64_t from = solver != SPX_CG              ? kGridRows
+                         : mixed                       ? kGridCgRowsMixed
+                         : !cluster_cg_on_chip(ctx, A) ? kGridCgRowsOff
+                         : precision == SPX_PREC_F64   ? kGridCgRows64
+                                                       : kGridCgRows32;
     if (A->n < from) return SPX_ERR_UNSUPPORTED;
     const int64_t min_rows = precision == SPX_PREC_F64 ? kGridMinRows64 : kGridMinRows32;
     const int64_t want = std::min<int64_t>(sms, ceil_div(A->n, min_rows));

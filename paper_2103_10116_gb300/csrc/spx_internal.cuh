@@ -205,6 +205,7 @@ int batch_max_rows(const spx_ctx *ctx);
 
 // CG on one thread-block cluster for small CSR systems (cluster.cu); synchronous.
 int cluster_cg_max_rows();
+bool cluster_cg_on_chip(const spx_ctx *ctx, const spx_matrix *A);
 int cluster_cg_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, double tol, int64_t maxit,
                      spx_solve_info *info);
 // A whole solve (CG, BiCGSTAB or CGS; F64, F32 or MIXED) of a CSR system in one
