@@ -960,14 +960,28 @@ __global__ void k_coo_rowtiles(int n, int64_t nnz, const int *__restrict__ crow,
     }
 }
 
-// the largest number of nonzeros in a tile of `rows` consecutive rows
-__global__ void k_tile_max_nnz(int n, const int *__restrict__ rp, int rows, int ntiles, int *out)
+// the largest number of nonzeros in a tile of `rows` consecutive rows (out[0]) and of
+// `small` rows, a divisor of `rows` (out[1])
+__global__ void k_tile_max_nnz(int n, const int *__restrict__ rp, int rows, int small, int ntiles, int *out)
 {
-    int m = 0;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += gridDim.x * blockDim.x)
-        m = max(m, rp[min(n, (t + 1) * rows)] - rp[t * rows]);
+    int m = 0, ms = 0;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += gridDim.x * blockDim.x) {
+        const int j0 = rp[t * rows];
+        int j = j0;
+        for (int r = 0; r < rows; r += small) {
+            const int je = rp[min(n, t * rows + r + small)];
+            ms = max(ms, je - j);
+            j = je;
+            if (t * rows + r + small >= n) break;
+        }
+        m = max(m, j - j0);
+    }
     m = warp_max(m);
-    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+    ms = warp_max(ms);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(out, m);
+        atomicMax(out + 1, ms);
+    }
 }
 
 // ------------------------------------------------------------------ nnz-split CSR (warp-independent)
@@ -1789,8 +1803,15 @@ __global__ void k_row_hint(int n, int nnz, const int *__restrict__ rp, int ipt, 
 
 // ------------------------------------------------------------------ ELL
 // Column-major ELL [width][ld]: thread g handles rows g*R .. g*R+R-1 and
-// reads R consecutive values (16 B for R = 16 / sizeof(T)) per slab, fully
-// coalesced across the warp.  Padding slots (col = -1) are skipped.
+// reads R consecutive values of each slab, coalesced across the warp; four
+// slabs' loads are issued together (the last ones too), then their gathers.
+// The slabs are read once (evict-first, so that x and a solver's vectors stay
+// in L2).  Padding slots (col = -1) are skipped.
+// One row per thread at full occupancy (32 registers; six blocks per SM with dots) by default: what the
+// kernel needs is loads in flight, and single rows leave less work in the last
+// round of the grid.  us, against two rows per thread with the last slabs one by
+// one: 7-point 101^3 FP64 21.6 / 26.3, 128^3 38.8 / 43.1, 27-point 100^3 63.8 /
+// 75.9; FP32 7-point 128^3 23.2 / 28.7, 27-point 100^3 40.1 / 44.1.
 template <class T, int R> struct Vec;
 template <> struct Vec<double, 1> { using V = double; using I = int; };
 template <> struct Vec<double, 2> { using V = double2; using I = int2; };
@@ -1799,7 +1820,7 @@ template <> struct Vec<float, 2> { using V = float2; using I = int2; };
 template <> struct Vec<float, 4> { using V = float4; using I = int4; };
 
 template <class T, int R, int BLOCK, int MODE>
-__global__ void __launch_bounds__(BLOCK)
+__global__ void __launch_bounds__(BLOCK, R == 1 ? (MODE == 1 ? 8 : 6) : 1)
     k_ell(int64_t n, int64_t ld, int w, const int *__restrict__ ecol, const T *__restrict__ eval,
           const T *__restrict__ x, Epi<T> e, T *partials, unsigned *ticket)
 {
@@ -1812,18 +1833,32 @@ __global__ void __launch_bounds__(BLOCK)
     for (int64_t g = blockIdx.x * (int64_t)BLOCK + threadIdx.x; g < ngroups;
          g += (int64_t)gridDim.x * BLOCK) {
         const int64_t i = g * R;
+        // the general epilogue's row operands, in flight beside the slabs (in the solvers'
+        // modes the registers are better spent on occupancy: CG on 101^3 14.3 ms, 15.0 with)
+        EpiRow<T> pre[R];
+        if constexpr (MODE == 0) {
+#pragma unroll
+            for (int q = 0; q < R; ++q) pre[q] = i + q < n ? epi_row_load<MODE>(e, i + q) : EpiRow<T>{T(0), T(0)};
+        }
         T s[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) s[q] = T(0);
-        int j = 0;
-        for (; j + U <= w; j += U) {
+        for (int j = 0; j < w; j += U) {
             VI c[U];
             VV v[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int64_t o = (int64_t)(j + u) * ld + i;
-                c[u] = __ldg(reinterpret_cast<const VI *>(ecol + o));
-                v[u] = __ldg(reinterpret_cast<const VV *>(eval + o));
+                if (j + u < w) {
+                    c[u] = __ldcs(reinterpret_cast<const VI *>(ecol + o));
+                    v[u] = __ldcs(reinterpret_cast<const VV *>(eval + o));
+                } else {
+#pragma unroll
+                    for (int q = 0; q < R; ++q) {
+                        reinterpret_cast<int *>(&c[u])[q] = -1;
+                        reinterpret_cast<T *>(&v[u])[q] = T(0);
+                    }
+                }
             }
             T xg[U][R];
 #pragma unroll
@@ -1834,6 +1869,7 @@ __global__ void __launch_bounds__(BLOCK)
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
+                if (sizeof(T) == 8 && j + u >= w) break;  // (warp-uniform)
                 const T *vv = reinterpret_cast<const T *>(&v[u]);
 #pragma unroll
                 for (int q = 0; q < R; ++q) {
@@ -1845,19 +1881,12 @@ __global__ void __launch_bounds__(BLOCK)
                 }
             }
         }
-        for (; j < w; ++j) {
-            const int64_t o = (int64_t)j * ld + i;
-            const VI c = __ldg(reinterpret_cast<const VI *>(ecol + o));
-            const VV v = __ldg(reinterpret_cast<const VV *>(eval + o));
-            const int *cc = reinterpret_cast<const int *>(&c);
-            const T *vv = reinterpret_cast<const T *>(&v);
-#pragma unroll
-            for (int q = 0; q < R; ++q)
-                if (cc[q] >= 0) s[q] = fma(vv[q], __ldg(x + cc[q]), s[q]);
-        }
 #pragma unroll
         for (int q = 0; q < R; ++q)
-            if (i + q < n) out_row<MODE>(e, i + q, s[q], d0, d1);
+            if (i + q < n) {
+                if constexpr (MODE == 0) out_row_pre<MODE>(e, i + q, s[q], pre[q], d0, d1);
+                else out_row<MODE>(e, i + q, s[q], d0, d1);
+            }
     }
     if constexpr (MODE == 0 || MODE >= 4)
         if (e.dots) finish_dots<T, BLOCK, MODE>(d0, d1, e, partials, ticket);
@@ -2294,26 +2323,37 @@ template <class T> int epi_mode(const Epi<T> &e)
 }
 
 constexpr int kRowsTile = 128;
+// Rows per tile of the row-block CSR kernel.  FP64 rows that take two threads each
+// have tiles large enough to leave two blocks of 128 rows per SM; tiles of 32 rows,
+// ten blocks per SM, let blocks wait for their copies and gathers independently
+// (27-point stencil 100^3: 67.6 us against 75.6; tiles of 64 rows 72.2).  FP32 and
+// single-thread rows measured the same or slower with smaller tiles (27-point FP32
+// 34.9 / 35.1, 7-point 128^3 FP64 34.9 / 34.8, FP32 20.7 / 24.5).
+constexpr int kRowsSmallTile = 32;
+template <class T, int TPR> constexpr int rows_tile = sizeof(T) == 8 && TPR == 2 ? kRowsSmallTile : kRowsTile;
 constexpr int kRowsStages = 2;  // default shared-memory stages per block of the row-block kernel
 
+// the most nonzeros in a tile of each size, measured once per matrix
 int ensure_rows_cap(spx_ctx *ctx, spx_matrix *A)
 {
     if (A->rows_cap >= 0) return SPX_OK;
     const int64_t ntiles = ceil_div(A->n, kRowsTile);
     DBuf m;
     SPX_TRY(dbuf_alloc(ctx, m, 16));
-    int cap = 0;
-    cudaError_t e = cudaMemsetAsync(m.p, 0, 4, ctx->stream);
+    int cap[2] = {0, 0};
+    cudaError_t e = cudaMemsetAsync(m.p, 0, 8, ctx->stream);
     if (e == cudaSuccess && ntiles > 0) {
         const int g = (int)std::min<int64_t>(ceil_div(ntiles, 256), (int64_t)ctx->grid_sms * 8);
-        k_tile_max_nnz<<<g, 256, 0, ctx->stream>>>((int)A->n, A->rp.as<int>(), kRowsTile, (int)ntiles, m.as<int>());
+        k_tile_max_nnz<<<g, 256, 0, ctx->stream>>>((int)A->n, A->rp.as<int>(), kRowsTile, kRowsSmallTile, (int)ntiles,
+                                                   m.as<int>());
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&cap, m.p, 4, cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(cap, m.p, 8, cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     dbuf_free(ctx, m);
     if (e != cudaSuccess) return cuda_fail(e, "row-block tile sizes");
-    A->rows_cap = cap;
+    A->rows_cap = cap[0];
+    A->rows_cap_small = cap[1];
     return SPX_OK;
 }
 
@@ -2326,21 +2366,25 @@ template <class T> int64_t rows_smem(const spx_matrix *A, int stages)
 template <class T, int STAGES, int MODE, int TPR>
 int launch_rows_m(spx_ctx *ctx, spx_matrix *A, const T *val, const T *x, const Epi<T> &e)
 {
-    auto kern = k_csr_rows<T, kRowsTile, STAGES, MODE, TPR>;
-    constexpr int block = kRowsTile * TPR;
+    constexpr int rows = rows_tile<T, TPR>;
+    auto kern = k_csr_rows<T, rows, STAGES, MODE, TPR>;
+    constexpr int block = rows * TPR;
     SPX_TRY(ensure_rows_cap(ctx, A));
+    const int64_t cap = rows == kRowsTile ? A->rows_cap : A->rows_cap_small;
     // the dynamic shared memory may reach the opt-in limit less the static part
     int dyn_max = 0;
     SPX_TRY(smem_optin(reinterpret_cast<const void *>(kern), -1, &dyn_max));
-    // (the dots' block sums reuse the stages)
-    const int64_t smem = std::max<int64_t>(rows_smem<T>(A, STAGES), MODE == 1 ? 0 : fin_smem<T, block, mode_dots<MODE>>);
-    if (smem > dyn_max)
+    // (a matrix whose tiles of 128 rows do not fit is refused whatever the tile in use)
+    if (rows_smem<T>(A, STAGES) > dyn_max)
         return fail(SPX_ERR_TOO_LARGE, "row-block CSR: a tile of 128 rows does not fit in shared memory");
-    const int64_t ntiles = ceil_div(A->n, kRowsTile);
+    // (the dots' block sums reuse the stages)
+    const int64_t smem = std::max<int64_t>(RowsShape<T, rows>::smem((int)cap, STAGES),
+                                           MODE == 1 ? 0 : fin_smem<T, block, mode_dots<MODE>>);
+    const int64_t ntiles = ceil_div(A->n, rows);
     const int grid = grid_for(ctx, kern, block, (int)smem, ntiles);
     SPX_TRY(ensure_scratch(ctx, A, 0, grid, sizeof(T)));
     kern<<<grid, block, (int)smem, ctx->stream>>>((int)A->n, A->rp.as<int>(), A->col.as<int>(), val, x,
-                                                      (int)ntiles, (int)A->rows_cap, A->partials.as<T>(),
+                                                      (int)ntiles, (int)cap, A->partials.as<T>(),
                                                       A->ticket.as<unsigned>(), ctx->dev_err, e);
     SPX_CUDA(cudaGetLastError());
     return SPX_OK;
@@ -2712,14 +2756,11 @@ int launch_ell_m(spx_ctx *ctx, spx_matrix *A, const T *eval, const T *x, const E
     return SPX_OK;
 }
 
-// The plain-store mode pays off in FP32 (47.8 vs 50.7 us on the 27-point stencil);
-// in FP64 it raises the kernel from 32 to 40 registers and the lost occupancy
-// costs more (76.3 vs 70.2 us) than the epilogue's FP64 instructions save.
 template <class T, int R>
 int launch_ell(spx_ctx *ctx, spx_matrix *A, const T *eval, const T *x, const Epi<T> &e)
 {
     switch (epi_mode(e)) {
-    case 1: return sizeof(T) == 4 ? launch_ell_m<T, R, 1>(ctx, A, eval, x, e) : launch_ell_m<T, R, 0>(ctx, A, eval, x, e);
+    case 1: return launch_ell_m<T, R, 1>(ctx, A, eval, x, e);
     case 4: return launch_ell_m<T, R, 4>(ctx, A, eval, x, e);
     case 5: return launch_ell_m<T, R, 5>(ctx, A, eval, x, e);
     case 6: return launch_ell_m<T, R, 6>(ctx, A, eval, x, e);
@@ -2836,7 +2877,7 @@ template <class T>
 int dispatch_ell(spx_ctx *ctx, spx_matrix *A, const T *eval, const T *x, const Epi<T> &e)
 {
     int p = A->kernel == SPX_KERNEL_ELL ? A->kparam : 0;
-    if (p <= 0) p = 2;  // two rows per thread (FP32 with four: 58.0 against 54.0 us on the 27-point stencil)
+    if (p <= 0) p = 1;  // one row per thread (see k_ell)
     if constexpr (sizeof(T) == 8) {
         if (p == 1) return launch_ell<T, 1>(ctx, A, eval, x, e);
         if (p == 2) return launch_ell<T, 2>(ctx, A, eval, x, e);

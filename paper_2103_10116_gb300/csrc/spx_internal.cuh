@@ -116,6 +116,7 @@ struct spx_matrix {
     int64_t nsplit = 0;       // boundaries that split a row (need the look-back)
     // row-block CSR: the most nonzeros in a tile of 128 rows (-1: not measured yet)
     int64_t rows_cap = -1;
+    int64_t rows_cap_small = 0;  // the same for its smaller tile (spmv.cu: rows_tile)
     // row hints of the nnz-split CSR kernel (row holding nonzero g * hint_ipt)
     spx::DBuf hint;
     int hint_ipt = 0;

@@ -121,6 +121,13 @@ def test_csr_row_block_copies_stay_in_bounds(name, V):
         assert _lane_partition_ok(lengths, tpr)
 
 
+@pytest.mark.parametrize("name", list(MATS))
+def test_csr_row_block_small_tiles_stay_in_bounds(name, monkeypatch):
+    """FP64 rows that take two threads each go in tiles of 32 rows."""
+    monkeypatch.setitem(globals(), "ROWS", 32)
+    test_csr_row_block_copies_stay_in_bounds(name, 8)
+
+
 @pytest.mark.parametrize("V", [8, 4], ids=["f64", "f32"])
 @pytest.mark.parametrize("name", ["lap2d_64", "st27_23", "convdiff_20", "ragged_tail", "poisson128"])
 def test_coo_row_block_copies_stay_in_bounds(name, V):
