@@ -27,6 +27,7 @@ struct spx_batch {
     spx_ctx *ctx = nullptr;
     int dtype = SPX_F64;
     int64_t nsys = 0, nrows = 0, nnz = 0, max_n = 0;
+    bool wide = false;  // some system's rows are long (krylov_rows.cuh: product_rows_wide)
     std::vector<int64_t> row_off, nnz_off;
     spx::DBuf d_row_off, d_nnz_off, rp, col, val, val32, order;
     spx::DBuf work;      // 4 vectors of nrows doubles
@@ -61,7 +62,7 @@ inline size_t bout_bytes(int64_t nsys) { return bout_off_cycles(nsys) + round_up
 // row; read through L1, the block being the only reader).  Launch bounds of
 // 1024 threads per SM hold every variant at 64 registers without spills
 // (without the bound, ptxas gave some variants 32 registers and spilled).
-template <class T, int BLOCK, int SOLVER, bool MIXED>
+template <class T, int BLOCK, int SOLVER, bool MIXED, bool WIDE>
 __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
     k_batch(int64_t nsys, const int64_t *__restrict__ row_off, const int64_t *__restrict__ nnz_off,
             const int *__restrict__ rp_all, const int *__restrict__ col_all, const T *__restrict__ val_all,
@@ -79,7 +80,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
         if (q >= nsys) break;
         const int s = order[q];
         const int64_t ro = row_off[s];
-        BlockRows<BLOCK> g((int)(row_off[s + 1] - ro));
+        BlockRows<BLOCK, WIDE> g((int)(row_off[s + 1] - ro));
         const SysOut o = solve_rows<T, BLOCK, SOLVER, MIXED>(
             g, rp_all + ro + s, col_all + nnz_off[s], val_all + nnz_off[s], MIXED ? val32_all + nnz_off[s] : nullptr,
             b_all + ro, x_all + ro, work, nrows, ro, smem_vec ? smem : nullptr, tol, maxit);
@@ -94,11 +95,11 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
 
 namespace {
 
-template <class T, int BLOCK, int SOLVER, bool MIXED>
+template <class T, int BLOCK, int SOLVER, bool MIXED, bool WIDE>
 int launch_batch_t(spx_ctx *ctx, spx_batch *B, const T *b, T *x, double tol, int64_t maxit, BOut out,
                    unsigned *queue)
 {
-    auto kern = k_batch<T, BLOCK, SOLVER, MIXED>;
+    auto kern = k_batch<T, BLOCK, SOLVER, MIXED, WIDE>;
     int smem = (int)(B->max_n * (MIXED ? 8 : sizeof(T)));
     // the opt-in is made once, to all that the kernel's static part leaves: the
     // server's batch lanes launch this kernel from several threads with different
@@ -130,13 +131,17 @@ template <class T, int SOLVER, bool MIXED>
 int launch_batch_b(spx_ctx *ctx, spx_batch *B, int block, const T *b, T *x, double tol, int64_t maxit, BOut out,
                    unsigned *queue)
 {
+#define SPX_BATCH(B_)                                                                                     \
+    B->wide ? launch_batch_t<T, B_, SOLVER, MIXED, true>(ctx, B, b, x, tol, maxit, out, queue)            \
+            : launch_batch_t<T, B_, SOLVER, MIXED, false>(ctx, B, b, x, tol, maxit, out, queue)
     switch (block) {
-    case 128: return launch_batch_t<T, 128, SOLVER, MIXED>(ctx, B, b, x, tol, maxit, out, queue);
-    case 256: return launch_batch_t<T, 256, SOLVER, MIXED>(ctx, B, b, x, tol, maxit, out, queue);
-    case 512: return launch_batch_t<T, 512, SOLVER, MIXED>(ctx, B, b, x, tol, maxit, out, queue);
-    case 1024: return launch_batch_t<T, 1024, SOLVER, MIXED>(ctx, B, b, x, tol, maxit, out, queue);
+    case 128: return SPX_BATCH(128);
+    case 256: return SPX_BATCH(256);
+    case 512: return SPX_BATCH(512);
+    case 1024: return SPX_BATCH(1024);
     default: return fail(SPX_ERR_INVALID, "batched block size must be 128, 256, 512 or 1024");
     }
+#undef SPX_BATCH
 }
 
 int launch_batch(spx_ctx *ctx, spx_batch *B, int block, int solver, int precision, const void *b, void *x,
@@ -237,6 +242,10 @@ extern "C" int spx_batch_create(spx_ctx *ctx, spx_batch **out, int dtype, int64_
     B->nrows = nrows;
     B->nnz = nnz;
     B->max_n = max_n;
+    for (int64_t s = 0; s < nsys && !B->wide; ++s) {
+        const int64_t n = row_off[s + 1] - row_off[s];
+        B->wide = n > 0 && nnz_off[s + 1] - nnz_off[s] >= kGroupWideRow * n;
+    }
     B->row_off.assign(row_off, row_off + nsys + 1);
     B->nnz_off.assign(nnz_off, nnz_off + nsys + 1);
     const size_t V = dtype == SPX_F64 ? 8 : 4;

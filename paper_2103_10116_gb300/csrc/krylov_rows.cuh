@@ -29,11 +29,17 @@
 namespace spx {
 
 constexpr int kGroupMaxRestarts = 3;
+constexpr int kGroupWideRow = 12;  // mean entries per row from which a product takes several lanes per row
 
-// One thread block owns rows [0, n).
-template <int BLOCK> struct BlockRows {
+// One thread block owns rows [0, n).  WIDE: the kernel also holds the product for long
+// rows (product_rows_wide), which a system takes by its own mean row length; kept out of the
+// kernels that meet no such system, whose registers it would take (a batch of 4096 2D
+// Laplacians 30.8 ms, 31.3 with it).
+template <int BLOCK, bool WIDE> struct BlockRows {
     static constexpr int U = 1;  // rows per thread in flight in a product
+    static constexpr bool kWide = WIDE;
     int lo, hi;
+    bool wide = false;
     __device__ explicit BlockRows(int n) : lo(0), hi(n) {}
     __device__ __forceinline__ void sync() { __syncthreads(); }
     template <class T> __device__ __forceinline__ T sum(T v) { return block_sum<T, BLOCK>(v); }
@@ -62,7 +68,9 @@ template <int BLOCK> struct BlockRows {
 template <int CL, int BLOCK, int UROWS = 2> struct ClusterRows {
     static_assert(CL >= 2 && CL <= 32, "cluster size");
     static constexpr int U = UROWS;  // rows per thread in flight in a product
+    static constexpr bool kWide = false;
     int lo, hi;
+    bool wide = false;
     double *part;  // shared: [2][4] partial slots of this block
     double *bc;    // shared: [2] broadcast of the totals
     int slot = 0;
@@ -128,6 +136,72 @@ __device__ __forceinline__ T row_dot(const G &g, const int *__restrict__ rp, con
     return s;
 }
 
+// A product over long rows: L adjacent lanes take a row's entries in turn, 32 bytes
+// of values at a time, and a shuffle tree adds them; a warp does the 32 rows its lanes
+// own, S row groups with CH entries per lane in flight together, and hands each sum to
+// the row's owner, which runs body.  (A thread walking a row of 20 random columns alone
+// fetches a sector per load and lane, and the lines of 1024 such walks do not stay in L1.)
+// ms, a thread per row first: one system of 20 000 rows of 20 random columns, mixed
+// BiCGSTAB 8.9 / 6.7, FP64 15.4 / 14.0; 400 systems of 3000 such rows 3.9 / 3.2, FP64 6.9 /
+// 5.7; 300 systems 27-point 20^3, FP64 CG 13.8 / 8.0, mixed 9.4 / 6.3.  With one row group in
+// flight the mixed solves were slower than a thread per row (one system 9.0).
+template <class T, class V, int BLOCK, class G, class F>
+__device__ __forceinline__ void product_rows_wide(const G &g, const int *__restrict__ rp, const int *__restrict__ col,
+                                                  const V *__restrict__ val, const T *xs, F body)
+{
+    constexpr int L = 32 / (int)sizeof(V), RS = 32 / L;  // lanes per row, rows per group
+    constexpr int S = sizeof(T) == 8 ? 2 : 4, CH = 4;
+    static_assert(L % S == 0, "whole rounds of row groups");
+    const int lane = threadIdx.x & 31, sub = lane % L;
+    for (int base = g.lo + (int)(threadIdx.x & ~31u); base < g.hi; base += BLOCK) {  // warp-uniform
+        const int a = base + lane < g.hi ? rp[base + lane] : 0;
+        const int len = base + lane < g.hi ? rp[base + lane + 1] - a : 0;
+        const int longest = __reduce_max_sync(0xffffffffu, len);
+        T mine = T(0);
+        for (int grp = 0; grp < L; grp += S) {
+            int ra[S], rl[S];
+            T s[S];
+#pragma unroll
+            for (int q = 0; q < S; ++q) {
+                const int src = (grp + q) * RS + lane / L;
+                ra[q] = __shfl_sync(0xffffffffu, a, src);
+                rl[q] = __shfl_sync(0xffffffffu, len, src);
+                s[q] = T(0);
+            }
+            for (int k = 0; k < longest; k += CH * L) {
+                int c[S][CH];
+                T v[S][CH];
+#pragma unroll
+                for (int q = 0; q < S; ++q)
+#pragma unroll
+                    for (int u = 0; u < CH; ++u) {
+                        const bool real = k + sub + u * L < rl[q];
+                        const int at = real ? ra[q] + k + sub + u * L : 0;
+                        c[q][u] = real ? col[at] : -1;
+                        v[q][u] = real ? (T)val[at] : T(0);
+                    }
+#pragma unroll
+                for (int u = 0; u < CH; ++u) {
+                    if (k + u * L >= longest) break;  // warp-uniform
+                    T x[S];
+#pragma unroll
+                    for (int q = 0; q < S; ++q) x[q] = c[q][u] >= 0 ? g.gather(xs, c[q][u]) : T(0);
+#pragma unroll
+                    for (int q = 0; q < S; ++q) s[q] = fma(v[q][u], x[q], s[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < S; ++q) {
+#pragma unroll
+                for (int o = L / 2; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+                const T t = __shfl_sync(0xffffffffu, s[q], (lane % RS) * L);
+                if (lane / RS == grp + q) mine = t;
+            }
+        }
+        if (base + lane < g.hi) body(base + lane, mine);
+    }
+}
+
 // A product over the rows this thread owns: t = (A x)_i, then body(i, t), rows
 // in ascending order.  G::U rows are reduced at once with their loads
 // interleaved, so a thread has U gathers in flight instead of one; each row is
@@ -137,6 +211,11 @@ __device__ __forceinline__ void product_rows(const G &g, const int *__restrict__
                                              const V *__restrict__ val, const T *xs, F body)
 {
     constexpr int U = G::U;
+    if constexpr (G::kWide)
+        if (g.wide) {
+            product_rows_wide<T, V, BLOCK>(g, rp, col, val, xs, body);
+            return;
+        }
     if constexpr (U == 1) {
         for (int i = g.lo + (int)threadIdx.x; i < g.hi; i += BLOCK) body(i, row_dot<T, V>(g, rp, col, val, xs, i));
     } else {
@@ -679,6 +758,7 @@ __device__ SysOut solve_rows(G &g, const int *__restrict__ rp, const int *__rest
     T relres = T(0);
     int status;
     int outer = 0;
+    if constexpr (G::kWide) g.wide = rp[g.hi] - rp[g.lo] >= kGroupWideRow * (g.hi - g.lo);
     if constexpr (!MIXED) {
         T *ps = smem_vec ? reinterpret_cast<T *>(smem_vec) : work + 6 * nrows + ro;
         T *w[6];
