@@ -26,7 +26,9 @@ constexpr int kGridMinRows32 = 256;
 // in ms, the other route first.  CG FP64: 8100 rows 1.36 / 2.05, 15 625 rows 0.86 / 0.88;
 // 27-point 10 648 rows, whose slices do not fit one cluster, 1.10 / 0.55; FP32: 8100 rows
 // 0.14 / 0.27.  Mixed CG: 900 rows 0.41 / 0.52, 2025 rows 1.02 / 0.74.  BiCGSTAB FP64:
-// 256 rows 0.25 / 0.32, 512 rows 0.50 / 0.40; FP32 the same at 512 rows (0.14).
+// 256 rows 0.25 / 0.32, 512 rows 0.50 / 0.40; FP32 the same at 512 rows (0.14).  ELL and COO
+// have the general path otherwise, slower at every size: CG FP64 on 1600 5-point rows in ELL
+// 3.7 / 0.93, mixed CG on 8100 rows in COO 8.5 / 1.4, CGS on 97 336 7-point rows in ELL 3.6 / 1.9.
 constexpr int64_t kGridCgRows64 = 14336;
 constexpr int64_t kGridCgRows32 = 16385;
 constexpr int64_t kGridCgRowsOff = 4096;  // ... where the cluster does not keep the matrix on chip
@@ -40,15 +42,22 @@ constexpr size_t kGridWordBytes = grid_words(kGridMaxBlocks) * 8;
 int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, double tol, int64_t maxit,
                int precision, spx_solve_info *info)
 {
-    if (A->format != SPX_CSR || !A->rp.p || A->n < 1 || A->nnz < 1) return SPX_ERR_UNSUPPORTED;
+    if (A->n < 1 || A->nnz < 1) return SPX_ERR_UNSUPPORTED;
+    const bool csr = A->format == SPX_CSR && A->rp.p;
+    const bool ell = A->ell_w > 0 && (A->format == SPX_ELL || (A->format == SPX_HYB && A->coo_nnz == 0));
+    const bool coo = A->format == SPX_COO && A->coo_nnz > 0;
+    if (!csr && !ell && !coo) return SPX_ERR_UNSUPPORTED;
     if (solver != SPX_CG && solver != SPX_BICGSTAB && solver != SPX_CGS) return SPX_ERR_UNSUPPORTED;
     const bool mixed = precision == SPX_PREC_MIXED;
-    if (mixed ? A->dtype != SPX_F64 || !A->val32.p : (precision == SPX_PREC_F64 ? SPX_F64 : SPX_F32) != A->dtype)
+    const DBuf &val = csr ? A->val : ell ? A->ell_val : A->coo_val;
+    const DBuf &val32 = csr ? A->val32 : ell ? A->ell_val32 : A->coo_val32;
+    if (mixed ? A->dtype != SPX_F64 || !val32.p : (precision == SPX_PREC_F64 ? SPX_F64 : SPX_F32) != A->dtype)
         return SPX_ERR_UNSUPPORTED;  // the general path reports the mismatch
     // one thread per row: rows of similar length only (the row-block SpMV's rule)
     if ((double)A->max_len > 2.0 * A->mean_len + 8.0) return SPX_ERR_UNSUPPORTED;
     const int64_t sms = std::min<int64_t>(ctx->grid_sms, kGridMaxBlocks);
-    const int64_t from = solver != SPX_CG              ? kGridRows
+    const int64_t from = !csr                          ? 1  // the small routes take CSR only
+                         : solver != SPX_CG            ? kGridRows
                          : mixed                       ? kGridCgRowsMixed
                          : !cluster_cg_on_chip(ctx, A) ? kGridCgRowsOff
                          : precision == SPX_PREC_F64   ? kGridCgRows64
@@ -61,7 +70,7 @@ int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, 
     const int r = rows <= kGridBlockMax ? 1 : rows <= 2 * kGridBlockMax ? 2 : 4;
     const int threads = (int)round_up((size_t)ceil_div(rows, (int64_t)r), 32);
     const int blocks = (int)ceil_div(A->n, rows);
-    const int64_t cap = std::min<int64_t>(A->max_len * rows, A->nnz);
+    const int64_t cap = ell ? A->ell_w * rows : std::min<int64_t>(A->max_len * rows, A->nnz);
     const size_t smem = A->dtype == SPX_F64 && !mixed ? grid_smem<double>((int)std::min<int64_t>(cap, 1 << 20))
                                                       : grid_smem<float>((int)std::min<int64_t>(cap, 1 << 20));
     if (smem > (size_t)ctx->max_smem_optin - 1024) return SPX_ERR_UNSUPPORTED;
@@ -73,10 +82,14 @@ int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, 
     g.n = (int)A->n;
     g.rows = (int)rows;
     g.cap = (int)cap;
-    g.rp = A->rp.as<int>();
-    g.col = A->col.as<int>();
-    g.val = mixed ? A->val32.p : A->val.p;
-    g.val64 = A->val.p;
+    g.rp = csr ? A->rp.as<int>() : nullptr;
+    g.crow = coo ? A->coo_row.as<int>() : nullptr;
+    g.nnz = (int)A->nnz;
+    g.ell_ld = ell ? A->ell_ld : 0;
+    g.ell_w = (int)A->ell_w;
+    g.col = csr ? A->col.as<int>() : ell ? A->ell_col.as<int>() : A->coo_col.as<int>();
+    g.val = mixed ? val32.p : val.p;
+    g.val64 = val.p;
     g.b = b;
     g.x = x;
     g.ps = w + head;

@@ -1,6 +1,6 @@
 // grid_solve.cuh -- a whole Krylov solve in one cooperative launch over the
 // device: CG, BiCGSTAB and CGS (FP64 or FP32), mixed-precision CG with reliable
-// updates, and FP64 refinement around FP32 BiCGSTAB / CGS, for CSR systems of
+// updates, and FP64 refinement around FP32 BiCGSTAB / CGS, for systems (CSR, ELL, COO) of
 // rows of similar length whose matrix fits the SMs' shared memory together.
 //
 // The general path pays three to five launches and as many device-wide
@@ -44,7 +44,11 @@ struct GridOut {
 
 struct GridArgs {
     int n, rows, cap;  // rows of the system and per block, entries the shared slice holds
-    const int *rp, *col;
+    const int *rp, *col;  // CSR; COO: crow instead of rp (rows found by search), nnz
+    const int *crow;
+    int nnz;
+    int64_t ell_ld;  // ELL (col, val column-major; rp, crow null): rows between slabs
+    int ell_w;
     const void *val, *val64;  // the values the products use; the FP64 values of a mixed solve
     const void *b;
     void *x;
@@ -330,6 +334,27 @@ __device__ __forceinline__ T slice_dot(const int *col, const V *val, int len, co
     return s;
 }
 
+// the same in FP64 with values `stride` apart (ELL keeps a row's values a slab apart)
+__device__ __forceinline__ double slice_dot64(const int *col, const double *val, int64_t stride, int len, const double *x)
+{
+    if (stride == 1) return slice_dot<double, double>(col, val, len, x);
+    double s = 0.0;
+    for (int k = 0; k < len; ++k) s = fma(val[k * stride], x[col[k]], s);
+    return s;
+}
+
+// first entry of row i (i <= n) in row-sorted COO
+__device__ __forceinline__ int coo_row_start(const int *__restrict__ crow, int nnz, int i)
+{
+    int lo = 0, hi = nnz;
+    while (lo < hi) {
+        const int mid = lo + ((hi - lo) >> 1);
+        if (crow[mid] < i) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
 // This thread's rows: u-th row lo + tid + u blockDim, its entries at [at, at + len) of the slice.
 template <int R> struct GridRows {
     int at[R], len[R], row[R];  // row: -1 past the block's rows
@@ -609,7 +634,7 @@ __device__ __forceinline__ int grid_solve_mixed(GridTeam &tm, const GridRows<R> 
                                                 const GridArgs &A, int j0, GridOut &o)
 {
     const double *b = static_cast<const double *>(A.b);
-    const double *v64 = static_cast<const double *>(A.val64) + j0;
+    const double *v64 = static_cast<const double *>(A.val64) + j0;  // (ELL: j0 = 0, a row's values ell_ld apart)
     double *xg = static_cast<double *>(A.x);
     float *ps = static_cast<float *>(A.ps);
     double x[R], r64[R], bb = 0.0;
@@ -633,7 +658,8 @@ __device__ __forceinline__ int grid_solve_mixed(GridTeam &tm, const GridRows<R> 
         rr64 = 0.0;
         SPX_EACH(u)
         {
-            r64[u] = b[G.row[u]] - slice_dot<double, double>(sc + G.at[u], v64 + G.at[u], G.len[u], A.xs);
+            const double *v = A.ell_ld ? v64 + G.row[u] : v64 + G.at[u];
+            r64[u] = b[G.row[u]] - slice_dot64(sc + G.at[u], v, A.ell_ld ? A.ell_ld : 1, G.len[u], A.xs);
             rr64 = fma(r64[u], r64[u], rr64);
         }
         return tm.sum(rr64);
@@ -800,26 +826,47 @@ __global__ void __launch_bounds__(kGridBlockMax, 1) k_grid_solve(GridArgs A)
     const int tid = threadIdx.x, nt = blockDim.x;
     if (tid == 0) s_dead = 0;
     const int lo = min(A.n, (int)blockIdx.x * A.rows), hi = min(A.n, lo + A.rows);
-    const int j0 = A.rp[lo], j1 = A.rp[hi];
     const V *val = static_cast<const V *>(A.val);
     GridRows<R> G;
+    int j0 = 0;
+    bool fits = true;
+    if (A.ell_ld) {
+        // a row's entries fill its first slots; row lo + q goes to the slice at q ell_w
+        fits = (hi - lo) * A.ell_w <= A.cap;
 #pragma unroll
-    for (int u = 0; u < R; ++u) {
-        const int i = lo + tid + u * nt;
-        G.row[u] = i < hi ? i : -1;
-        G.at[u] = i < hi ? A.rp[i] - j0 : 0;
-        G.len[u] = i < hi ? A.rp[i + 1] - j0 - G.at[u] : 0;
-    }
-    if (j1 - j0 <= A.cap) {
-        for (int k = tid; k < j1 - j0; k += nt) {
-            sc[k] = A.col[j0 + k];
-            sv[k] = val[j0 + k];
+        for (int u = 0; u < R; ++u) {
+            const int q = tid + u * nt, i = lo + q;
+            G.row[u] = i < hi ? i : -1;
+            G.at[u] = q * A.ell_w;
+            G.len[u] = 0;
+            if (i >= hi || !fits) continue;
+            for (int k = 0; k < A.ell_w; ++k) {
+                const int c = A.col[k * A.ell_ld + i];
+                if (c < 0) break;
+                sc[G.at[u] + k] = c;
+                sv[G.at[u] + k] = val[k * A.ell_ld + i];
+                G.len[u] = k + 1;
+            }
         }
-    } else {  // never, for the matrix the slice was sized for
-        if (tid == 0) atomicOr(A.err, DEVERR_BOUNDS);
+    } else {
+        auto start = [&](int i) { return A.crow ? coo_row_start(A.crow, A.nnz, i) : A.rp[i]; };
+        j0 = start(lo);
+        const int nz = start(hi) - j0;
+        fits = nz <= A.cap;
 #pragma unroll
-        for (int u = 0; u < R; ++u) G.len[u] = 0;
+        for (int u = 0; u < R; ++u) {
+            const int i = lo + tid + u * nt;
+            G.row[u] = i < hi ? i : -1;
+            G.at[u] = i < hi ? start(i) - j0 : 0;
+            G.len[u] = i < hi && fits ? start(i + 1) - j0 - G.at[u] : 0;
+        }
+        if (fits)
+            for (int k = tid; k < nz; k += nt) {
+                sc[k] = A.col[j0 + k];
+                sv[k] = val[j0 + k];
+            }
     }
+    if (!fits && tid == 0) atomicOr(A.err, DEVERR_BOUNDS);  // never, for the matrix the slice was sized for
     __syncthreads();
     GridOut o{1, SPX_MAX_ITER, 0, 0, 0, 0.0, 0.0};
     int st;

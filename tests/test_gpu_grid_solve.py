@@ -36,17 +36,18 @@ def _t(a):
     return torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
 
 
-def _both(spx, ctx, mat, b, solver, precision, tol, maxit=20000, x0=None):
+def _both(spx, ctx, mat, b, solver, precision, tol, maxit=20000, x0=None, fmt="csr"):
     """(info, x) by the automatic route, solved twice (equal bits), and by the general path."""
     rp, col, val = mat
     f32 = precision == "f32"
     dt = torch.float32 if f32 else torch.float64
     out = []
     for pinned in (False, True):
-        A = spx.spx_matrix_create(ctx, "csr", _t(rp), _t(col), _t(val).to(dt),
+        A = spx.spx_matrix_create(ctx, fmt, _t(rp), _t(col), _t(val).to(dt),
                                   flags=spx.SPX_MIXED_SHADOW if precision == "mixed" else 0)
         if pinned:
-            spx.spx_matrix_set_kernel(A, spx.SPX_KERNEL_CSR_ROWS, 0)
+            kernel = {"csr": (spx.SPX_KERNEL_CSR_ROWS, 0), "coo": (spx.SPX_KERNEL_COO, 216)}.get(fmt, (spx.SPX_KERNEL_ELL, 1))
+            spx.spx_matrix_set_kernel(A, *kernel)
         bt = _t(b).to(dt)
         xs = []
         for _ in range(1 if pinned else 2):
@@ -99,6 +100,23 @@ def test_long_rows(spx, ctx, solver, precision):
     assert abs(info.iterations - ginfo.iterations) <= max(3, ginfo.iterations // 10)
     # the diagonal is twice the sum of the others' magnitudes: ||A^-1||_inf <= 1 / min(diag / 2)
     assert np.linalg.norm(x - xs) <= 1e3 * tol * np.linalg.norm(xs)
+
+
+@pytest.mark.parametrize("fmt", ["ell", "coo", "hyb"])
+@pytest.mark.parametrize("solver,precision", [("cg", "f64"), ("cg", "mixed"), ("bicgstab", "f64"), ("cgs", "mixed"), ("bicgstab", "f32")])
+@pytest.mark.parametrize("n", [1, 33, 4099, 90001])
+def test_other_formats(spx, ctx, n, solver, precision, fmt):
+    """ELL (HYB without overflow included) and COO fill the same slices: ragged rows, empty ones beside them."""
+    mat = synth.ragged_laplace2d(n, 0.2) if solver == "cg" or n < 40 else synth.DiagDomFamily(n, seed=5).matrix(n)
+    if fmt == "hyb" and solver != "cg" and n >= 40:
+        pytest.skip("overflow entries: the general path")
+    b = oracle.spmv_csr(*mat, synth.uniform_vector(n, seed=3))
+    tol = 1e-5 if precision == "f32" else 1e-10
+    (info, x), (ginfo, gx) = _both(spx, ctx, mat, b, solver, precision, tol, fmt=fmt)
+    assert info.status == ginfo.status == spx.SPX_CONVERGED and info.relres_true <= tol
+    assert abs(info.iterations - ginfo.iterations) <= max(4, ginfo.iterations // 5)
+    if precision != "f32":
+        assert np.linalg.norm(b - oracle.spmv_csr(*mat, x)) / np.linalg.norm(b) <= residual_limit(*mat, b, x, tol)
 
 
 @pytest.mark.parametrize("solver", ["cg", "bicgstab", "cgs"])
