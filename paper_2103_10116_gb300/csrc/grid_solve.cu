@@ -6,11 +6,14 @@
 
 namespace spx {
 
-template <class T, class V>
+template <class T, class V, bool PRE>
 int grid_launch(spx_ctx *ctx, const GridArgs &A, int solver, int blocks, int threads, int r);
-extern template int grid_launch<double, double>(spx_ctx *, const GridArgs &, int, int, int, int);
-extern template int grid_launch<float, float>(spx_ctx *, const GridArgs &, int, int, int, int);
-extern template int grid_launch<double, float>(spx_ctx *, const GridArgs &, int, int, int, int);
+extern template int grid_launch<double, double, false>(spx_ctx *, const GridArgs &, int, int, int, int);
+extern template int grid_launch<double, double, true>(spx_ctx *, const GridArgs &, int, int, int, int);
+extern template int grid_launch<float, float, false>(spx_ctx *, const GridArgs &, int, int, int, int);
+extern template int grid_launch<float, float, true>(spx_ctx *, const GridArgs &, int, int, int, int);
+extern template int grid_launch<double, float, false>(spx_ctx *, const GridArgs &, int, int, int, int);
+extern template int grid_launch<double, float, true>(spx_ctx *, const GridArgs &, int, int, int, int);
 
 namespace {
 
@@ -29,6 +32,9 @@ constexpr int kGridMinRows32 = 256;
 // 256 rows 0.25 / 0.32, 512 rows 0.50 / 0.40; FP32 the same at 512 rows (0.14).  ELL and COO
 // have the general path otherwise, slower at every size: CG FP64 on 1600 5-point rows in ELL
 // 3.7 / 0.93, mixed CG on 8100 rows in COO 8.5 / 1.4, CGS on 97 336 7-point rows in ELL 3.6 / 1.9.
+// So has Jacobi: CG FP64 on 400 5-point rows 2.0 / 0.52, on 262 144 7-point rows 6.9 / 4.0, mixed
+// on 4096 5-point rows 5.8 / 1.5; BiCGSTAB FP64 on 300 random rows 0.90 / 0.16, on 30 000 in COO
+// 0.65 / 0.25.
 constexpr int64_t kGridCgRows64 = 14336;
 constexpr int64_t kGridCgRows32 = 16385;
 constexpr int64_t kGridCgRowsOff = 4096;  // ... where the cluster does not keep the matrix on chip
@@ -40,7 +46,7 @@ constexpr size_t kGridWordBytes = grid_words(kGridMaxBlocks) * 8;
 
 // See spx_internal.cuh.
 int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, double tol, int64_t maxit,
-               int precision, spx_solve_info *info)
+               int precision, bool jacobi, spx_solve_info *info)
 {
     if (A->n < 1 || A->nnz < 1) return SPX_ERR_UNSUPPORTED;
     const bool csr = A->format == SPX_CSR && A->rp.p;
@@ -56,7 +62,7 @@ int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, 
     // one thread per row: rows of similar length only (the row-block SpMV's rule)
     if ((double)A->max_len > 2.0 * A->mean_len + 8.0) return SPX_ERR_UNSUPPORTED;
     const int64_t sms = std::min<int64_t>(ctx->grid_sms, kGridMaxBlocks);
-    const int64_t from = !csr                          ? 1  // the small routes take CSR only
+    const int64_t from = !csr || jacobi                ? 1  // the small routes take plain CSR only
                          : solver != SPX_CG            ? kGridRows
                          : mixed                       ? kGridCgRowsMixed
                          : !cluster_cg_on_chip(ctx, A) ? kGridCgRowsOff
@@ -101,9 +107,15 @@ int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, 
     g.maxit = (long long)maxit;
     SPX_CUDA(cudaMemsetAsync(w, 0, grid_words(blocks) * 8, ctx->stream));
     SPX_CUDA(cudaMemsetAsync(g.out, 0, sizeof(GridOut), ctx->stream));
-    const int st = mixed ? grid_launch<double, float>(ctx, g, solver, blocks, threads, r)
-                   : A->dtype == SPX_F64 ? grid_launch<double, double>(ctx, g, solver, blocks, threads, r)
-                                         : grid_launch<float, float>(ctx, g, solver, blocks, threads, r);
+    int st;
+    if (jacobi)
+        st = mixed                   ? grid_launch<double, float, true>(ctx, g, solver, blocks, threads, r)
+             : A->dtype == SPX_F64   ? grid_launch<double, double, true>(ctx, g, solver, blocks, threads, r)
+                                     : grid_launch<float, float, true>(ctx, g, solver, blocks, threads, r);
+    else
+        st = mixed                   ? grid_launch<double, float, false>(ctx, g, solver, blocks, threads, r)
+             : A->dtype == SPX_F64   ? grid_launch<double, double, false>(ctx, g, solver, blocks, threads, r)
+                                     : grid_launch<float, float, false>(ctx, g, solver, blocks, threads, r);
     if (st != SPX_OK) return st;
     GridOut h;
     SPX_CUDA(cudaMemcpyAsync(&h, g.out, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));

@@ -1,7 +1,8 @@
 // grid_solve.cuh -- a whole Krylov solve in one cooperative launch over the
 // device: CG, BiCGSTAB and CGS (FP64 or FP32), mixed-precision CG with reliable
 // updates, and FP64 refinement around FP32 BiCGSTAB / CGS, for systems (CSR, ELL, COO) of
-// rows of similar length whose matrix fits the SMs' shared memory together.
+// rows of similar length whose matrix fits the SMs' shared memory together; without
+// preconditioner or with Jacobi (mixed CG then as refinement around FP32 CG).
 //
 // The general path pays three to five launches and as many device-wide
 // reductions per iteration, 15 to 25 us however small the system (FP32 CG on a
@@ -371,20 +372,29 @@ constexpr int kDead = -1;
 
 // CG, the recurrence of cg_iter.  x: the iterate (registers); r: on entry the
 // residual.  Ends with a status; iters and last (||r||^2) go on from the caller's.
-template <class T, class V, int R>
+// PRE (here and below): Jacobi, di the rows' M^-1.
+template <class T, class V, int R, bool PRE>
 __device__ __forceinline__ int grid_cg(GridTeam &tm, const GridRows<R> &G, const int *sc, const V *sv, T *ps, T (&x)[R],
-                                       T (&r)[R], T rho, T tol2, long long maxit, long long &iters, T &last)
+                                       T (&r)[R], const T (&di)[R], T rho, T tol2, long long maxit, long long &iters,
+                                       T &last)
 {
     T p[R], q[R];
     last = rho;
     if (rho <= tol2) return SPX_CONVERGED;
     if (iters >= maxit) return SPX_MAX_ITER;
+    if constexpr (PRE) rho = T(0);
     SPX_EACH(u)
     {
-        p[u] = r[u];
+        p[u] = PRE ? di[u] * r[u] : r[u];
         ps[G.row[u]] = p[u];
+        if constexpr (PRE) rho = fma(r[u], p[u], rho);
     }
-    SPX_LIVE(tm.sync());
+    if constexpr (PRE) {  // r.z; also publishes p
+        SPX_LIVE(tm.sum_pub(rho));
+        if (rho == T(0)) return SPX_BREAKDOWN;
+    } else {
+        SPX_LIVE(tm.sync());
+    }
     for (;;) {
         T pq = T(0);
         SPX_EACH(u)
@@ -395,23 +405,26 @@ __device__ __forceinline__ int grid_cg(GridTeam &tm, const GridRows<R> &G, const
         T alpha;
         SPX_LIVE(tm.sum(pq, alpha, [=](T s) { return rho / s; }));
         if (pq == T(0)) return SPX_BREAKDOWN;
-        T rr = T(0);
+        T rr = T(0), rz = T(0);
         SPX_EACH(u)
         {
             r[u] = fma(-alpha, q[u], r[u]);
             rr = fma(r[u], r[u], rr);
+            if constexpr (PRE) rz = fma(r[u], di[u] * r[u], rz);
             x[u] = fma(alpha, p[u], x[u]);
         }
         T beta;
-        SPX_LIVE(tm.sum(rr, beta, [=](T s) { return s / rho; }));
+        if constexpr (PRE) SPX_LIVE(tm.sum2(rr, rz, beta, [=](T, T c) { return c / rho; }));
+        else SPX_LIVE(tm.sum(rr, beta, [=](T s) { return s / rho; }));
         ++iters;
         last = rr;
         if (rr <= tol2) return SPX_CONVERGED;
         if (iters >= maxit) return SPX_MAX_ITER;
-        rho = rr;
+        if (PRE && rz == T(0)) return SPX_BREAKDOWN;
+        rho = PRE ? rz : rr;
         SPX_EACH(u)
         {
-            p[u] = fma(beta, p[u], r[u]);
+            p[u] = fma(beta, p[u], PRE ? di[u] * r[u] : r[u]);
             ps[G.row[u]] = p[u];
         }
         SPX_LIVE(tm.sync());
@@ -419,10 +432,10 @@ __device__ __forceinline__ int grid_cg(GridTeam &tm, const GridRows<R> &G, const
 }
 
 // BiCGSTAB, the recurrence of bi_iter (r^ = the residual on entry)
-template <class T, class V, int R>
+template <class T, class V, int R, bool PRE>
 __device__ __forceinline__ int grid_bicgstab(GridTeam &tm, const GridRows<R> &G, const int *sc, const V *sv, T *ps,
-                                             T (&x)[R], T (&r)[R], T rho, T tol2, long long maxit, long long &iters,
-                                             T &last)
+                                             T (&x)[R], T (&r)[R], const T (&di)[R], T rho, T tol2, long long maxit,
+                                             long long &iters, T &last)
 {
     T rh[R], p[R], v[R];
     last = rho;
@@ -432,7 +445,7 @@ __device__ __forceinline__ int grid_bicgstab(GridTeam &tm, const GridRows<R> &G,
     {
         rh[u] = r[u];
         p[u] = r[u];
-        ps[G.row[u]] = r[u];
+        ps[G.row[u]] = PRE ? di[u] * r[u] : r[u];
     }
     SPX_LIVE(tm.sync());
     for (;;) {
@@ -449,13 +462,13 @@ __device__ __forceinline__ int grid_bicgstab(GridTeam &tm, const GridRows<R> &G,
         SPX_EACH(u)
         {
             r[u] = fma(-alpha, v[u], r[u]);  // s, in r's place
-            ps[G.row[u]] = r[u];
+            ps[G.row[u]] = PRE ? di[u] * r[u] : r[u];
             ss = fma(r[u], r[u], ss);
         }
         SPX_LIVE(tm.sum_pub(ss));
         ++iters;
         if (ss <= tol2) {
-            SPX_EACH(u) x[u] = fma(alpha, p[u], x[u]);
+            SPX_EACH(u) x[u] = fma(alpha, PRE ? di[u] * p[u] : p[u], x[u]);
             last = ss;
             return SPX_CONVERGED;
         }
@@ -472,7 +485,8 @@ __device__ __forceinline__ int grid_bicgstab(GridTeam &tm, const GridRows<R> &G,
         T rr = T(0), rhr = T(0);
         SPX_EACH(u)
         {
-            x[u] = fma(omega, r[u], fma(alpha, p[u], x[u]));
+            x[u] = PRE ? fma(omega, di[u] * r[u], fma(alpha, di[u] * p[u], x[u]))
+                       : fma(omega, r[u], fma(alpha, p[u], x[u]));
             r[u] = fma(-omega, t[u], r[u]);
             rr = fma(r[u], r[u], rr);
             rhr = fma(rh[u], r[u], rhr);
@@ -488,7 +502,7 @@ __device__ __forceinline__ int grid_bicgstab(GridTeam &tm, const GridRows<R> &G,
         SPX_EACH(u)
         {
             p[u] = fma(beta, fma(-omega, v[u], p[u]), r[u]);
-            ps[G.row[u]] = p[u];
+            ps[G.row[u]] = PRE ? di[u] * p[u] : p[u];
         }
         SPX_LIVE(tm.sync());
     }
@@ -496,10 +510,10 @@ __device__ __forceinline__ int grid_bicgstab(GridTeam &tm, const GridRows<R> &G,
 
 // CGS, the recurrence of cgs_iter (r^ = the residual on entry).  stall > 0: the
 // inner cycle's stall rule.
-template <class T, class V, int R>
+template <class T, class V, int R, bool PRE>
 __device__ __forceinline__ int grid_cgs(GridTeam &tm, const GridRows<R> &G, const int *sc, const V *sv, T *ps, T (&x)[R],
-                                        T (&r)[R], T rho, T bb, T tol2, long long maxit, int stall, long long &iters,
-                                        T &last)
+                                        T (&r)[R], const T (&di)[R], T rho, T bb, T tol2, long long maxit, int stall,
+                                        long long &iters, T &last)
 {
     T rh[R], p[R], uu[R], q[R];
     T mark = T(1);
@@ -510,7 +524,7 @@ __device__ __forceinline__ int grid_cgs(GridTeam &tm, const GridRows<R> &G, cons
     SPX_EACH(u)
     {
         rh[u] = p[u] = uu[u] = r[u];
-        ps[G.row[u]] = r[u];
+        ps[G.row[u]] = PRE ? di[u] * r[u] : r[u];
     }
     SPX_LIVE(tm.sync());
     for (;;) {
@@ -526,7 +540,7 @@ __device__ __forceinline__ int grid_cgs(GridTeam &tm, const GridRows<R> &G, cons
         SPX_EACH(u)
         {
             q[u] = fma(-alpha, q[u], uu[u]);
-            const T w = uu[u] + q[u];
+            const T w = PRE ? di[u] * (uu[u] + q[u]) : uu[u] + q[u];
             x[u] = fma(alpha, w, x[u]);
             ps[G.row[u]] = w;
         }
@@ -560,16 +574,16 @@ __device__ __forceinline__ int grid_cgs(GridTeam &tm, const GridRows<R> &G, cons
         {
             uu[u] = fma(beta, q[u], r[u]);
             p[u] = fma(beta, fma(beta, p[u], q[u]), uu[u]);
-            ps[G.row[u]] = p[u];
+            ps[G.row[u]] = PRE ? di[u] * p[u] : p[u];
         }
         SPX_LIVE(tm.sync());
     }
 }
 
 // One solve in one precision: b = 0, restarts from the true residual (run_short's policy)
-template <class T, int SOLVER, int R>
+template <class T, int SOLVER, int R, bool PRE>
 __device__ __forceinline__ int grid_solve_one(GridTeam &tm, const GridRows<R> &G, const int *sc, const T *sv,
-                                              const GridArgs &A, GridOut &o)
+                                              const T (&di)[R], const GridArgs &A, GridOut &o)
 {
     const T *b = static_cast<const T *>(A.b);
     T *xg = static_cast<T *>(A.x), *ps = static_cast<T *>(A.ps);
@@ -603,10 +617,11 @@ __device__ __forceinline__ int grid_solve_one(GridTeam &tm, const GridRows<R> &G
     for (;;) {
         T last;
         int st;
-        if constexpr (SOLVER == SPX_CG) st = grid_cg<T, T, R>(tm, G, sc, sv, ps, x, r, rr, tol2, A.maxit, o.iters, last);
+        if constexpr (SOLVER == SPX_CG)
+            st = grid_cg<T, T, R, PRE>(tm, G, sc, sv, ps, x, r, di, rr, tol2, A.maxit, o.iters, last);
         else if constexpr (SOLVER == SPX_CGS)
-            st = grid_cgs<T, T, R>(tm, G, sc, sv, ps, x, r, rr, bb, tol2, A.maxit, 0, o.iters, last);
-        else st = grid_bicgstab<T, T, R>(tm, G, sc, sv, ps, x, r, rr, tol2, A.maxit, o.iters, last);
+            st = grid_cgs<T, T, R, PRE>(tm, G, sc, sv, ps, x, r, di, rr, bb, tol2, A.maxit, 0, o.iters, last);
+        else st = grid_bicgstab<T, T, R, PRE>(tm, G, sc, sv, ps, x, r, di, rr, tol2, A.maxit, o.iters, last);
         if (st == kDead) return kDead;
         o.status = st;
         o.relres = (double)sqrt(last / bb);
@@ -626,12 +641,12 @@ __device__ __forceinline__ int grid_solve_one(GridTeam &tm, const GridRows<R> &G
     return 0;
 }
 
-// Mixed precision: CG with reliable updates (run_cg_reliable's policy), BiCGSTAB
-// and CGS as FP64 refinement (run_ir's policy).  sv: FP32 values; the FP64
+// Mixed precision: CG with reliable updates (run_cg_reliable's policy), BiCGSTAB,
+// CGS and preconditioned CG as FP64 refinement (run_ir's policy).  sv: FP32 values; the FP64
 // residual reads the FP64 values from global memory.
-template <int SOLVER, int R>
+template <int SOLVER, int R, bool PRE>
 __device__ __forceinline__ int grid_solve_mixed(GridTeam &tm, const GridRows<R> &G, const int *sc, const float *sv,
-                                                const GridArgs &A, int j0, GridOut &o)
+                                                const float (&di)[R], const GridArgs &A, int j0, GridOut &o)
 {
     const double *b = static_cast<const double *>(A.b);
     const double *v64 = static_cast<const double *>(A.val64) + j0;  // (ELL: j0 = 0, a row's values ell_ld apart)
@@ -665,7 +680,7 @@ __device__ __forceinline__ int grid_solve_mixed(GridTeam &tm, const GridRows<R> 
         return tm.sum(rr64);
     };
     SPX_LIVE(residual64());
-    if constexpr (SOLVER == SPX_CG) {
+    if constexpr (SOLVER == SPX_CG && !PRE) {
         o.relres = sqrt(rr64 / bb);
         o.status = o.relres <= A.tol ? SPX_CONVERGED : SPX_MAX_ITER;
         if (o.status != SPX_CONVERGED) {
@@ -784,9 +799,12 @@ __device__ __forceinline__ int grid_solve_mixed(GridTeam &tm, const GridRows<R> 
                 const long long cyc = min(A.maxit - o.iters, (long long)kIrInnerCap);
                 long long it = 0;
                 if constexpr (SOLVER == SPX_CGS)
-                    st = grid_cgs<float, float, R>(tm, G, sc, sv, ps, d, r, bb32, bb32, tol2, cyc, kIrCgsStall, it, last);
+                    st = grid_cgs<float, float, R, PRE>(tm, G, sc, sv, ps, d, r, di, bb32, bb32, tol2, cyc, kIrCgsStall,
+                                                        it, last);
+                else if constexpr (SOLVER == SPX_CG)
+                    st = grid_cg<float, float, R, PRE>(tm, G, sc, sv, ps, d, r, di, bb32, tol2, cyc, it, last);
                 else
-                    st = grid_bicgstab<float, float, R>(tm, G, sc, sv, ps, d, r, bb32, tol2, cyc, it, last);
+                    st = grid_bicgstab<float, float, R, PRE>(tm, G, sc, sv, ps, d, r, di, bb32, tol2, cyc, it, last);
                 o.iters += it;
             }
             if (st == kDead) return kDead;
@@ -809,7 +827,7 @@ template <class V> constexpr size_t grid_smem(int cap)
 }
 
 // T: the precision of b and x; V: of the values the products use (V = float, T = double: mixed)
-template <class T, class V, int SOLVER, int R>
+template <class T, class V, int SOLVER, int R, bool PRE>
 __global__ void __launch_bounds__(kGridBlockMax, 1) k_grid_solve(GridArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -868,19 +886,38 @@ __global__ void __launch_bounds__(kGridBlockMax, 1) k_grid_solve(GridArgs A)
     }
     if (!fits && tid == 0) atomicOr(A.err, DEVERR_BOUNDS);  // never, for the matrix the slice was sized for
     __syncthreads();
+    // M^-1 = 1 / (the sum of the row's diagonal entries), 1 where that is 0 (k_jacobi_dinv's rule, from
+    // the matrix's own values)
+    V di[R];
+    if constexpr (PRE) {
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            double d = 0.0;
+            for (int k = 0; k < G.len[u]; ++k)
+                if (sc[G.at[u] + k] == G.row[u]) {
+                    if constexpr (sizeof(T) == sizeof(V)) {
+                        d += (double)sv[G.at[u] + k];
+                    } else {
+                        const double *v64 = static_cast<const double *>(A.val64);
+                        d += A.ell_ld ? v64[k * A.ell_ld + G.row[u]] : v64[j0 + G.at[u] + k];
+                    }
+                }
+            di[u] = d != 0.0 ? (V)(1.0 / d) : V(1);
+        }
+    }
     GridOut o{1, SPX_MAX_ITER, 0, 0, 0, 0.0, 0.0};
     int st;
-    if constexpr (sizeof(T) != sizeof(V)) st = grid_solve_mixed<SOLVER, R>(tm, G, sc, sv, A, j0, o);
-    else st = grid_solve_one<T, SOLVER, R>(tm, G, sc, sv, A, o);
+    if constexpr (sizeof(T) != sizeof(V)) st = grid_solve_mixed<SOLVER, R, PRE>(tm, G, sc, sv, di, A, j0, o);
+    else st = grid_solve_one<T, SOLVER, R, PRE>(tm, G, sc, sv, di, A, o);
     if (st != kDead && blockIdx.x == 0 && tid == 0) *A.out = o;
 }
 
 // Launch of one (T, V): grid_f64.cu, grid_f32.cu, grid_mixed.cu.  SPX_ERR_UNSUPPORTED
 // when the device cannot hold the grid at once.
-template <class T, class V, int SOLVER, int R>
+template <class T, class V, int SOLVER, int R, bool PRE>
 int grid_launch_r(spx_ctx *ctx, const GridArgs &A, int blocks, int threads)
 {
-    auto kern = k_grid_solve<T, V, SOLVER, R>;
+    auto kern = k_grid_solve<T, V, SOLVER, R, PRE>;
     const size_t smem = grid_smem<V>(A.cap);
     int lim = 0;
     SPX_TRY(smem_optin(reinterpret_cast<const void *>(kern), -1, &lim));
@@ -903,20 +940,20 @@ int grid_launch_r(spx_ctx *ctx, const GridArgs &A, int blocks, int threads)
     return e == cudaSuccess ? SPX_OK : cuda_fail(e, "cudaLaunchKernelEx(k_grid_solve)");
 }
 
-template <class T, class V, int SOLVER>
+template <class T, class V, int SOLVER, bool PRE>
 int grid_launch_s(spx_ctx *ctx, const GridArgs &A, int blocks, int threads, int r)
 {
-    if (r == 1) return grid_launch_r<T, V, SOLVER, 1>(ctx, A, blocks, threads);
-    if (r == 2) return grid_launch_r<T, V, SOLVER, 2>(ctx, A, blocks, threads);
-    return grid_launch_r<T, V, SOLVER, 4>(ctx, A, blocks, threads);
+    if (r == 1) return grid_launch_r<T, V, SOLVER, 1, PRE>(ctx, A, blocks, threads);
+    if (r == 2) return grid_launch_r<T, V, SOLVER, 2, PRE>(ctx, A, blocks, threads);
+    return grid_launch_r<T, V, SOLVER, 4, PRE>(ctx, A, blocks, threads);
 }
 
-template <class T, class V>
+template <class T, class V, bool PRE>
 int grid_launch(spx_ctx *ctx, const GridArgs &A, int solver, int blocks, int threads, int r)
 {
-    if (solver == SPX_CG) return grid_launch_s<T, V, SPX_CG>(ctx, A, blocks, threads, r);
-    if (solver == SPX_CGS) return grid_launch_s<T, V, SPX_CGS>(ctx, A, blocks, threads, r);
-    return grid_launch_s<T, V, SPX_BICGSTAB>(ctx, A, blocks, threads, r);
+    if (solver == SPX_CG) return grid_launch_s<T, V, SPX_CG, PRE>(ctx, A, blocks, threads, r);
+    if (solver == SPX_CGS) return grid_launch_s<T, V, SPX_CGS, PRE>(ctx, A, blocks, threads, r);
+    return grid_launch_s<T, V, SPX_BICGSTAB, PRE>(ctx, A, blocks, threads, r);
 }
 
 }  // namespace spx

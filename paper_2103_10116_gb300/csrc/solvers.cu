@@ -2154,11 +2154,11 @@ int solve_typed(spx_ctx *ctx, spx_matrix *A, const T *b, T *x, int solver, doubl
 // Small and mid-size systems are solved by one launch that runs every iteration,
 // where the general path pays three launches and a device-wide reduction per
 // iteration (the 2D Laplacian on a 64 x 64 grid, n = 4096: 23 us per CG iteration
-// there).  CSR matrices whose SpMV kernel is left to the library, no
-// preconditioner, run to a tolerance:
-//   * from the sizes at which it measured fastest (grid_solve.cu), and up to what
-//     the SMs' shared memory and registers hold, over the whole device;
-//   * below, CG in FP64 or FP32 on one cluster of 16 (or 8) SMs (cluster.cu; up to
+// there).  Matrices whose SpMV kernel is left to the library, run to a tolerance:
+//   * without preconditioner or with Jacobi, from the sizes at which it measured
+//     fastest (grid_solve.cu), and up to what the SMs' shared memory and registers
+//     hold, over the whole device;
+//   * below, CSR without preconditioner: CG in FP64 or FP32 on one cluster of 16 (or 8) SMs (cluster.cu; up to
 //     kSmallSolveRows rows where the first route does not take the system), and
 //     BiCGSTAB, CGS and mixed precision on up to kSmallBatchRows rows in the
 //     persistent batched kernel as a batch of one (one SM, whose two FP64 lanes
@@ -2222,8 +2222,8 @@ int solve_entry(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver,
         info->time_ms = tm.ms();
         return st;
     }
-    if (fixed == 0 && !pre && bs == 0 && A->kernel == SPX_KERNEL_AUTO) {  // a pinned SpMV kernel keeps the general path
-        st = grid_solve(ctx, A, b, x, solver, tol, maxit, precision, info);
+    if (fixed == 0 && bs == 0 && A->kernel == SPX_KERNEL_AUTO) {  // a pinned SpMV kernel keeps the general path
+        st = grid_solve(ctx, A, b, x, solver, tol, maxit, precision, pre, info);
         if (st != SPX_ERR_UNSUPPORTED) {
             info->time_ms = tm.ms();
             return st;

@@ -215,12 +215,12 @@ int cluster_cg_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, double
 int cluster_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, double tol, int64_t maxit,
                   int precision, spx_solve_info *info);
 
-// A whole solve (CG, BiCGSTAB or CGS; F64, F32 or MIXED) of a CSR system of rows of
-// similar length in one cooperative launch over the device, the matrix in the
+// A whole solve (CG, BiCGSTAB or CGS; F64, F32 or MIXED; jacobi: with M = diag(A)) of a
+// system of rows of similar length in one cooperative launch over the device, the matrix in the
 // SMs' shared memory (grid_solve.cu); synchronous.  SPX_ERR_UNSUPPORTED (no error
 // message) when the system does not qualify or fit.
 int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, double tol, int64_t maxit,
-               int precision, spx_solve_info *info);
+               int precision, bool jacobi, spx_solve_info *info);
 
 // SPX_ERR_TIMEOUT (with a message; the word is cleared) when a bounded device wait has
 // given up on this context; synchronises the stream (solvers.cu).

@@ -36,7 +36,7 @@ def _t(a):
     return torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
 
 
-def _both(spx, ctx, mat, b, solver, precision, tol, maxit=20000, x0=None, fmt="csr"):
+def _both(spx, ctx, mat, b, solver, precision, tol, maxit=20000, x0=None, fmt="csr", precond=None):
     """(info, x) by the automatic route, solved twice (equal bits), and by the general path."""
     rp, col, val = mat
     f32 = precision == "f32"
@@ -52,7 +52,7 @@ def _both(spx, ctx, mat, b, solver, precision, tol, maxit=20000, x0=None, fmt="c
         xs = []
         for _ in range(1 if pinned else 2):
             x = torch.zeros_like(bt) if x0 is None else _t(x0).to(dt)
-            info = spx.spx_solve(ctx, A, bt, x, solver, tol, maxit, precision=precision)
+            info = spx.spx_solve(ctx, A, bt, x, solver, tol, maxit, precision=precision, precond=precond)
             xs.append(x.double().cpu().numpy())
         if not pinned:
             assert np.array_equal(xs[0], xs[1], equal_nan=True)  # no dependence on timing
@@ -117,6 +117,62 @@ def test_other_formats(spx, ctx, n, solver, precision, fmt):
     assert abs(info.iterations - ginfo.iterations) <= max(4, ginfo.iterations // 5)
     if precision != "f32":
         assert np.linalg.norm(b - oracle.spmv_csr(*mat, x)) / np.linalg.norm(b) <= residual_limit(*mat, b, x, tol)
+
+
+def _graded(n, solver, seed):
+    """S A S with S spread over a decade, so that Jacobi matters; the diagonal of every fifth row in two entries."""
+    rp, col, val = synth.ragged_laplace2d(n, 0.2) if solver == "cg" or n < 40 else synth.DiagDomFamily(n, seed=5).matrix(n)
+    row = np.repeat(np.arange(n), np.diff(rp))
+    s = 10.0 ** np.random.default_rng(seed).uniform(-0.5, 0.5, n)
+    val = s[row] * val * s[col]
+    twice = (col == row) & (row % 5 == 0)
+    count = 1 + twice.astype(np.int64)
+    at = np.repeat(np.arange(len(col)), count)
+    out = np.zeros(n + 1, np.int32)
+    out[1:] = np.cumsum(np.bincount(row, weights=count, minlength=n))
+    return out, col[at].astype(np.int32), val[at] / count[at]
+
+
+@pytest.mark.parametrize("fmt", ["csr", "ell", "coo"])
+@pytest.mark.parametrize("solver", ["cg", "bicgstab", "cgs"])
+@pytest.mark.parametrize("precision", ["f64", "f32", "mixed"])
+@pytest.mark.parametrize("n", [1, 33, 4099, 90001])
+def test_jacobi(spx, ctx, n, solver, precision, fmt):
+    """Jacobi in the launch: as on the general path, over storages, one and two rows per thread."""
+    mat = _graded(n, solver, seed=n)
+    b = oracle.spmv_csr(*mat, synth.uniform_vector(n, seed=3))
+    tol = 1e-4 if precision == "f32" else 1e-10
+    (info, x), (ginfo, gx) = _both(spx, ctx, mat, b, solver, precision, tol, fmt=fmt, precond="jacobi")
+    assert info.status == ginfo.status == spx.SPX_CONVERGED and info.relres_true <= tol
+    assert abs(info.iterations - ginfo.iterations) <= max(4, ginfo.iterations // 5), (info, ginfo)
+    if precision != "f32":
+        assert np.linalg.norm(b - oracle.spmv_csr(*mat, x)) / np.linalg.norm(b) <= residual_limit(*mat, b, x, tol)
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32", "mixed"])
+@pytest.mark.parametrize("solver", ["cg", "bicgstab", "cgs"])
+def test_jacobi_other_ends(spx, ctx, solver, precision):
+    """Without a diagonal M is I; b = 0, the iteration limit and a NaN as on the general path."""
+    n = 5003
+    mat = _graded(n, "cg", seed=1)
+    b = synth.uniform_vector(n, seed=4)
+    (info, x), (ginfo, _) = _both(spx, ctx, mat, np.zeros(n), solver, precision, 1e-4, x0=b, precond="jacobi")
+    assert (info.status, info.iterations) == (ginfo.status, ginfo.iterations) == (spx.SPX_CONVERGED, 0)
+    assert not x.any()
+    (info, x), (ginfo, gx) = _both(spx, ctx, mat, b, solver, precision, 1e-14, maxit=5, precond="jacobi")
+    assert (info.status, info.iterations) == (ginfo.status, ginfo.iterations) == (spx.SPX_MAX_ITER, 5)
+    # five iterations of one recurrence in two orders of summation
+    eps = 2.0 ** -53 if precision == "f64" else 2.0 ** -24
+    assert np.linalg.norm(x - gx) <= 1e4 * eps * np.linalg.norm(gx)
+    bn = b.copy()
+    bn[n // 2] = np.nan
+    (info, x), (ginfo, _) = _both(spx, ctx, mat, bn, solver, precision, 1e-4, maxit=5, precond="jacobi")
+    assert (info.status, info.iterations) == (ginfo.status, ginfo.iterations)
+    shift = (np.arange(n + 1, dtype=np.int32), ((np.arange(n) + 1) % n).astype(np.int32), np.ones(n))  # r . A r = 0
+    e = np.zeros(n)
+    e[3] = 1.0
+    (info, _), (ginfo, _) = _both(spx, ctx, shift, e, solver, precision, 1e-4, maxit=50, precond="jacobi")
+    assert (info.status, info.iterations) == (ginfo.status, ginfo.iterations)
 
 
 @pytest.mark.parametrize("solver", ["cg", "bicgstab", "cgs"])
