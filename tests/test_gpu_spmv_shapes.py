@@ -78,3 +78,10 @@ def test_row_block_small_tiles(spx, ctx, n, dt):
     mat = _random(lens, n)
     assert np.mean(lens) >= 16 and lens.max() <= 2 * np.mean(lens) + 8  # the automatic choice: row-block, two threads
     _check(spx, ctx, mat, "csr", dt)
+
+
+@pytest.mark.parametrize("m", [49, 70])
+@pytest.mark.parametrize("dt", [torch.float64, torch.float32])
+def test_row_block_matrix_copies(spx, ctx, m, dt):
+    """Matrices of 24, 36, 73 and 109 MB (FP32, FP64 by size): the copies' hint changes at half of L2."""
+    _check(spx, ctx, synth.stencil3d_27pt(m), "csr", dt)
