@@ -2020,9 +2020,9 @@ int run_cg_reliable(spx_ctx *ctx, spx_matrix *A, const double *b, double *x, dou
     KrylovRun<float> R{ctx, A, wi, nullptr, d32, true, SPX_CG};
     const int chunk = n < 200000 ? 32 : 16;
     const bool graphs = graphs_for(A);
-    int64_t launched = 0;
     while (status != SPX_CONVERGED) {
         SPX_TRY(read_state<float>(ctx, wi, sizeof(KState<float>)));
+        int64_t launched = 0;  // since the last update, each of which leaves part of a chunk unused
         while (!h->done) {
             const uint64_t key[8] = {(uint64_t)SPX_CG,   (uint64_t)(uintptr_t)d32, 0, 1, (uint64_t)chunk, 4 | (1u << 30),
                                      (uint64_t)(uintptr_t)A, (uint64_t)(uintptr_t)ctx << 1};

@@ -348,3 +348,16 @@ def test_small_mixed_single_launch_route(spx, ctx, solver):
             assert abs(info.restarts - oi.restarts) <= 2, (info, oi)
     finally:
         spx.spx_matrix_destroy(A)
+
+
+def test_mixed_cg_small_limits_general_path(spx, ctx):
+    """Each reliable update leaves part of a chunk of queued iterations unused: a small limit ends the solve as a
+    limit, however many updates came before it."""
+    mat = synth.ragged_laplace2d(5003, 0.2)
+    b = oracle.spmv_csr(*mat, synth.uniform_vector(5003, seed=3))
+    A = _make(spx, ctx, "csr", *mat, flags=spx.SPX_MIXED_SHADOW, kernel=spx.SPX_KERNEL_CSR_ROWS)
+    for maxit in range(1, 60, 3):
+        x = torch.zeros(5003, dtype=torch.float64, device=DEV)
+        info = spx.spx_solve(ctx, A, _t(b), x, "cg", 3e-15, maxit, precision="mixed")
+        assert info.iterations == maxit and info.status == spx.SPX_MAX_ITER, info
+    spx.spx_matrix_destroy(A)
