@@ -765,6 +765,10 @@ __device__ __forceinline__ int grid_solve_mixed(GridTeam &tm, const GridRows<R> 
                 SPX_LIVE(tm.sum(r2));
                 const float beta = r2 / rho;
                 rho = maxr2 = r2;
+                if (o.iters >= A.maxit) {  // the iteration that met tol in FP32 was the last allowed
+                    st = SPX_MAX_ITER;
+                    go = false;
+                }
                 SPX_EACH(u)
                 {
                     p[u] = fmaf(beta, p[u], r[u]);

@@ -219,3 +219,19 @@ def test_other_ends(spx, ctx, solver, precision):
     (info, x), (ginfo, _) = _both(spx, ctx, mat, bn, solver, precision, tol, maxit=5)
     assert info.status == ginfo.status and info.iterations == ginfo.iterations
     assert np.isnan(x).any() or info.iterations == 0
+
+
+def test_mixed_cg_iteration_limit(spx, ctx):
+    """A limit that falls on the iteration after which the FP32 residual is below tol but the FP64 one is not: the
+    solve ends there, as on the general path."""
+    n = 5003
+    mat = synth.ragged_laplace2d(n, 0.2)
+    b = _t(oracle.spmv_csr(*mat, synth.uniform_vector(n, seed=3)))
+    A = spx.spx_matrix_create(ctx, "csr", *(_t(a) for a in mat), flags=spx.SPX_MIXED_SHADOW)
+    solve = lambda tol, k: spx.spx_solve(ctx, A, b, torch.zeros_like(b), "cg", tol, k, precision="mixed")
+    for tol in (1e-7, 1e-12, 4e-16, 3e-16, 2e-16, 1.5e-16, 1e-16):  # the last ones about what FP64 can reach
+        full = solve(tol, 200).iterations
+        for k in range(max(1, full - 40), full):
+            info = solve(tol, k)
+            assert (info.status, info.iterations) == (spx.SPX_MAX_ITER, k), (tol, info)
+    spx.spx_matrix_destroy(A)
