@@ -22,6 +22,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "dev_common.cuh"
@@ -60,6 +61,7 @@ template <class T> struct GState {
     int restarts;  // cycles that ended on the estimate but failed the true residual
     int m;
     int reorth;    // the current Arnoldi step needs the second Gram-Schmidt pass
+    int scale_u;   // its dots take t_j u (k_gm_dots)
     long long iters, maxit;
 };
 
@@ -825,7 +827,10 @@ __global__ void __launch_bounds__(kVB)
 // Basis V[k] = base + k*ld, k = 0..m, stored unnormalised past V[0]: v_k = s_k V[k]
 // with s_k = 1 / ||V[k]|| kept beside the Hessenberg matrix, so that no pass over a
 // vector only scales it.  The cycle runs on A / rho, rho = ||A v_0||, so that the
-// stored vectors' norms stay near 1 however A is scaled.  The Arnoldi step j forms
+// stored vectors' norms do not depend on the scale of A as a whole (where ||A v_0||^2
+// is 0 or infinite in T, in FP32 outside about 1e-22 .. 1e19 for ||A v_0||, rho is 1).
+// ||V[j+1]|| = H(j+1, j) is near 1 where A scales the cycle's vectors alike; its
+// square has to be in T's range (FP32: 1e-19 .. 1e19).  The Arnoldi step j forms
 // u = A V[j] in V[j+1], then, with t_j = s_j / rho, classical Gram-Schmidt with
 // selective reorthogonalisation: h1_k = v_k . (t_j u); w = t_j u - V_j h1; and only
 // if that pass cancelled nearly all of the vector (||w|| < ||t_j u|| / 8) a second
@@ -858,6 +863,10 @@ constexpr double kGmReorthKeep2 = 1.0 / 64.0;  // (||w|| / ||t_j u||)^2 below wh
 constexpr int kGmB = 8;  // basis vectors in flight together
 constexpr int kGmDotsBlocks = 2, kGmUpdBlocks = 3, kGmUpdU = 1;  // blocks per SM; U of the update
 template <int KB> constexpr int gm_dots_u = KB == 1 ? 2 : 1;  // U of the dots
+// The first dots take t_j u instead of u where t_j lies outside 1 / lim .. lim: u carries the norm of
+// V[j], so that a product of V[k] and u could leave the range that V[k] and V[j] are in.  A loop of
+// its own, chosen by a flag beside `skip`: with the test in one loop a cycle took 3% longer.
+template <class T> constexpr T gm_scale_lim = sizeof(T) == 8 ? T(1ull << 60) : T(1 << 8);
 
 template <class T> struct GmVec;
 template <> struct GmVec<double> { using V = double2; };
@@ -946,6 +955,7 @@ __global__ void __launch_bounds__(kVB, kGmDotsBlocks)
 {
     constexpr int U = gm_dots_u<KB>;
     using S = GmTile<T, U>;
+    const bool scaled = !second && gs->scale_u != 0;  // (loaded beside skip)
     if (gs->skip || (second && !gs->reorth)) return;
     const T *w = V + (int64_t)(j + 1) * ld;
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -956,29 +966,37 @@ __global__ void __launch_bounds__(kVB, kGmDotsBlocks)
 #pragma unroll
         for (int q = 0; q < kGmB; ++q) acc[g][q] = T(0);
     const int64_t ntiles = (n + S::ROWS - 1) / S::ROWS, nw = (int64_t)gridDim.x * (kVB / 32);
-    for (int64_t t = (int64_t)wp * gridDim.x + blockIdx.x; t < ntiles; t += nw) {
-        const int64_t r0 = t * S::ROWS, left = n - r0;
-        const bool full = left >= S::ROWS;
-        T wv[S::E];
-        gm_load<T, U>(w + r0, lane, full, left, wv);
+    auto tiles = [&](auto scale, T tw) {
+        for (int64_t t = (int64_t)wp * gridDim.x + blockIdx.x; t < ntiles; t += nw) {
+            const int64_t r0 = t * S::ROWS, left = n - r0;
+            const bool full = left >= S::ROWS;
+            T wv[S::E];
+            gm_load<T, U>(w + r0, lane, full, left, wv);
+            if constexpr (decltype(scale)::value) {
 #pragma unroll
-        for (int g = 0; g < KB; ++g) {
-            T v[kGmB][S::E];
+                for (int e = 0; e < S::E; ++e) wv[e] *= tw;
+            }
 #pragma unroll
-            for (int q = 0; q < kGmB; ++q)
-                if (g < KB - 1 || q < last) gm_load<T, U>(V + (int64_t)(g * kGmB + q) * ld + r0, lane, full, left, v[q]);
-            auto add = [&](int q) {
+            for (int g = 0; g < KB; ++g) {
+                T v[kGmB][S::E];
 #pragma unroll
-                for (int e = 0; e < S::E; ++e) acc[g][q] = fma(v[q][e], wv[e], acc[g][q]);
-            };
-            if (g < KB - 1) {
+                for (int q = 0; q < kGmB; ++q)
+                    if (g < KB - 1 || q < last) gm_load<T, U>(V + (int64_t)(g * kGmB + q) * ld + r0, lane, full, left, v[q]);
+                auto add = [&](int q) {
 #pragma unroll
-                for (int q = 0; q < kGmB; ++q) add(q);
-            } else {
-                gm_first(last, add);
+                    for (int e = 0; e < S::E; ++e) acc[g][q] = fma(v[q][e], wv[e], acc[g][q]);
+                };
+                if (g < KB - 1) {
+#pragma unroll
+                    for (int q = 0; q < kGmB; ++q) add(q);
+                } else {
+                    gm_first(last, add);
+                }
             }
         }
-    }
+    };
+    if (scaled) tiles(std::true_type{}, ldcg(sm.s + j) * gs->rinv);
+    else tiles(std::false_type{}, T(1));
     // block sums, eight vectors at a time: warp q adds the block's sums of vector q
     __shared__ T buf[kGmB][kVB];
     static_assert(kGmB == kVB / 32, "a warp per vector of a group");
@@ -1004,7 +1022,7 @@ __global__ void __launch_bounds__(kVB, kGmDotsBlocks)
     } else {
         rinv = gs->rinv;
     }
-    const T tj = second ? T(1) : sm.s[j] * rinv;
+    const T tj = second || scaled ? T(1) : sm.s[j] * rinv;
 #pragma unroll
     for (int g = 0; g < KB; ++g) {
         const int k = g * kGmB + wp;
@@ -1069,7 +1087,9 @@ template <class T> __device__ void gm_finish_column(GState<T> *gs, GSmall<T> sm,
         const T gj = sm.g[j];
         sm.g[j + 1] = -sj * gj;
         sm.g[j] = cj * gj;
-        sm.s[j + 1] = T(1) / hn;  // (not used when hn = 0: the cycle ends)
+        const T sj1 = T(1) / hn, t = sj1 * gs->rinv;  // (not used when hn = 0: the cycle ends)
+        sm.s[j + 1] = sj1;
+        gs->scale_u = t <= gm_scale_lim<T> && t >= T(1) / gm_scale_lim<T> ? 0 : 1;
         gs->iters += 1;
         gs->jdone = j + 1;
         gs->relres = fabs(sm.g[j + 1]) / gs->bnorm;
@@ -1247,6 +1267,7 @@ __global__ void __launch_bounds__(kVB) k_gm_start(int64_t n, T *__restrict__ v0,
         gs->est_conv = 0;
         gs->jdone = 0;
         gs->skip = 0;
+        gs->scale_u = 0;
         sm.s[0] = T(1);
         sm.g[0] = beta;
         for (int k = 1; k <= gs->m; ++k) sm.g[k] = T(0);

@@ -119,3 +119,28 @@ def test_scaled_fp32(spx, ctx, scale):
     a = _relres(spx, ctx, (rp, col, val), b, k, torch.float32)
     c = _relres(spx, ctx, (rp, col, val * scale), b, k, torch.float32)
     assert abs(a - c) <= 200 * (k + 8) * 2.0 ** -24, (a, c)
+
+
+@pytest.mark.parametrize("first,rest", [(1e-14, 1e4), (1e-4, 1e14), (1e10, 1e-7)])
+def test_norms_far_apart_fp32(spx, ctx, first, rest):
+    """A maps e1 -> first e2, e2 -> rest e3, e3 -> rest (e1 + e3), in n / 3 equal blocks: the stored basis vectors'
+    norms lie rest / first = 1e18 or 1e-17 apart, and raw products of their entries leave FP32's range."""
+    blocks = 1000
+    i = 3 * np.arange(blocks)
+    rows = np.concatenate([i, i + 1, i + 2, i + 2])
+    cols = np.concatenate([i + 2, i, i + 1, i + 2])
+    vals = np.concatenate([np.full(blocks, v) for v in (rest, first, rest, rest)])
+    order = np.lexsort((cols, rows))
+    rp = np.zeros(3 * blocks + 1, np.int32)
+    rp[1:] = np.cumsum(np.bincount(rows, minlength=3 * blocks))
+    A = spx.spx_matrix_create(ctx, "csr", _t(rp), _t(cols[order].astype(np.int32)), _t(vals[order]).float())
+    b = np.zeros(3 * blocks)
+    b[i] = 1.0
+    x = torch.zeros(3 * blocks, dtype=torch.float32, device=DEV)
+    spx.spx_solve_fixed(ctx, A, _t(b).float(), x, "gmres", 3, restart=3, precision="f32")
+    spx.spx_matrix_destroy(A)
+    # A x = b: x = (0, -1, 1) / rest, to the roundings of three steps, row by row of A: the error of e1's coefficient
+    # weighs `first`, that of the others `rest`
+    err = x.double().cpu().numpy() - np.tile([0.0, -1.0, 1.0], blocks) / rest
+    err[i] *= first / rest
+    assert np.abs(err).max() * rest <= 100 * 2.0 ** -24, err[:3] * rest
