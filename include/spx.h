@@ -515,8 +515,11 @@ int spx_probe_gather(spx_ctx *ctx, int64_t nnz, const int32_t *col_idx, const vo
 /* Test hook for the failure path: launch one wait that nothing will satisfy
  * (which = 0: a look-back flag; 1: an mbarrier phase), limited to about a
  * millisecond of SM clocks.  It gives up, records the error and returns, so
- * the following spx_ctx_check reports SPX_ERR_TIMEOUT.  Nothing hangs or
- * faults.  Asynchronous.  Errors: SPX_ERR_INVALID. */
+ * the following spx_ctx_check reports SPX_ERR_TIMEOUT.  Asynchronous.
+ * which = 2: such a wait in one block of a one-launch solve, whose other block
+ * reports a converged result; synchronous, returns what the solve would:
+ * SPX_ERR_TIMEOUT, the error cleared.  Nothing hangs or faults.  Errors:
+ * SPX_ERR_INVALID. */
 int spx_selftest_wait_timeout(spx_ctx *ctx, int which);
 
 /* ------------------------------------------------------------------ errors */

@@ -42,7 +42,57 @@ constexpr int64_t kGridCgRowsMixed = 1280;
 constexpr int64_t kGridRows = 512;
 constexpr size_t kGridWordBytes = grid_words(kGridMaxBlocks) * 8;
 
+// The record of a launch on the context's stream; an error unless block 0 finished and no block reported any.
+int grid_result(spx_ctx *ctx, const GridOut *out, GridOut &h)
+{
+    SPX_CUDA(cudaMemcpyAsync(&h, out, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
+    SPX_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (h.done && !h.err) return SPX_OK;
+    return check_dev_err(ctx) != SPX_OK ? SPX_ERR_TIMEOUT : fail(SPX_ERR_CUDA, "the solve did not finish");
+}
+
+// Block 0 reports a result while block 1 waits, for a millisecond, for a sum that block 0 has no part in.
+__global__ void k_grid_selftest(GridArgs A)
+{
+    __shared__ double buf[2 * kGridBlockMax], total[4];
+    __shared__ int s_dead;
+    GridTeam tm;
+    tm.words = A.words;
+    tm.buf = buf;
+    tm.total = total;
+    tm.s_dead = &s_dead;
+    tm.limit = 2000000;
+    if (threadIdx.x == 0) s_dead = 0;
+    __syncthreads();
+    float v = 1.f;
+    const bool ok = blockIdx.x == 0 || tm.sum(v);
+    if (threadIdx.x != 0) return;
+    if (!ok) grid_error(A, DEVERR_QUEUE_TIMEOUT);
+    if (blockIdx.x == 0) grid_report(A, GridOut{1, SPX_CONVERGED, 0, 0u, 0, 0.0, 0.0});
+}
+
 }  // namespace
+
+// See spx_internal.cuh.
+int grid_selftest(spx_ctx *ctx)
+{
+    const size_t words = grid_words(2) * 8;
+    DBuf w;
+    SPX_TRY(dbuf_alloc(ctx, w, words + sizeof(GridOut)));
+    GridArgs g = {};
+    g.words = w.as<unsigned long long>();
+    g.out = reinterpret_cast<GridOut *>(w.as<char>() + words);
+    g.err = ctx->dev_err;
+    cudaError_t e = cudaMemsetAsync(w.p, 0, words + sizeof(GridOut), ctx->stream);
+    if (e == cudaSuccess) {
+        k_grid_selftest<<<2, 32, 0, ctx->stream>>>(g);
+        e = cudaGetLastError();
+    }
+    GridOut h;
+    const int st = e == cudaSuccess ? grid_result(ctx, g.out, h) : cuda_fail(e, "k_grid_selftest");
+    dbuf_free(ctx, w);
+    return st;
+}
 
 // See spx_internal.cuh.
 int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, double tol, int64_t maxit,
@@ -118,9 +168,7 @@ int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, 
                                      : grid_launch<float, float, false>(ctx, g, solver, blocks, threads, r);
     if (st != SPX_OK) return st;
     GridOut h;
-    SPX_CUDA(cudaMemcpyAsync(&h, g.out, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
-    SPX_CUDA(cudaStreamSynchronize(ctx->stream));
-    if (!h.done) return check_dev_err(ctx) != SPX_OK ? SPX_ERR_TIMEOUT : fail(SPX_ERR_CUDA, "the solve did not finish");
+    SPX_TRY(grid_result(ctx, g.out, h));
     info->status = h.status;
     info->iterations = h.iters;
     info->restarts = h.restarts;

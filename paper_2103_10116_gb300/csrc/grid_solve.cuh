@@ -20,8 +20,10 @@
 // in FP64, the SMs' FP64 rate.
 //
 // The launch is cooperative (all blocks resident), so every wait ends; each
-// wait is bounded all the same: one that gives up sets the context's error word
-// and its block leaves the kernel, as do the others when their waits run out.
+// wait is bounded all the same: a block whose wait gives up leaves the kernel, setting
+// the context's error word and the result record's, as do the others when their waits
+// run out; those may have finished, so the host takes a result only from a record
+// without errors.
 #pragma once
 
 #include "dev_common.cuh"
@@ -36,9 +38,13 @@ constexpr int kGridCopies = 16;      // places a block writes its slot to
 constexpr int kGridRestarts = 3;
 constexpr float kGridRuDelta2 = 0.01f;  // reliable updates: delta^2, delta = 0.1 (as run_cg_reliable)
 
-// Result record; done = 1 once block 0 has written it.
+constexpr long long kGridWaitCycles = 2000000000LL;  // a wait's limit, about a second
+
+// Result record, zero at launch: block 0 writes all but err, done = 1 among it; err: any
+// block's errors, and those that the context's word held already.
 struct GridOut {
-    int done, status, restarts, pad;
+    int done, status, restarts;
+    unsigned err;
     long long iters;
     double relres, relres_true;
 };
@@ -76,10 +82,10 @@ struct GridArgs {
 //     for tagged words with the same fences, whose polling slows the fences.
 struct GridTeam {
     unsigned long long *words;
-    unsigned *err;
     double *buf;    // shared: 2 kGridBlockMax
     double *total;  // shared: 4
     int *s_dead;    // shared: a wait gave up
+    long long limit = kGridWaitCycles;
     unsigned epoch = 0, fenced = 0;
 
     static __device__ __forceinline__ void put(unsigned long long *slot, unsigned long long a, unsigned long long b)
@@ -93,11 +99,7 @@ struct GridTeam {
     }
     static __device__ __forceinline__ void fence() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
-    __device__ __forceinline__ void give_up()
-    {
-        atomicOr(err, DEVERR_QUEUE_TIMEOUT);
-        *s_dead = 1;
-    }
+    __device__ __forceinline__ void give_up() { *s_dead = 1; }
 
     // s[q] (valid in warp 0's lanes) = the value of block l + 32 k in a[q][k], all blocks' values
     // ready.  Tagged words: a slot is rewritten two sums later, by when every block has
@@ -139,7 +141,7 @@ struct GridTeam {
 #pragma unroll
                 for (int k = 0; k < NS; ++k)
                     ready = ready && (unsigned)(w0[q][k] >> 32) == epoch && (unsigned)(w1[q][k] >> 32) == epoch;
-            if (!ready && clock64() - t0 > 2000000000LL) {
+            if (!ready && clock64() - t0 > limit) {
                 give_up();
                 break;
             }
@@ -177,7 +179,7 @@ struct GridTeam {
                 unsigned v;
                 asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
                 if ((int)(v - want) >= 0) break;
-                if (clock64() - t0 > 2000000000LL) {
+                if (clock64() - t0 > limit) {
                     give_up();
                     break;
                 }
@@ -830,6 +832,24 @@ template <class V> constexpr size_t grid_smem(int cap)
     return ((size_t)cap * 4 + 15) / 16 * 16 + ((size_t)cap * sizeof(V) + 15) / 16 * 16 + 2 * kGridBlockMax * 8;
 }
 
+__device__ __forceinline__ void grid_error(const GridArgs &A, unsigned bits)
+{
+    atomicOr(A.err, bits);
+    atomicOr(&A.out->err, bits);
+}
+
+// block 0: the result, err left to atomics
+__device__ __forceinline__ void grid_report(const GridArgs &A, const GridOut &o)
+{
+    if (const unsigned before = ldcg(A.err)) grid_error(A, before);
+    A.out->status = o.status;
+    A.out->restarts = o.restarts;
+    A.out->iters = o.iters;
+    A.out->relres = o.relres;
+    A.out->relres_true = o.relres_true;
+    A.out->done = 1;
+}
+
 // T: the precision of b and x; V: of the values the products use (V = float, T = double: mixed)
 template <class T, class V, int SOLVER, int R, bool PRE>
 __global__ void __launch_bounds__(kGridBlockMax, 1) k_grid_solve(GridArgs A)
@@ -841,7 +861,6 @@ __global__ void __launch_bounds__(kGridBlockMax, 1) k_grid_solve(GridArgs A)
     V *sv = reinterpret_cast<V *>(smem + ((size_t)A.cap * 4 + 15) / 16 * 16);
     GridTeam tm;
     tm.words = A.words;
-    tm.err = A.err;
     tm.buf = reinterpret_cast<double *>(reinterpret_cast<unsigned char *>(sv) + ((size_t)A.cap * sizeof(V) + 15) / 16 * 16);
     tm.total = total;
     tm.s_dead = &s_dead;
@@ -888,7 +907,7 @@ __global__ void __launch_bounds__(kGridBlockMax, 1) k_grid_solve(GridArgs A)
                 sv[k] = val[j0 + k];
             }
     }
-    if (!fits && tid == 0) atomicOr(A.err, DEVERR_BOUNDS);  // never, for the matrix the slice was sized for
+    if (!fits && tid == 0) grid_error(A, DEVERR_BOUNDS);  // never, for the matrix the slice was sized for
     __syncthreads();
     // M^-1 = 1 / (the sum of the row's diagonal entries), 1 where that is 0 (k_jacobi_dinv's rule, from
     // the matrix's own values)
@@ -909,11 +928,12 @@ __global__ void __launch_bounds__(kGridBlockMax, 1) k_grid_solve(GridArgs A)
             di[u] = d != 0.0 ? (V)(1.0 / d) : V(1);
         }
     }
-    GridOut o{1, SPX_MAX_ITER, 0, 0, 0, 0.0, 0.0};
+    GridOut o{1, SPX_MAX_ITER, 0, 0u, 0, 0.0, 0.0};
     int st;
     if constexpr (sizeof(T) != sizeof(V)) st = grid_solve_mixed<SOLVER, R, PRE>(tm, G, sc, sv, di, A, j0, o);
     else st = grid_solve_one<T, SOLVER, R, PRE>(tm, G, sc, sv, di, A, o);
-    if (st != kDead && blockIdx.x == 0 && tid == 0) *A.out = o;
+    if (st == kDead && tid == 0) grid_error(A, DEVERR_QUEUE_TIMEOUT);
+    if (st != kDead && blockIdx.x == 0 && tid == 0) grid_report(A, o);
 }
 
 // Launch of one (T, V): grid_f64.cu, grid_f32.cu, grid_mixed.cu.  SPX_ERR_UNSUPPORTED

@@ -3224,10 +3224,15 @@ __global__ void k_selftest_wait(int which, long long limit_cycles, int *never_se
 
 extern "C" int spx_selftest_wait_timeout(spx_ctx *ctx, int which)
 {
-    if (!ctx || (which != 0 && which != 1)) return spx::fail(SPX_ERR_INVALID, "spx_selftest_wait_timeout: bad argument");
+    if (!ctx || which < 0 || which > 2) return spx::fail(SPX_ERR_INVALID, "spx_selftest_wait_timeout: bad argument");
     int prev = 0;
     cudaGetDevice(&prev);
     if (prev != ctx->device) cudaSetDevice(ctx->device);
+    if (which == 2) {
+        const int st = spx::grid_selftest(ctx);
+        if (prev != ctx->device) cudaSetDevice(prev);
+        return st;
+    }
     int *flag = nullptr;
     cudaError_t e = cudaMallocAsync(&flag, 16, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(flag, 0, 16, ctx->stream);

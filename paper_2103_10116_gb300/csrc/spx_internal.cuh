@@ -221,6 +221,8 @@ int cluster_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solve
 // message) when the system does not qualify or fit.
 int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, double tol, int64_t maxit,
                int precision, bool jacobi, spx_solve_info *info);
+// The status of a launch in which one block of such a solve gives up while another reports its result.
+int grid_selftest(spx_ctx *ctx);
 
 // SPX_ERR_TIMEOUT (with a message; the word is cleared) when a bounded device wait has
 // given up on this context; synchronises the stream (solvers.cu).

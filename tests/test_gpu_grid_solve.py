@@ -235,3 +235,17 @@ def test_mixed_cg_iteration_limit(spx, ctx):
             info = solve(tol, k)
             assert (info.status, info.iterations) == (spx.SPX_MAX_ITER, k), (tol, info)
     spx.spx_matrix_destroy(A)
+
+
+def test_pending_error_is_reported(spx, ctx):
+    """A wait that gave up on this context before the solve is reported by it, as on the general path, and cleared."""
+    n = 5003
+    mat = synth.ragged_laplace2d(n, 0.2)
+    A = spx.spx_matrix_create(ctx, "csr", *(_t(a) for a in mat))
+    b, x = _t(synth.uniform_vector(n, seed=3)), torch.zeros(n, dtype=torch.float64, device=DEV)
+    spx.spx_selftest_wait_timeout(ctx, 0)
+    with pytest.raises(spx.SpxError) as ei:
+        spx.spx_solve(ctx, A, b, x, "bicgstab", 1e-10, 1000)
+    assert ei.value.status == spx.SPX_ERR_TIMEOUT
+    assert spx.spx_solve(ctx, A, b, x, "bicgstab", 1e-10, 1000).status == spx.SPX_CONVERGED
+    spx.spx_matrix_destroy(A)
