@@ -516,10 +516,10 @@ int spx_probe_gather(spx_ctx *ctx, int64_t nnz, const int32_t *col_idx, const vo
  * (which = 0: a look-back flag; 1: an mbarrier phase), limited to about a
  * millisecond of SM clocks.  It gives up, records the error and returns, so
  * the following spx_ctx_check reports SPX_ERR_TIMEOUT.  Asynchronous.
- * which = 2: such a wait in one block of a one-launch solve, whose other block
- * reports a converged result; synchronous, returns what the solve would:
- * SPX_ERR_TIMEOUT, the error cleared.  Nothing hangs or faults.  Errors:
- * SPX_ERR_INVALID. */
+ * which = 2, 3: such a wait in one block of a one-launch solve (2: over the
+ * device, 3: on a cluster), whose other block reports a converged result;
+ * synchronous, returns what the solve would: SPX_ERR_TIMEOUT, the error
+ * cleared.  Nothing hangs or faults.  Errors: SPX_ERR_INVALID. */
 int spx_selftest_wait_timeout(spx_ctx *ctx, int which);
 
 /* ------------------------------------------------------------------ errors */

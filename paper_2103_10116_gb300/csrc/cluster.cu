@@ -232,6 +232,7 @@ template <int CL> struct PushSum {
     unsigned *err;
     int *dead;            // shared
     unsigned count = 0;
+    long long limit = 2000000000LL;  // clocks a wait may take, about a second
 
     static __device__ __forceinline__ uint32_t remote(uint32_t addr, uint32_t rank)
     {
@@ -280,7 +281,7 @@ template <int CL> struct PushSum {
                     : "r"(smem_addr(&bar[set])), "r"(parity)
                     : "memory");
                 ok = done != 0u;
-            } while (!ok && clock64() - t0 < 2000000000LL);
+            } while (!ok && clock64() - t0 < limit);
             if (!ok && l == 0) {
                 atomicOr(err, DEVERR_MBAR_TIMEOUT);
                 *dead = 1;
@@ -306,6 +307,27 @@ template <int CL> struct PushSum {
         return sum<T, BLOCK>(v, none, [](T s) { return s; });
     }
 };
+
+// A block is done with the cluster: tells every block, with its outcome, and stays until all are
+// done, so that no one pushes to, or reads from, a block that has left.  A block whose wait
+// gave up comes here early; its barriers here pair with the others' barriers in the solve, whose
+// own waits then give up in turn.  Returns whether every block succeeded.  gone: shared, 0 before
+// the first barrier of the kernel; thread 0 alone reads it, so that the block's threads
+// leave by the same barrier.
+template <int CL> __device__ __forceinline__ bool leave_cluster(cg::cluster_group &cl, bool ok, int *gone)
+{
+    __shared__ int seen;
+    __syncthreads();
+    if (threadIdx.x < CL) atomicAdd(cl.map_shared_rank(gone, threadIdx.x), ok ? 1 : 0x10001);
+    for (int k = 0; k < (1 << 20); ++k) {
+        cl.sync();
+        if (threadIdx.x == 0) seen = *(volatile int *)gone;
+        __syncthreads();
+        if ((seen & 0xffff) == CL) break;
+        __syncthreads();
+    }
+    return seen >> 16 == 0;
+}
 
 // the entry at a cluster shared-memory address, 0 where !take
 template <class T> __device__ __forceinline__ T ld_cluster(uint32_t addr, bool take)
@@ -379,9 +401,10 @@ __global__ void __launch_bounds__(BLOCK, 1)
     uint32_t *sa = reinterpret_cast<uint32_t *>(sv + cap);  // cap addresses
     __shared__ uint64_t bar[2];
     __shared__ double slots[2 * CL], buf[BLOCK], tot[2];
-    __shared__ int dead;
+    __shared__ int dead, gone;
     PushSum<CL> ps_sum{bar, slots, tot, buf, err, &dead};
     if (tid == 0) {
+        gone = 0;
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
         fence_barrier_init();
@@ -496,11 +519,41 @@ __global__ void __launch_bounds__(BLOCK, 1)
     }
     SPX_EACH(u) x[r0 + tid + u * BLOCK] = xr[u];
 #undef SPX_EACH
-    if (rank == 0 && tid == 0) {
-        if (!ok) res.status = -1;
-        *out = res;
+    if (!leave_cluster<CL>(cl, ok && nz <= cap, &gone)) res.status = -1;
+    if (rank == 0 && tid == 0) *out = res;
+}
+
+// Rank 0 reports a result while rank 1 waits, for a millisecond, for a sum that rank 0 has no part in.
+__global__ void k_cluster_selftest(ClOut *out, unsigned *err)
+{
+    constexpr int CL = 2, BLOCK = 32;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ uint64_t bar[2];
+    __shared__ double slots[2 * CL], buf[BLOCK], tot[2];
+    __shared__ int dead, gone;
+    PushSum<CL> ps_sum{bar, slots, tot, buf, err, &dead};
+    ps_sum.limit = 2000000;
+    if (threadIdx.x == 0) {
+        gone = dead = 0;
+        mbar_init(&bar[0], 1);
+        mbar_init(&bar[1], 1);
+        fence_barrier_init();
     }
-    cl.sync();  // no block leaves while another may still read its shared memory
+    cl.sync();
+    float v = 1.f;
+    const bool ok = cl.block_rank() == 0 || ps_sum.template sum<float, BLOCK>(v);
+    ClOut res{SPX_CONVERGED, 0, 0, 0.0};
+    if (!leave_cluster<CL>(cl, ok, &gone)) res.status = -1;
+    if (cl.block_rank() == 0 && threadIdx.x == 0) *out = res;
+}
+
+// The record of a launch on the context's stream; an error unless every block succeeded.
+int cluster_result(spx_ctx *ctx, const ClOut *out, ClOut &h)
+{
+    SPX_CUDA(cudaMemcpyAsync(&h, out, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
+    SPX_CUDA(cudaStreamSynchronize(ctx->stream));
+    if (h.status >= 0) return SPX_OK;
+    return check_dev_err(ctx) != SPX_OK ? SPX_ERR_TIMEOUT : fail(SPX_ERR_CUDA, "the solve did not finish");
 }
 
 }  // namespace
@@ -652,6 +705,29 @@ bool cluster_cg_on_chip(const spx_ctx *ctx, const spx_matrix *A)
     return A->dtype == SPX_F64 ? push_takes<double>(ctx, A) : push_takes<float>(ctx, A);
 }
 
+// See spx_internal.cuh.
+int cluster_selftest(spx_ctx *ctx)
+{
+    DBuf w;
+    SPX_TRY(dbuf_alloc(ctx, w, kOutBytes));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2);
+    cfg.blockDim = dim3(32);
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_cluster_selftest, w.as<ClOut>(), ctx->dev_err);
+    ClOut h;
+    const int st = e == cudaSuccess ? cluster_result(ctx, w.as<ClOut>(), h) : cuda_fail(e, "k_cluster_selftest");
+    dbuf_free(ctx, w);
+    return st;
+}
+
 // CG on one cluster (see the file comment); synchronous.  b, x: device, dtype
 // of A (FP64 or FP32); x holds the initial guess.  SPX_ERR_UNSUPPORTED when
 // the matrix is not a CSR matrix of at most cluster_cg_max_rows() rows or no
@@ -669,9 +745,7 @@ int cluster_cg_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, double
                                                  maxit, out);
     if (st != SPX_OK) return st;
     ClOut h;
-    SPX_CUDA(cudaMemcpyAsync(&h, out, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
-    SPX_CUDA(cudaStreamSynchronize(ctx->stream));
-    if (h.status < 0) return check_dev_err(ctx) != SPX_OK ? SPX_ERR_TIMEOUT : fail(SPX_ERR_CUDA, "the solve did not finish");
+    SPX_TRY(cluster_result(ctx, out, h));
     info->status = h.status;
     info->iterations = h.iters;
     info->restarts = h.restarts;

@@ -3224,12 +3224,12 @@ __global__ void k_selftest_wait(int which, long long limit_cycles, int *never_se
 
 extern "C" int spx_selftest_wait_timeout(spx_ctx *ctx, int which)
 {
-    if (!ctx || which < 0 || which > 2) return spx::fail(SPX_ERR_INVALID, "spx_selftest_wait_timeout: bad argument");
+    if (!ctx || which < 0 || which > 3) return spx::fail(SPX_ERR_INVALID, "spx_selftest_wait_timeout: bad argument");
     int prev = 0;
     cudaGetDevice(&prev);
     if (prev != ctx->device) cudaSetDevice(ctx->device);
-    if (which == 2) {
-        const int st = spx::grid_selftest(ctx);
+    if (which >= 2) {
+        const int st = which == 2 ? spx::grid_selftest(ctx) : spx::cluster_selftest(ctx);
         if (prev != ctx->device) cudaSetDevice(prev);
         return st;
     }

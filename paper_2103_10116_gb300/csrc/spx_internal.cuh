@@ -209,6 +209,8 @@ int cluster_cg_max_rows();
 bool cluster_cg_on_chip(const spx_ctx *ctx, const spx_matrix *A);
 int cluster_cg_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, double tol, int64_t maxit,
                      spx_solve_info *info);
+// The status of a launch in which one block of a cluster gives up while another reports its result.
+int cluster_selftest(spx_ctx *ctx);
 // A whole solve (CG, BiCGSTAB or CGS; F64, F32 or MIXED) of a CSR system in one
 // launch on one thread-block cluster, vectors in global memory (cluster.cu);
 // synchronous.  SPX_ERR_UNSUPPORTED when no cluster fits the device.

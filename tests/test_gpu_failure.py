@@ -51,10 +51,11 @@ def test_bounded_wait_reports_timeout_and_context_survives(spx, ctx, which):
         spx.spx_matrix_destroy(A)
 
 
-def test_one_launch_solve_reports_a_block_that_gave_up(spx, ctx):
+@pytest.mark.parametrize("which", [2, 3], ids=["device", "cluster"])
+def test_one_launch_solve_reports_a_block_that_gave_up(spx, ctx, which):
     """A result that one block reported does not count when another block's wait ran out."""
     with pytest.raises(spx.SpxError) as ei:
-        spx.spx_selftest_wait_timeout(ctx, 2)
+        spx.spx_selftest_wait_timeout(ctx, which)
     assert ei.value.status == spx.SPX_ERR_TIMEOUT
     spx.spx_ctx_check(ctx)  # cleared
 
