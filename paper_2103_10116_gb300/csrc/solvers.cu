@@ -2233,6 +2233,8 @@ int solve_entry(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver,
         info->status = SPX_CONVERGED;
         return SPX_OK;
     }
+    if (precision != SPX_PREC_F64 && precision != SPX_PREC_F32 && precision != SPX_PREC_MIXED)
+        return fail(SPX_ERR_INVALID, "spx_solve: unknown precision");  // (the routes below compare it with the dtype only)
     Timer tm;
     int st;
     if (one_cluster) {
@@ -2264,7 +2266,7 @@ int solve_entry(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver,
         if (fixed > 0) return fail(SPX_ERR_UNSUPPORTED, "fixed-iteration mode runs in one precision");
         st = run_ir(ctx, A, static_cast<const double *>(b), static_cast<double *>(x), solver, tol, maxit, restart, pre,
                     bs, adapt, info);
-    } else if (precision == SPX_PREC_F64 || precision == SPX_PREC_F32) {
+    } else {
         const int want = precision == SPX_PREC_F64 ? SPX_F64 : SPX_F32;
         if (A->dtype != want) return fail(SPX_ERR_UNSUPPORTED, "precision must match the matrix dtype (or use MIXED)");
         st = A->dtype == SPX_F64
@@ -2272,8 +2274,6 @@ int solve_entry(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver,
                                        maxit, restart, false, fixed, pre, bs, adapt, info)
                  : solve_typed<float>(ctx, A, static_cast<const float *>(b), static_cast<float *>(x), solver, tol,
                                       maxit, restart, false, fixed, pre, bs, adapt, info);
-    } else {
-        return fail(SPX_ERR_INVALID, "spx_solve: unknown precision");
     }
     info->time_ms = tm.ms();
     return st;

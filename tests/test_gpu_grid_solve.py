@@ -249,3 +249,15 @@ def test_pending_error_is_reported(spx, ctx):
     assert ei.value.status == spx.SPX_ERR_TIMEOUT
     assert spx.spx_solve(ctx, A, b, x, "bicgstab", 1e-10, 1000).status == spx.SPX_CONVERGED
     spx.spx_matrix_destroy(A)
+
+
+@pytest.mark.parametrize("fmt", ["csr", "ell", "coo"])
+@pytest.mark.parametrize("n", [300, 5003, 40009])
+def test_unknown_precision_is_refused(spx, ctx, n, fmt):
+    mat = synth.ragged_laplace2d(n, 0.2)
+    A = spx.spx_matrix_create(ctx, fmt, _t(mat[0]), _t(mat[1]), _t(mat[2]).float())
+    b, x = _t(synth.uniform_vector(n, seed=3)).float(), torch.zeros(n, dtype=torch.float32, device=DEV)
+    with pytest.raises(spx.SpxError) as ei:
+        spx.spx_solve(ctx, A, b, x, "cg", 1e-4, 1000, precision=7)
+    assert ei.value.status == spx.SPX_ERR_INVALID
+    spx.spx_matrix_destroy(A)
