@@ -291,11 +291,11 @@ int spx_spmv_host(spx_ctx *ctx, const spx_matrix *A, const void *x_host, void *y
  *   - The first call on a device sets that device up: it looks up the array's
  *     device address (cudaGetSymbolAddress) and opts the kernel in to its
  *     shared memory; make that first call before any stream capture.
- *   - Every call shares the one array, which keeps the previous call's
- *     contents; calls on one stream leave it ready for the next, and a call on
- *     another stream or under capture clears what it needs.  Calls whose kernels
- *     overlap on the GPU (different streams with no ordering between them)
- *     race on the array and give wrong results; order them on one stream.
+ *   - Every call shares the one array, which keeps the previous calls'
+ *     contents.  Calls whose kernels overlap on the GPU (different streams with
+ *     no ordering between them) race on the array and give wrong results;
+ *     order them on one stream.  Calls made after those have ended are not
+ *     affected.
  *   - The return code reports argument and launch errors only; the work runs
  *     asynchronously.  If one of the kernel's bounded waits gives up (about a
  *     second without progress, which a valid matrix never causes), every
@@ -521,6 +521,11 @@ int spx_probe_gather(spx_ctx *ctx, int64_t nnz, const int32_t *col_idx, const vo
  * synchronous, returns what the solve would: SPX_ERR_TIMEOUT, the error
  * cleared.  Nothing hangs or faults.  Errors: SPX_ERR_INVALID. */
 int spx_selftest_wait_timeout(spx_ctx *ctx, int which);
+
+/* Test hook for spx_spmv_csr_noalloc: fill its array on the current device, in
+ * order on `stream`, with what calls that overlapped can leave there.  Calls
+ * ordered after it give the same results as without it.  Errors: SPX_ERR_CUDA. */
+int spx_selftest_noalloc_spoil(void *stream);
 
 /* ------------------------------------------------------------------ errors */
 

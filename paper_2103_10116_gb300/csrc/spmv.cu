@@ -320,15 +320,15 @@ __device__ __forceinline__ int2 merge_boundary_warp(int n, int nnz, const int *_
 }
 
 // NA > 0: the product straight from a caller's arrays with fixed scratch that keeps the
-// previous call's contents: flags carry the call's number (call[0], raised by the last
-// block), and the last block turns y into NaN if a wait gave up.  NA = 2: every block
-// has one tile and finds its boundaries itself (no tile map, no launch before this one).
+// previous call's contents: flags carry the call's number `call`, and the last block
+// turns y into NaN if a wait gave up.  NA = 2: every block has one tile and finds its
+// boundaries itself (no tile map, no launch before this one).
 template <class T, int BLOCK, int IPT, int NA = 0>
 __global__ void __launch_bounds__(BLOCK)
     k_csr_merge(int n, const int *__restrict__ rp, const int *__restrict__ col,
                 const T *__restrict__ val, const T *__restrict__ x, const int2 *__restrict__ tiles,
                 int ntiles, int *carry_row_g, T *carry_val_g, int *flags, T *partials, unsigned *ticket,
-                unsigned *err, Epi<T> e, unsigned *call = nullptr, int nnz = 0)
+                unsigned *err, Epi<T> e, int call = 0, int nnz = 0)
 {
     using S = MergeShape<T, BLOCK, IPT>;
     constexpr int CH = S::CH;
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(BLOCK)
     bool ok = true;
     bool pending_prefetch = false;
     int2 na = make_int2(0, 0), nb = make_int2(0, 0);  // thread 0: coordinates of the tile after next
-    const int tag = NA ? (int)(ldcg(call) + 1u) : 1;
+    const int tag = NA ? call : 1;
     if constexpr (NA == 2) {
         __shared__ int2 s_own[2];
         if (tid < 64) {
@@ -517,14 +517,13 @@ __global__ void __launch_bounds__(BLOCK)
         mbar_wait(&bar[(it + 1) & 1], (uint32_t)(((it + 1) >> 1) & 1), err, 200000000LL);
     }
     if constexpr (NA > 0) {
-        // the last block to arrive: every block has read call and written its rows
+        // the last block to arrive: every block has written its rows
         if (!last_block(ticket, gridDim.x)) return;
         if (ldcg(err) != 0u) {
             for (int i = tid; i < n; i += BLOCK) e.y[i] = T(NAN);
             __syncthreads();
             if (tid == 0) *err = 0u;
         }
-        if (tid == 0) *call = (unsigned)tag;
     } else {
         if (e.dots) finish_dots<T, BLOCK>(d0, d1, e, partials, ticket);
     }
@@ -2288,7 +2287,7 @@ int launch_merge(spx_ctx *ctx, spx_matrix *A, const T *val, const T *x, const Ep
                     (const int *)A->rp.as<int>(), (const int *)A->col.as<int>(), val, x,
                     (const int2 *)A->tiles.as<int2>(), (int)A->ntiles, A->carry_row.as<int>(), A->carry_val.as<T>(),
                     A->flags.as<int>(), A->partials.as<T>(), A->ticket.as<unsigned>(), ctx->dev_err, e,
-                    (unsigned *)nullptr, 0);
+                    0, 0);
 }
 
 int ensure_hint(spx_ctx *ctx, spx_matrix *A, int ipt)
@@ -3029,21 +3028,25 @@ constexpr int64_t kNoAllocMaxTiles = SPX_NOALLOC_MAX_TILES;
 constexpr size_t kNoAllocBytes = 1u << 20;  // 1 MiB
 
 // scratch layout: tiles int2[max+1] | carry_val 8B[max] | carry_row int[max] | flags int[max] |
-// arrivals, call number; the error word of the bounded waits in the last 64 bytes.  All zero at
-// load.  Calls that follow one another on a stream clear nothing: flags hold call numbers, and
-// the last block of a call leaves arrivals and error word at zero.  A call on another stream
-// than the last one, and a captured one, clear what they need at zero first, so that calls
-// that overlapped by mistake spoil no later one.
+// slots uint2[kNoAllocSlots + 1]: a call's arrivals and the error word of its bounded waits.
+// All zero at load.  The host numbers a device's calls, and a call uses the slot of its number,
+// which its last block leaves at zero: a direct call finds its slot at zero and no flag with its
+// number, whatever the calls before it did, and clears nothing.  (Calls that overlap by mistake
+// spoil one another's carries and tile map, but no later call's.)  A graph replays one
+// number: captured calls share one of their own, clear their flags first, and use the last slot.
+constexpr int kNoAllocSlots = 8192;
+constexpr unsigned kNoAllocCaptured = 0x80000000u;  // the number of captured calls; direct ones: 1 .. 2^31 - 1
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
-static_assert((kNoAllocMaxTiles + 1) * 8 + kNoAllocMaxTiles * (8 + 4 + 4) + 256 <= (int64_t)kNoAllocBytes,
+constexpr int64_t kNoAllocFlagsAt = (kNoAllocMaxTiles + 1) * 8 + kNoAllocMaxTiles * (8 + 4);
+constexpr int64_t kNoAllocSlotsAt = kNoAllocFlagsAt + kNoAllocMaxTiles * 4;
+static_assert(kNoAllocSlotsAt % 8 == 0 && kNoAllocSlotsAt + (kNoAllocSlots + 1) * 8 <= (int64_t)kNoAllocBytes,
               "no-alloc scratch too small for its tile limit");
 
 std::mutex g_noalloc_mu;
 void *g_noalloc_ptr[256];  // device address of the scratch per device, set once
-cudaStream_t g_noalloc_last[256];  // the stream of the device's last call
+unsigned g_noalloc_calls[256];  // number of the device's last direct call
 
-// *clear: the call follows work of another stream, or is captured
-int noalloc_scratch(int dev, cudaStream_t st, void **out, bool *clear)
+int noalloc_scratch(int dev, char **out)
 {
     if (dev < 0 || dev >= 256) return fail(SPX_ERR_INVALID, "device ordinal out of range");
     std::lock_guard<std::mutex> lk(g_noalloc_mu);
@@ -3053,14 +3056,27 @@ int noalloc_scratch(int dev, cudaStream_t st, void **out, bool *clear)
         cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(no-alloc scratch)");
         g_noalloc_ptr[dev] = p;
-        g_noalloc_last[dev] = st;  // the array is zero: the first call clears nothing
     }
-    *out = g_noalloc_ptr[dev];
+    *out = static_cast<char *>(g_noalloc_ptr[dev]);
+    return SPX_OK;
+}
+
+// the number of a call about to be enqueued
+unsigned noalloc_number(int dev, cudaStream_t st)
+{
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
-    *clear = cap != cudaStreamCaptureStatusNone || g_noalloc_last[dev] != st;
-    if (cap == cudaStreamCaptureStatusNone) g_noalloc_last[dev] = st;
-    return SPX_OK;
+    if (cap != cudaStreamCaptureStatusNone) return kNoAllocCaptured;
+    std::lock_guard<std::mutex> lk(g_noalloc_mu);
+    unsigned &k = g_noalloc_calls[dev];
+    k = k + 1 == kNoAllocCaptured ? 1 : k + 1;
+    return k;
+}
+
+unsigned *noalloc_slot(char *scratch, unsigned number)  // arrivals, error word
+{
+    return reinterpret_cast<unsigned *>(scratch + kNoAllocSlotsAt) +
+           2 * (number == kNoAllocCaptured ? kNoAllocSlots : (int)(number % kNoAllocSlots));
 }
 
 // blocks of `kernel` the device holds at once
@@ -3073,15 +3089,13 @@ template <class K> int64_t noalloc_capacity(K kernel, int smem, int sm_count)
 }
 
 template <class T>
-int spmv_noalloc(cudaStream_t st, void *scratch, int64_t n, int64_t nnz, const int *rp, const int *col, const T *val,
-                 const T *x, T *y, int sm_count, unsigned *err, bool clear)
+int spmv_noalloc(int dev, cudaStream_t st, char *scratch, int64_t n, int64_t nnz, const int *rp, const int *col,
+                 const T *val, const T *x, T *y, int sm_count)
 {
-    char *base = static_cast<char *>(scratch);
-    int2 *tiles = reinterpret_cast<int2 *>(base);
-    T *carry_val = reinterpret_cast<T *>(base + (kNoAllocMaxTiles + 1) * 8);
-    int *carry_row = reinterpret_cast<int *>(base + (kNoAllocMaxTiles + 1) * 8 + kNoAllocMaxTiles * 8);
-    int *flags = carry_row + kNoAllocMaxTiles;
-    unsigned *counters = reinterpret_cast<unsigned *>(flags + kNoAllocMaxTiles);  // arrivals, call number
+    int2 *tiles = reinterpret_cast<int2 *>(scratch);
+    T *carry_val = reinterpret_cast<T *>(scratch + (kNoAllocMaxTiles + 1) * 8);
+    int *carry_row = reinterpret_cast<int *>(scratch + (kNoAllocMaxTiles + 1) * 8 + kNoAllocMaxTiles * 8);
+    int *flags = reinterpret_cast<int *>(scratch + kNoAllocFlagsAt);
     Epi<T> e;
     e.y = y;
     using S = MergeShape<T, kMergeBlock, kNoAllocIpt>;
@@ -3092,21 +3106,25 @@ int spmv_noalloc(cudaStream_t st, void *scratch, int64_t n, int64_t nnz, const i
     SPX_TRY(set_smem(one, S1::SMEM));
     const int64_t ntiles = ceil_div(n + nnz, S::TILE), ntiles1 = ceil_div(n + nnz, S1::TILE);
     const bool map = ntiles1 > noalloc_capacity(one, S1::SMEM, sm_count);
-    if (clear) {
+    const unsigned number = noalloc_number(dev, st);
+    const int call = (int)number;
+    unsigned *arrivals = noalloc_slot(scratch, number), *err = arrivals + 1;
+    if (number == kNoAllocCaptured) {
         SPX_CUDA(cudaMemsetAsync(flags, 0, (size_t)(map ? ntiles : ntiles1) * 4, st));
-        SPX_CUDA(cudaMemsetAsync(counters, 0, 4, st));  // (the call number goes on: other flags hold earlier ones)
-        SPX_CUDA(cudaMemsetAsync(err, 0, sizeof(unsigned), st));
+        SPX_CUDA(cudaMemsetAsync(arrivals, 0, 8, st));
+    } else if (number == 1) {  // the first call, and the first after 2^31: no flag with a number to come
+        SPX_CUDA(cudaMemsetAsync(flags, 0, (size_t)kNoAllocMaxTiles * 4, st));
     }
     // the split count is not read back (no synchronisation): always launch cooperatively
     if (!map)
         return launch_k(one, (int)ntiles1, kMergeBlock, S1::SMEM, st, true, (int)n, rp, col, val, x, (const int2 *)nullptr,
-                        (int)ntiles1, carry_row, carry_val, flags, (T *)nullptr, counters, err, e, counters + 1, (int)nnz);
+                        (int)ntiles1, carry_row, carry_val, flags, (T *)nullptr, arrivals, err, e, call, (int)nnz);
     k_merge_tiles<<<(int)ceil_div(ntiles + 1, 256), 256, 0, st>>>((int)n, (int)nnz, rp, S::TILE, S::SLACK, (int)ntiles,
                                                                  tiles, (unsigned *)nullptr);
     SPX_CUDA(cudaGetLastError());
     const int64_t grid = std::min<int64_t>(ntiles, noalloc_capacity(kern, S::SMEM, sm_count));
     return launch_k(kern, (int)grid, kMergeBlock, S::SMEM, st, true, (int)n, rp, col, val, x, (const int2 *)tiles,
-                    (int)ntiles, carry_row, carry_val, flags, (T *)nullptr, counters, err, e, counters + 1, (int)nnz);
+                    (int)ntiles, carry_row, carry_val, flags, (T *)nullptr, arrivals, err, e, call, (int)nnz);
 }
 
 }  // namespace
@@ -3132,22 +3150,46 @@ extern "C" int spx_spmv_csr_noalloc(void *stream, int dtype, int64_t nrows, int6
         return fail(SPX_ERR_INVALID, "spx_spmv_csr_noalloc: row_ptr, col_idx and values must be 16-byte aligned");
     int dev = 0;
     SPX_CUDA(cudaGetDevice(&dev));
-    void *scratch = nullptr;
+    char *scratch = nullptr;
+    SPX_TRY(noalloc_scratch(dev, &scratch));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    bool clear = false;
-    SPX_TRY(noalloc_scratch(dev, st, &scratch, &clear));
     int sms = 0;
     SPX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    unsigned *err = reinterpret_cast<unsigned *>(static_cast<char *>(scratch) + kNoAllocBytes - 64);
     if (nnz == 0) {  // y = 0
         const cudaError_t e = cudaMemsetAsync(y, 0, (size_t)nrows * (dtype == SPX_F64 ? 8 : 4), st);
         return e == cudaSuccess ? SPX_OK : cuda_fail(e, "cudaMemsetAsync");
     }
     if (dtype == SPX_F64)
-        return spmv_noalloc<double>(st, scratch, nrows, nnz, row_ptr, col_idx, static_cast<const double *>(values),
-                                    static_cast<const double *>(x), static_cast<double *>(y), sms, err, clear);
-    return spmv_noalloc<float>(st, scratch, nrows, nnz, row_ptr, col_idx, static_cast<const float *>(values),
-                               static_cast<const float *>(x), static_cast<float *>(y), sms, err, clear);
+        return spmv_noalloc<double>(dev, st, scratch, nrows, nnz, row_ptr, col_idx, static_cast<const double *>(values),
+                                    static_cast<const double *>(x), static_cast<double *>(y), sms);
+    return spmv_noalloc<float>(dev, st, scratch, nrows, nnz, row_ptr, col_idx, static_cast<const float *>(values),
+                               static_cast<const float *>(x), static_cast<float *>(y), sms);
+}
+
+namespace {
+__global__ void k_noalloc_spoil(int *map_and_carries, int *flags, int last, int *captured_slot)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < (int)(spx::kNoAllocFlagsAt / 4); i += gridDim.x * blockDim.x) {
+        map_and_carries[i] = 0x47474747;
+        if (i < spx::kNoAllocMaxTiles) flags[i] = i % 2 ? last : (int)spx::kNoAllocCaptured;
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 2) captured_slot[threadIdx.x] = 5;
+}
+}  // namespace
+
+extern "C" int spx_selftest_noalloc_spoil(void *stream)
+{
+    int dev = 0;
+    SPX_CUDA(cudaGetDevice(&dev));
+    char *scratch = nullptr;
+    SPX_TRY(spx::noalloc_scratch(dev, &scratch));
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const int last = (int)spx::noalloc_number(dev, st);
+    k_noalloc_spoil<<<64, 256, 0, st>>>(reinterpret_cast<int *>(scratch),
+                                        reinterpret_cast<int *>(scratch + spx::kNoAllocFlagsAt), last,
+                                        reinterpret_cast<int *>(spx::noalloc_slot(scratch, spx::kNoAllocCaptured)));
+    SPX_CUDA(cudaGetLastError());
+    return SPX_OK;
 }
 
 // ------------------------------------------------------------------ gather probe

@@ -120,6 +120,7 @@ SIGNATURES = {
     "spx_probe_gather": (_I, [_P, _I64, _P, _P, _I, _P]),
     "spx_ctx_check": (_I, [_P]),
     "spx_selftest_wait_timeout": (_I, [_P, _I]),
+    "spx_selftest_noalloc_spoil": (_I, [_P]),
     "spx_server_pending": (_I, [_P, C.POINTER(C.c_int64), C.POINTER(C.c_int64), C.POINTER(C.c_int64)]),
     "spx_server_destroy": (_I, [_P]),
     "spx_last_error": (C.c_char_p, []),
@@ -520,6 +521,11 @@ def spx_ctx_check(ctx: int):
 
 def spx_selftest_wait_timeout(ctx: int, which: int = 0):
     _check(load().spx_selftest_wait_timeout(ctx, int(which)))
+
+
+def spx_selftest_noalloc_spoil(stream=None):
+    stream = torch.cuda.current_stream() if stream is None else stream
+    _check(load().spx_selftest_noalloc_spoil(stream.cuda_stream))
 
 
 def spx_probe_gather(ctx: int, col_idx: torch.Tensor, x: torch.Tensor, out: torch.Tensor):

@@ -103,3 +103,27 @@ def test_captured(spx, name):
         _, y2, xh2 = _call(spx, "map_route", torch.float64, seed)  # a direct call of another size after a replay
         torch.cuda.synchronize()
         _check("map_route", torch.float64, xh2, y2)
+
+
+@pytest.mark.parametrize("name", ["one_tile_and_one", "long_rows", "map_route"])
+def test_after_overlapping_calls(spx, name):
+    """What overlapping calls can leave in the scratch (their tile map, carries and flags, a captured call's counts)
+    changes no later call: direct ones, on two streams in turn, and the replays of a captured one."""
+    args, y, xh = _call(spx, name, torch.float64, 5)
+    g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=s):
+        spx.spx_spmv_csr_noalloc(*args, y, ncols=args[3].numel(), stream=s)
+    for k in range(4):
+        with torch.cuda.stream(s if k % 2 else torch.cuda.default_stream()):
+            spx.spx_selftest_noalloc_spoil()
+            if k >= 2:
+                y.fill_(float("nan"))
+                g.replay()
+                torch.cuda.synchronize()
+                _check(name, torch.float64, xh, y)
+            _, y1, xh1 = _call(spx, name, torch.float32, 20 + k)
+            _, y2, xh2 = _call(spx, "long_rows", torch.float64, 30 + k)
+            torch.cuda.synchronize()
+        _check(name, torch.float32, xh1, y1)
+        _check("long_rows", torch.float64, xh2, y2)
