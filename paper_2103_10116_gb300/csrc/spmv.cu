@@ -628,10 +628,13 @@ template <class T, int ROWS> struct RowsShape {
     static __host__ __device__ int smem(int cap, int stages) { return stages * stage(cap) + 32 + 16; }
 };
 
-template <class T, int ROWS, int STAGES, int MODE, int TPR>
-__global__ void __launch_bounds__(ROWS * TPR)
+// STREAM: evict-first copies (launch_rows_m says when).  FP32 with several threads per row:
+// registers for 1536 threads per SM; left to itself ptxas took fewer, for 2048, and rows of
+// random columns kept fewer gathers in flight (64 000 rows of 20: 8.45 us, 7.55 with the bound).
+template <class T, int ROWS, int STAGES, int MODE, int TPR, bool STREAM>
+__global__ void __launch_bounds__(ROWS * TPR, sizeof(T) == 4 && TPR > 1 ? 1536 / (ROWS * TPR) : 0)
     k_csr_rows(int n, const int *__restrict__ rp, const int *__restrict__ col, const T *__restrict__ val,
-               const T *__restrict__ x, int ntiles, int cap, bool stream, T *partials, unsigned *ticket, unsigned *err,
+               const T *__restrict__ x, int ntiles, int cap, T *partials, unsigned *ticket, unsigned *err,
                Epi<T> e)
 {
     using S = RowsShape<T, ROWS>;
@@ -651,7 +654,7 @@ __global__ void __launch_bounds__(ROWS * TPR)
     }
     __syncthreads();
 
-    const uint64_t once = stream && tid == 0 ? policy_evict_first() : 0;
+    const uint64_t once = STREAM && tid == 0 ? policy_evict_first() : 0;
     // thread 0 only: copy the tile with rows [r0, r1) and nonzeros [j0, j1) into `stage`
     auto issue = [&](int r0, int r1, int j0, int j1, int stage) {
         unsigned char *base = smem + stage * stage_bytes;
@@ -667,7 +670,7 @@ __global__ void __launch_bounds__(ROWS * TPR)
         s_coord[stage] = make_int4(r0, j0, r1, j1);
         mbar_arrive_expect_tx(&bar[stage], (uint32_t)(rbytes + cbytes + vbytes));
         bulk_g2s(base, rp + ra, (uint32_t)rbytes, &bar[stage]);
-        if (cbytes && stream) {
+        if (STREAM && cbytes) {
             bulk_g2s_once(base + S::RP_BYTES, col + ca, (uint32_t)cbytes, &bar[stage], once);
             bulk_g2s_once(base + S::RP_BYTES + S::col_bytes(cap), val + va, (uint32_t)vbytes, &bar[stage], once);
         } else if (cbytes) {
@@ -2370,7 +2373,13 @@ template <class T, int STAGES, int MODE, int TPR>
 int launch_rows_m(spx_ctx *ctx, spx_matrix *A, const T *val, const T *x, const Epi<T> &e)
 {
     constexpr int rows = rows_tile<T, TPR>;
-    auto kern = k_csr_rows<T, rows, STAGES, MODE, TPR>;
+    // Evict-first copies (bulk_g2s_once) of a matrix above half of L2, which beside the vectors L2 does not keep from
+    // one product to the next; a smaller one is copied plainly.  us, with the hint / without: FP64 27-point 50^3
+    // (39 MB) repeated 14.4 / 12.4, 7-point 80^3 (43 MB) 13.4 / 12.4, its CG 7985 / 7885; CG on 101^3 (85 MB)
+    // 14 020 / 14 640.  Two kernels: with both copies in one, small products were slower (per launch in a graph,
+    // FP32 27-point 11^3 2.54 / 2.47, 55^3 6.74 / 6.63, FP64 10^4 rows of 20 random columns 4.25 / 4.18).
+    auto kern = k_csr_rows<T, rows, STAGES, MODE, TPR, false>;
+    if (2 * A->nnz * (int64_t)(sizeof(T) + 4) > (int64_t)ctx->l2_bytes) kern = k_csr_rows<T, rows, STAGES, MODE, TPR, true>;
     constexpr int block = rows * TPR;
     SPX_TRY(ensure_rows_cap(ctx, A));
     const int64_t cap = rows == kRowsTile ? A->rows_cap : A->rows_cap_small;
@@ -2386,13 +2395,8 @@ int launch_rows_m(spx_ctx *ctx, spx_matrix *A, const T *val, const T *x, const E
     const int64_t ntiles = ceil_div(A->n, rows);
     const int grid = grid_for(ctx, kern, block, (int)smem, ntiles);
     SPX_TRY(ensure_scratch(ctx, A, 0, grid, sizeof(T)));
-    // Evict-first copies (bulk_g2s_once) of a matrix above half of L2, which beside the vectors L2 does not keep from
-    // one product to the next; a smaller one is copied plainly.  us, with the hint / without: FP64 27-point 50^3
-    // (39 MB) repeated 14.4 / 12.4, 7-point 80^3 (43 MB) 13.4 / 12.4, its CG 7985 / 7885; CG on 101^3 (85 MB)
-    // 14 020 / 14 640.
-    const bool stream = 2 * A->nnz * (int64_t)(sizeof(T) + 4) > (int64_t)ctx->l2_bytes;
     kern<<<grid, block, (int)smem, ctx->stream>>>((int)A->n, A->rp.as<int>(), A->col.as<int>(), val, x,
-                                                      (int)ntiles, (int)cap, stream, A->partials.as<T>(),
+                                                      (int)ntiles, (int)cap, A->partials.as<T>(),
                                                       A->ticket.as<unsigned>(), ctx->dev_err, e);
     SPX_CUDA(cudaGetLastError());
     return SPX_OK;
