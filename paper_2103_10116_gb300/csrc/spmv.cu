@@ -2369,17 +2369,30 @@ template <class T> int64_t rows_smem(const spx_matrix *A, int stages)
     return RowsShape<T, kRowsTile>::smem((int)std::min<int64_t>(A->rows_cap, 1 << 24), stages);
 }
 
+// Whether a matrix is read evict-first: when L2 does not hold it beside the vectors from one product to the next.  Read
+// so, it leaves the vectors in L2; read plainly where all fits, it stays there itself.  Vectors: x and y of a product; x,
+// r, p, q of CG (p.q: mode 4 with w = x) and of a residual (7); seven in the other solvers (r^.v, t.s and t.t; GMRES: mode
+// 1 with skip).  us, hint / no hint, by MB of matrix and vectors together (L2: 135.5): products FP32 27-point 64^3 (58) 12.3 / 10.3, 76^3 (98)
+// 18.5 / 16.4, 79^3 (110) 20.5 / 18.6, 82^3 (123) 20.9 / 23.0; FP64 7-point 100^3 (103) 20.5 / 18.5, 105^3 (120) 22.6 /
+// 23.8; ms, CG FP64 7-point 95^3 (102) 10.05 / 9.66, 100^3 (119) 9.22 / 9.58, 27-point 65^3 (96) 4.55 / 4.26, 70^3
+// (120) 5.36 / 5.48; mixed 7-point 105^3 (88) 8.22 / 7.58, 118^3 (124) 10.97 / 12.56; BiCGSTAB FP64 90^3 (104) 13.7 /
+// 13.2, 95^3 (123) 13.1 / 13.4.
+template <class T, int MODE>
+bool past_l2(const spx_ctx *ctx, int64_t n, int64_t matrix_bytes, const T *x, const Epi<T> &e)
+{
+    const int64_t k = MODE == 7 || (MODE == 4 && e.w == x) ? 4 : MODE >= 4 || (MODE == 1 && e.skip) ? 7 : 2;
+    return 6 * (matrix_bytes + k * n * (int64_t)sizeof(T)) > 5 * (int64_t)ctx->l2_bytes;
+}
+
 template <class T, int STAGES, int MODE, int TPR>
 int launch_rows_m(spx_ctx *ctx, spx_matrix *A, const T *val, const T *x, const Epi<T> &e)
 {
     constexpr int rows = rows_tile<T, TPR>;
-    // Evict-first copies (bulk_g2s_once) of a matrix above half of L2, which beside the vectors L2 does not keep from
-    // one product to the next; a smaller one is copied plainly.  us, with the hint / without: FP64 27-point 50^3
-    // (39 MB) repeated 14.4 / 12.4, 7-point 80^3 (43 MB) 13.4 / 12.4, its CG 7985 / 7885; CG on 101^3 (85 MB)
-    // 14 020 / 14 640.  Two kernels: with both copies in one, small products were slower (per launch in a graph,
-    // FP32 27-point 11^3 2.54 / 2.47, 55^3 6.74 / 6.63, FP64 10^4 rows of 20 random columns 4.25 / 4.18).
+    // (two kernels: with both kinds of copies in one, small products were slower; per launch in a graph, FP32 27-point
+    // 11^3 2.54 / 2.47, 55^3 6.74 / 6.63, FP64 10^4 rows of 20 random columns 4.25 / 4.18)
     auto kern = k_csr_rows<T, rows, STAGES, MODE, TPR, false>;
-    if (2 * A->nnz * (int64_t)(sizeof(T) + 4) > (int64_t)ctx->l2_bytes) kern = k_csr_rows<T, rows, STAGES, MODE, TPR, true>;
+    if (past_l2<T, MODE>(ctx, A->n, A->nnz * (int64_t)(sizeof(T) + 4) + 4 * A->n, x, e))
+        kern = k_csr_rows<T, rows, STAGES, MODE, TPR, true>;
     constexpr int block = rows * TPR;
     SPX_TRY(ensure_rows_cap(ctx, A));
     const int64_t cap = rows == kRowsTile ? A->rows_cap : A->rows_cap_small;
