@@ -18,6 +18,7 @@
 #include <climits>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 
 #include "dev_common.cuh"
@@ -1810,14 +1811,18 @@ __global__ void k_row_hint(int n, int nnz, const int *__restrict__ rp, int ipt, 
 // ------------------------------------------------------------------ ELL
 // Column-major ELL [width][ld]: thread g handles rows g*R .. g*R+R-1 and
 // reads R consecutive values of each slab, coalesced across the warp; four
-// slabs' loads are issued together (the last ones too), then their gathers.
-// The slabs are read once (evict-first, so that x and a solver's vectors stay
-// in L2).  Padding slots (col = -1) are skipped.
-// One row per thread at full occupancy (32 registers; six blocks per SM with dots) by default: what the
-// kernel needs is loads in flight, and single rows leave less work in the last
-// round of the grid.  us, against two rows per thread with the last slabs one by
-// one: 7-point 101^3 FP64 21.6 / 26.3, 128^3 38.8 / 43.1, 27-point 100^3 63.8 /
-// 75.9; FP32 7-point 128^3 23.2 / 28.7, 27-point 100^3 40.1 / 44.1.
+// slabs' loads are issued together, then their gathers.  STREAM: the slabs are
+// read evict-first (ell_past_l2 says when).  Padding slots (col = -1) are skipped.
+//   What the kernel needs is loads in flight.  One row per thread at full
+// occupancy (32 registers; six blocks per SM with dots) takes the last slabs
+// four at a time too, and single rows leave less work in the last round of the
+// grid: us, against two rows with the last slabs one by one, 7-point 101^3 FP64
+// 21.6 / 26.3, 128^3 38.8 / 43.1, 27-point 100^3 63.8 / 75.9; FP32 7-point 128^3
+// 23.2 / 28.7.  FP32 from L2 is bound by its load instructions instead: two rows
+// per thread, the last slabs two and one at a time (5-point 500^2 4.1 us, 6.2 with
+// one row; 7-point 60^3 4.1 / 6.2, 27-point 65^3 8.2 / 10.3; CG on 90^3 5.28 / 6.17
+// ms), unless too few rows are left to fill the SMs (10^4 rows of 20 random columns
+// 8.2, 6.2 with one row) or a product streams the matrix (27-point 80^3 22.6 / 20.5).
 template <class T, int R> struct Vec;
 template <> struct Vec<double, 1> { using V = double; using I = int; };
 template <> struct Vec<double, 2> { using V = double2; using I = int2; };
@@ -1825,8 +1830,10 @@ template <> struct Vec<float, 1> { using V = float; using I = int; };
 template <> struct Vec<float, 2> { using V = float2; using I = int2; };
 template <> struct Vec<float, 4> { using V = float4; using I = int4; };
 
-template <class T, int R, int BLOCK, int MODE>
-__global__ void __launch_bounds__(BLOCK, R == 1 ? (MODE == 1 ? 8 : 6) : 1)
+template <class V, bool STREAM> __device__ __forceinline__ V ell_load(const V *p) { return STREAM ? __ldcs(p) : __ldg(p); }
+
+template <class T, int R, int BLOCK, int MODE, bool STREAM>
+__global__ void __launch_bounds__(BLOCK, R == 1 ? (MODE == 1 ? 8 : 6) : R == 2 && sizeof(T) == 4 ? (MODE == 1 ? 6 : 5) : 0)
     k_ell(int64_t n, int64_t ld, int w, const int *__restrict__ ecol, const T *__restrict__ eval,
           const T *__restrict__ x, Epi<T> e, T *partials, unsigned *ticket)
 {
@@ -1849,15 +1856,17 @@ __global__ void __launch_bounds__(BLOCK, R == 1 ? (MODE == 1 ? 8 : 6) : 1)
         T s[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) s[q] = T(0);
-        for (int j = 0; j < w; j += U) {
-            VI c[U];
-            VV v[U];
+        // K slabs from j on, those past the last one as padding
+        auto slabs = [&](auto count, int j) {
+            constexpr int K = decltype(count)::value;
+            VI c[K];
+            VV v[K];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
+            for (int u = 0; u < K; ++u) {
                 const int64_t o = (int64_t)(j + u) * ld + i;
-                if (j + u < w) {
-                    c[u] = __ldcs(reinterpret_cast<const VI *>(ecol + o));
-                    v[u] = __ldcs(reinterpret_cast<const VV *>(eval + o));
+                if (R > 1 || j + u < w) {
+                    c[u] = ell_load<VI, STREAM>(reinterpret_cast<const VI *>(ecol + o));
+                    v[u] = ell_load<VV, STREAM>(reinterpret_cast<const VV *>(eval + o));
                 } else {
 #pragma unroll
                     for (int q = 0; q < R; ++q) {
@@ -1866,16 +1875,16 @@ __global__ void __launch_bounds__(BLOCK, R == 1 ? (MODE == 1 ? 8 : 6) : 1)
                     }
                 }
             }
-            T xg[U][R];
+            T xg[K][R];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
+            for (int u = 0; u < K; ++u) {
                 const int *cc = reinterpret_cast<const int *>(&c[u]);
 #pragma unroll
                 for (int q = 0; q < R; ++q) xg[u][q] = cc[q] >= 0 ? __ldg(x + cc[q]) : T(0);
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (sizeof(T) == 8 && j + u >= w) break;  // (warp-uniform)
+            for (int u = 0; u < K; ++u) {
+                if (R == 1 && sizeof(T) == 8 && j + u >= w) break;  // (warp-uniform)
                 const T *vv = reinterpret_cast<const T *>(&v[u]);
 #pragma unroll
                 for (int q = 0; q < R; ++q) {
@@ -1886,6 +1895,17 @@ __global__ void __launch_bounds__(BLOCK, R == 1 ? (MODE == 1 ? 8 : 6) : 1)
                     }
                 }
             }
+        };
+        if constexpr (R == 1) {
+            for (int j = 0; j < w; j += U) slabs(std::integral_constant<int, U>{}, j);
+        } else {
+            int j = 0;
+            for (; j + U <= w; j += U) slabs(std::integral_constant<int, U>{}, j);
+            if (w - j >= 2) {
+                slabs(std::integral_constant<int, 2>{}, j);
+                j += 2;
+            }
+            if (w > j) slabs(std::integral_constant<int, 1>{}, j);
         }
 #pragma unroll
         for (int q = 0; q < R; ++q)
@@ -2378,10 +2398,10 @@ template <class T> int64_t rows_smem(const spx_matrix *A, int stages)
 // (120) 5.36 / 5.48; mixed 7-point 105^3 (88) 8.22 / 7.58, 118^3 (124) 10.97 / 12.56; BiCGSTAB FP64 90^3 (104) 13.7 /
 // 13.2, 95^3 (123) 13.1 / 13.4.
 template <class T, int MODE>
-bool past_l2(const spx_ctx *ctx, int64_t n, int64_t matrix_bytes, const T *x, const Epi<T> &e)
+bool past_l2(const spx_ctx *ctx, int64_t n, int64_t matrix_bytes, const T *x, const Epi<T> &e, double share = 5.0 / 6)
 {
     const int64_t k = MODE == 7 || (MODE == 4 && e.w == x) ? 4 : MODE >= 4 || (MODE == 1 && e.skip) ? 7 : 2;
-    return 6 * (matrix_bytes + k * n * (int64_t)sizeof(T)) > 5 * (int64_t)ctx->l2_bytes;
+    return (double)(matrix_bytes + k * n * (int64_t)sizeof(T)) > share * (double)ctx->l2_bytes;
 }
 
 template <class T, int STAGES, int MODE, int TPR>
@@ -2768,10 +2788,21 @@ int launch_vector(spx_ctx *ctx, spx_matrix *A, const T *val, const T *x, const E
     return SPX_OK;
 }
 
+// Evict-first loads (k_ell's STREAM): past_l2's rule, from 0.72 of L2 (97.6 MB).  us, with / without, by MB of matrix and
+// vectors (HYB: with its COO part): FP32 27-point 50^3 (28) 8.2 / 6.2, 70^3 (77) 16.4 / 10.3, 7-point 115^3 (97) 16.4 /
+// 14.6, 128^3 (134) 20.7 / 26.7; FP64 95^3 (86) 19.5 / 18.5, 101^3 (103) 20.8 / 21.3, 110^3 (133) 25.0 / 28.7; ms, CG FP64
+// 85^3 (71) 7.31 / 7.23, 95^3 (99) 10.25 / 10.44, 27-point 68^3 (112) 4.71 / 4.91, 7-point 101^3 (119) 10.98 / 11.83.
+template <class T, int MODE> bool ell_past_l2(const spx_ctx *ctx, const spx_matrix *A, const T *x, const Epi<T> &e)
+{
+    return past_l2<T, MODE>(
+        ctx, A->n, A->ell_w * A->ell_ld * (int64_t)(sizeof(T) + 4) + A->coo_nnz * (int64_t)(sizeof(T) + 8), x, e, 0.72);
+}
+
 template <class T, int R, int MODE>
 int launch_ell_m(spx_ctx *ctx, spx_matrix *A, const T *eval, const T *x, const Epi<T> &e)
 {
-    auto kern = k_ell<T, R, kEllBlock, MODE>;
+    auto kern = k_ell<T, R, kEllBlock, MODE, false>;
+    if (ell_past_l2<T, MODE>(ctx, A, x, e)) kern = k_ell<T, R, kEllBlock, MODE, true>;
     const int grid = grid_for(ctx, kern, kEllBlock, 0, ceil_div(ceil_div(A->n, R), kEllBlock));
     SPX_TRY(ensure_scratch(ctx, A, 0, grid, sizeof(T)));
     kern<<<grid, kEllBlock, 0, ctx->stream>>>(A->n, A->ell_ld, (int)A->ell_w, A->ell_col.as<int>(),
@@ -2902,7 +2933,10 @@ template <class T>
 int dispatch_ell(spx_ctx *ctx, spx_matrix *A, const T *eval, const T *x, const Epi<T> &e)
 {
     int p = A->kernel == SPX_KERNEL_ELL ? A->kparam : 0;
-    if (p <= 0) p = 1;  // one row per thread (see k_ell)
+    if (p <= 0) {  // see k_ell
+        const bool two = sizeof(T) == 4 && A->n >= 2LL * kEllBlock * ctx->sm_count;
+        p = two && !(epi_mode(e) <= 1 && ell_past_l2<T, 1>(ctx, A, x, e)) ? 2 : 1;
+    }
     if constexpr (sizeof(T) == 8) {
         if (p == 1) return launch_ell<T, 1>(ctx, A, eval, x, e);
         if (p == 2) return launch_ell<T, 2>(ctx, A, eval, x, e);

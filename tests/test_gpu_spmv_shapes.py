@@ -41,7 +41,7 @@ def _random(lens, seed):
     return rp, rng.integers(0, n, rp[-1]).astype(np.int32), rng.standard_normal(rp[-1])
 
 
-def _check(spx, ctx, mat, fmt, dt):
+def _check(spx, ctx, mat, fmt, dt, rows_per_thread=0):
     rp, col, val = mat
     n = rp.shape[0] - 1
     key = "f64" if dt == torch.float64 else "f32"
@@ -49,6 +49,8 @@ def _check(spx, ctx, mat, fmt, dt):
     xh, yh = synth.uniform_vector(n, 1), synth.uniform_vector(n, 2)
     ref, bound = oracle.spmv_csr(rp, col, r(val), r(xh)), oracle.spmv_absbound(rp, col, r(val), r(xh))
     A = spx.spx_matrix_create(ctx, fmt, _t(rp), _t(col), _t(val).to(dt))
+    if rows_per_thread:
+        spx.spx_matrix_set_kernel(A, spx.SPX_KERNEL_ELL, rows_per_thread)
     y = torch.full((n,), float("nan"), dtype=dt, device=DEV)
     spx.spx_spmv(ctx, A, _t(xh).to(dt), y)
     assert_spmv_close(y.double().cpu().numpy(), ref, bound, TOL[key])
@@ -85,3 +87,19 @@ def test_row_block_small_tiles(spx, ctx, n, dt):
 def test_row_block_matrix_copies(spx, ctx, m, dt):
     """Matrices of 24, 36, 73 and 109 MB (FP32, FP64 by size): the copies' hint changes at half of L2."""
     _check(spx, ctx, synth.stencil3d_27pt(m), "csr", dt)
+
+
+@pytest.mark.parametrize("dt,rows", [(torch.float64, 2), (torch.float32, 2), (torch.float32, 4), (torch.float32, 0)])
+@pytest.mark.parametrize("width", [1, 2, 3, 4, 5, 6, 7, 9])
+def test_ell_several_rows_per_thread(spx, ctx, width, dt, rows):
+    """The last slabs two and one at a time; 0: the automatic choice for as many rows (two in FP32)."""
+    n = 257 if rows else 90001
+    lens = np.random.default_rng(width).integers(0, width + 1, n)
+    lens[-1] = width
+    _check(spx, ctx, _random(lens, n), "ell", dt, rows)
+
+
+@pytest.mark.parametrize("m,dt", [(66, torch.float64), (70, torch.float64), (74, torch.float32), (80, torch.float32)])
+def test_ell_matrix_loads(spx, ctx, m, dt):
+    """Matrices of 93, 111, 88 and 111 MB: plain loads, and evict-first ones."""
+    _check(spx, ctx, synth.stencil3d_27pt(m), "ell", dt)
