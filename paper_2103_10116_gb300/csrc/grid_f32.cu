@@ -2,6 +2,6 @@
 #include "grid_solve.cuh"
 
 namespace spx {
-template int grid_launch<float, float, false>(spx_ctx *, const GridArgs &, int, int, int, int);
-template int grid_launch<float, float, true>(spx_ctx *, const GridArgs &, int, int, int, int);
+template int grid_launch<float, float, false, false>(spx_ctx *, const GridArgs &, int, int, int, int);
+template int grid_launch<float, float, true, false>(spx_ctx *, const GridArgs &, int, int, int, int);
 }

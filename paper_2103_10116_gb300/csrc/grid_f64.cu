@@ -2,6 +2,6 @@
 #include "grid_solve.cuh"
 
 namespace spx {
-template int grid_launch<double, double, false>(spx_ctx *, const GridArgs &, int, int, int, int);
-template int grid_launch<double, double, true>(spx_ctx *, const GridArgs &, int, int, int, int);
+template int grid_launch<double, double, false, false>(spx_ctx *, const GridArgs &, int, int, int, int);
+template int grid_launch<double, double, true, false>(spx_ctx *, const GridArgs &, int, int, int, int);
 }

@@ -3,17 +3,21 @@
 #include "grid_solve.cuh"
 
 #include <algorithm>
+#include <atomic>
 
 namespace spx {
 
-template <class T, class V, bool PRE>
+template <class T, class V, bool PRE, bool COMPACT>
 int grid_launch(spx_ctx *ctx, const GridArgs &A, int solver, int blocks, int threads, int r);
-extern template int grid_launch<double, double, false>(spx_ctx *, const GridArgs &, int, int, int, int);
-extern template int grid_launch<double, double, true>(spx_ctx *, const GridArgs &, int, int, int, int);
-extern template int grid_launch<float, float, false>(spx_ctx *, const GridArgs &, int, int, int, int);
-extern template int grid_launch<float, float, true>(spx_ctx *, const GridArgs &, int, int, int, int);
-extern template int grid_launch<double, float, false>(spx_ctx *, const GridArgs &, int, int, int, int);
-extern template int grid_launch<double, float, true>(spx_ctx *, const GridArgs &, int, int, int, int);
+#define SPX_GRID(T, V)                                                                                \
+    extern template int grid_launch<T, V, false, false>(spx_ctx *, const GridArgs &, int, int, int, int); \
+    extern template int grid_launch<T, V, true, false>(spx_ctx *, const GridArgs &, int, int, int, int);  \
+    extern template int grid_launch<T, V, false, true>(spx_ctx *, const GridArgs &, int, int, int, int);  \
+    extern template int grid_launch<T, V, true, true>(spx_ctx *, const GridArgs &, int, int, int, int);
+SPX_GRID(double, double)
+SPX_GRID(float, float)
+SPX_GRID(double, float)
+#undef SPX_GRID
 
 namespace {
 
@@ -41,6 +45,39 @@ constexpr int64_t kGridCgRowsOff = 4096;  // ... where the cluster does not keep
 constexpr int64_t kGridCgRowsMixed = 1280;
 constexpr int64_t kGridRows = 512;
 constexpr size_t kGridWordBytes = grid_words(kGridMaxBlocks) * 8;
+
+// Solves of this route that are running on each device: with others at its side, a solve takes the
+// COMPACT kernel, which leaves room on the SMs for a second one (its results are the same bits).
+// A cooperative launch waits until all its blocks fit, so without it solves of several contexts
+// ran one after the other.  us per solve, 16 contexts at once, without / with, and alone without /
+// with: CG mixed 46^3 1304 / 778, 1402 / 1507; 63^3 2137 / 1273, 2161 / 2265; FP64 40^3 1604 /
+// 996, 1617 / 1654; BiCGSTAB FP64 35^3 1781 / 775, 1872 / 1830.  Rows of 12 or more entries keep
+// the FP64 pipe or the gathers busy as they are (BiCGSTAB mixed, 30 001 rows of 20: 373 / 577).
+std::atomic<int> g_grid_running[256];
+constexpr double kGridCompactMeanLen = 12.0;
+
+struct Running {
+    std::atomic<int> *n;
+    bool others;
+    explicit Running(int dev) : n(dev >= 0 && dev < 256 ? &g_grid_running[dev] : nullptr)
+    {
+        others = n && n->fetch_add(1) > 0;
+    }
+    ~Running()
+    {
+        if (n) n->fetch_sub(1);
+    }
+};
+
+template <class T, class V>
+int launch(spx_ctx *ctx, const GridArgs &g, bool jacobi, bool compact, int solver, int blocks, int threads, int r)
+{
+    if (compact)
+        return jacobi ? grid_launch<T, V, true, true>(ctx, g, solver, blocks, threads, r)
+                      : grid_launch<T, V, false, true>(ctx, g, solver, blocks, threads, r);
+    return jacobi ? grid_launch<T, V, true, false>(ctx, g, solver, blocks, threads, r)
+                  : grid_launch<T, V, false, false>(ctx, g, solver, blocks, threads, r);
+}
 
 // The record of a launch on the context's stream; an error unless block 0 finished and no block reported any.
 int grid_result(spx_ctx *ctx, const GridOut *out, GridOut &h)
@@ -157,15 +194,12 @@ int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, 
     g.maxit = (long long)maxit;
     SPX_CUDA(cudaMemsetAsync(w, 0, grid_words(blocks) * 8, ctx->stream));
     SPX_CUDA(cudaMemsetAsync(g.out, 0, sizeof(GridOut), ctx->stream));
-    int st;
-    if (jacobi)
-        st = mixed                   ? grid_launch<double, float, true>(ctx, g, solver, blocks, threads, r)
-             : A->dtype == SPX_F64   ? grid_launch<double, double, true>(ctx, g, solver, blocks, threads, r)
-                                     : grid_launch<float, float, true>(ctx, g, solver, blocks, threads, r);
-    else
-        st = mixed                   ? grid_launch<double, float, false>(ctx, g, solver, blocks, threads, r)
-             : A->dtype == SPX_F64   ? grid_launch<double, double, false>(ctx, g, solver, blocks, threads, r)
-                                     : grid_launch<float, float, false>(ctx, g, solver, blocks, threads, r);
+    const Running running(ctx->device);
+    const bool f64 = A->dtype == SPX_F64 && !mixed;
+    const bool compact = running.others && A->mean_len < kGridCompactMeanLen && !(f64 && r == 4);
+    const int st = mixed ? launch<double, float>(ctx, g, jacobi, compact, solver, blocks, threads, r)
+                   : f64 ? launch<double, double>(ctx, g, jacobi, compact, solver, blocks, threads, r)
+                         : launch<float, float>(ctx, g, jacobi, compact, solver, blocks, threads, r);
     if (st != SPX_OK) return st;
     GridOut h;
     SPX_TRY(grid_result(ctx, g.out, h));

@@ -850,9 +850,11 @@ __device__ __forceinline__ void grid_report(const GridArgs &A, const GridOut &o)
     A.out->done = 1;
 }
 
-// T: the precision of b and x; V: of the values the products use (V = float, T = double: mixed)
-template <class T, class V, int SOLVER, int R, bool PRE>
-__global__ void __launch_bounds__(kGridBlockMax, 1) k_grid_solve(GridArgs A)
+// T: the precision of b and x; V: of the values the products use (V = float, T = double: mixed).
+// COMPACT: the same with at most 64 registers per thread, so that the solves of two contexts fit
+// on an SM beside each other; the same operations in the same order, so the same bits.
+template <class T, class V, int SOLVER, int R, bool PRE, bool COMPACT>
+__global__ void __launch_bounds__(kGridBlockMax, COMPACT ? 2 : 1) k_grid_solve(GridArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double total[4];
@@ -936,12 +938,12 @@ __global__ void __launch_bounds__(kGridBlockMax, 1) k_grid_solve(GridArgs A)
     if (st != kDead && blockIdx.x == 0 && tid == 0) grid_report(A, o);
 }
 
-// Launch of one (T, V): grid_f64.cu, grid_f32.cu, grid_mixed.cu.  SPX_ERR_UNSUPPORTED
-// when the device cannot hold the grid at once.
-template <class T, class V, int SOLVER, int R, bool PRE>
+// Launch of one (T, V, COMPACT): grid_f64.cu, grid_f32.cu, grid_mixed.cu and their _compact
+// forms.  SPX_ERR_UNSUPPORTED when the device cannot hold the grid at once.
+template <class T, class V, int SOLVER, int R, bool PRE, bool COMPACT>
 int grid_launch_r(spx_ctx *ctx, const GridArgs &A, int blocks, int threads)
 {
-    auto kern = k_grid_solve<T, V, SOLVER, R, PRE>;
+    auto kern = k_grid_solve<T, V, SOLVER, R, PRE, COMPACT>;
     const size_t smem = grid_smem<V>(A.cap);
     int lim = 0;
     SPX_TRY(smem_optin(reinterpret_cast<const void *>(kern), -1, &lim));
@@ -964,20 +966,21 @@ int grid_launch_r(spx_ctx *ctx, const GridArgs &A, int blocks, int threads)
     return e == cudaSuccess ? SPX_OK : cuda_fail(e, "cudaLaunchKernelEx(k_grid_solve)");
 }
 
-template <class T, class V, int SOLVER, bool PRE>
+template <class T, class V, int SOLVER, bool PRE, bool COMPACT>
 int grid_launch_s(spx_ctx *ctx, const GridArgs &A, int blocks, int threads, int r)
 {
-    if (r == 1) return grid_launch_r<T, V, SOLVER, 1, PRE>(ctx, A, blocks, threads);
-    if (r == 2) return grid_launch_r<T, V, SOLVER, 2, PRE>(ctx, A, blocks, threads);
-    return grid_launch_r<T, V, SOLVER, 4, PRE>(ctx, A, blocks, threads);
+    if (r == 1) return grid_launch_r<T, V, SOLVER, 1, PRE, COMPACT>(ctx, A, blocks, threads);
+    if (r == 2) return grid_launch_r<T, V, SOLVER, 2, PRE, COMPACT>(ctx, A, blocks, threads);
+    if constexpr (COMPACT && sizeof(V) == 8) return SPX_ERR_UNSUPPORTED;  // (spills: no gain)
+    else return grid_launch_r<T, V, SOLVER, 4, PRE, COMPACT>(ctx, A, blocks, threads);
 }
 
-template <class T, class V, bool PRE>
+template <class T, class V, bool PRE, bool COMPACT>
 int grid_launch(spx_ctx *ctx, const GridArgs &A, int solver, int blocks, int threads, int r)
 {
-    if (solver == SPX_CG) return grid_launch_s<T, V, SPX_CG, PRE>(ctx, A, blocks, threads, r);
-    if (solver == SPX_CGS) return grid_launch_s<T, V, SPX_CGS, PRE>(ctx, A, blocks, threads, r);
-    return grid_launch_s<T, V, SPX_BICGSTAB, PRE>(ctx, A, blocks, threads, r);
+    if (solver == SPX_CG) return grid_launch_s<T, V, SPX_CG, PRE, COMPACT>(ctx, A, blocks, threads, r);
+    if (solver == SPX_CGS) return grid_launch_s<T, V, SPX_CGS, PRE, COMPACT>(ctx, A, blocks, threads, r);
+    return grid_launch_s<T, V, SPX_BICGSTAB, PRE, COMPACT>(ctx, A, blocks, threads, r);
 }
 
 }  // namespace spx

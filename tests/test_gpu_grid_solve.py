@@ -5,6 +5,8 @@ which a pinned SpMV kernel keeps: same status, about the same iterations, same
 solution; at the sizes where the partition changes (one, two and four rows per
 thread, the largest system, a ragged last block), for every solver and
 precision, and for the ends of a solve other than convergence."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -261,3 +263,44 @@ def test_unknown_precision_is_refused(spx, ctx, n, fmt):
         spx.spx_solve(ctx, A, b, x, "cg", 1e-4, 1000, precision=7)
     assert ei.value.status == spx.SPX_ERR_INVALID
     spx.spx_matrix_destroy(A)
+
+
+@pytest.mark.parametrize("solver,precision,n,precond", [
+    ("cg", "f64", 40009, None), ("cg", "mixed", 97336, None), ("cg", "f32", 200003, None), ("bicgstab", "f64", 90001, None),
+    ("cgs", "mixed", 70001, None), ("cg", "mixed", 160001, "jacobi"), ("cg", "f64", 250007, None)])
+def test_contexts_at_once(spx, solver, precision, n, precond):
+    """Solves of several contexts and threads at once give the bits of the solve alone: with others running, a solve
+    takes the kernel with fewer registers (three of these sizes at four rows per thread, one of them FP64)."""
+    mat = synth.ragged_laplace2d(n, 0.2)
+    dt = torch.float32 if precision == "f32" else torch.float64
+    b = _t(oracle.spmv_csr(*mat, synth.uniform_vector(n, seed=n))).to(dt)
+    tol = 1e-4 if precision == "f32" else 1e-9
+    args = [_t(mat[0]), _t(mat[1]), _t(mat[2]).to(dt)]
+    flags = spx.SPX_MIXED_SHADOW if precision == "mixed" else 0
+    torch.cuda.synchronize()
+
+    def solves(out, count):
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            c = spx.spx_ctx_create(0, stream=st, allocator="cuda")
+            A = spx.spx_matrix_create(c, "csr", *args, flags=flags)
+            for _ in range(count):
+                x = torch.zeros_like(b)
+                info = spx.spx_solve(c, A, b, x, solver, tol, 20000, precision=precision, precond=precond)
+                out.append((info.status, info.iterations, x.cpu().numpy()))
+            spx.spx_matrix_destroy(A)
+            spx.spx_ctx_destroy(c)
+
+    alone = []
+    solves(alone, 1)
+    assert alone[0][0] == spx.SPX_CONVERGED
+    outs = [[] for _ in range(6)]
+    threads = [threading.Thread(target=solves, args=(o, 4)) for o in outs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for o in outs:
+        assert len(o) == 4
+        for status, iterations, x in o:
+            assert (status, iterations) == alone[0][:2] and np.array_equal(x, alone[0][2])
