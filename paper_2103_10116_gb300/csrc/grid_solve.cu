@@ -32,8 +32,11 @@ constexpr int kGridMinRows32 = 256;
 // cluster.cu) or one SM (the others, the batched kernel as a batch of one), measured
 // in ms, the other route first.  CG FP64: 8100 rows 1.36 / 2.05, 15 625 rows 0.86 / 0.88;
 // 27-point 10 648 rows, whose slices do not fit one cluster, 1.10 / 0.55; FP32: 8100 rows
-// 0.14 / 0.27.  Mixed CG: 900 rows 0.41 / 0.52, 2025 rows 1.02 / 0.74.  BiCGSTAB FP64:
-// 256 rows 0.25 / 0.32, 512 rows 0.50 / 0.40; FP32 the same at 512 rows (0.14).  ELL and COO
+// 0.14 / 0.27.  Against one SM what counts is the entries: mixed CG on 1296 5-point rows (6336
+// entries) 0.44 / 0.50, 1600 rows (7840) 0.56 / 0.57, 1764 rows (8652) 0.71 / 0.55, 1331 27-point rows
+// (29 791) 0.65 / 0.21; mixed BiCGSTAB 1000 7-point rows (6400) 0.24 / 0.26, 1331 rows (8591) 0.36 / 0.25;
+// FP64 729 rows (4617) 0.34 / 0.35, 1000 rows 0.40 / 0.38; 256 rows of 20 0.25 / 0.32, 520 rows 0.49 / 0.38,
+// those with grids for one SM 0.46 / 0.55, 1000 rows 1.01 / 0.85.  ELL and COO
 // have the general path otherwise, slower at every size: CG FP64 on 1600 5-point rows in ELL
 // 3.7 / 0.93, mixed CG on 8100 rows in COO 8.5 / 1.4, CGS on 97 336 7-point rows in ELL 3.6 / 1.9.
 // So has Jacobi: CG FP64 on 400 5-point rows 2.0 / 0.52, on 262 144 7-point rows 6.9 / 4.0, mixed
@@ -42,8 +45,9 @@ constexpr int kGridMinRows32 = 256;
 constexpr int64_t kGridCgRows64 = 14336;
 constexpr int64_t kGridCgRows32 = 16385;
 constexpr int64_t kGridCgRowsOff = 4096;  // ... where the cluster does not keep the matrix on chip
-constexpr int64_t kGridCgRowsMixed = 1280;
 constexpr int64_t kGridRows = 512;
+constexpr int64_t kGridEntries32 = 8192;  // FP32 products (mixed precision among them)
+constexpr int64_t kGridEntries64 = 5632, kGridEntries64Sm = 9216;  // FP64: the first plus the second over the SMs
 constexpr size_t kGridWordBytes = grid_words(kGridMaxBlocks) * 8;
 
 // Solves of this route that are running on each device: with others at its side, a solve takes the
@@ -150,12 +154,13 @@ int grid_solve(spx_ctx *ctx, spx_matrix *A, const void *b, void *x, int solver, 
     if ((double)A->max_len > 2.0 * A->mean_len + 8.0) return SPX_ERR_UNSUPPORTED;
     const int64_t sms = std::min<int64_t>(ctx->grid_sms, kGridMaxBlocks);
     const int64_t from = !csr || jacobi                ? 1  // the small routes take plain CSR only
-                         : solver != SPX_CG            ? kGridRows
-                         : mixed                       ? kGridCgRowsMixed
+                         : solver != SPX_CG || mixed   ? kGridRows
                          : !cluster_cg_on_chip(ctx, A) ? kGridCgRowsOff
                          : precision == SPX_PREC_F64   ? kGridCgRows64
                                                        : kGridCgRows32;
     if (A->n < from) return SPX_ERR_UNSUPPORTED;
+    const int64_t entries = precision == SPX_PREC_F64 ? kGridEntries64 + kGridEntries64Sm / sms : kGridEntries32;
+    if (from == kGridRows && A->nnz < entries) return SPX_ERR_UNSUPPORTED;
     const int64_t min_rows = precision == SPX_PREC_F64 ? kGridMinRows64 : kGridMinRows32;
     const int64_t want = std::min<int64_t>(sms, ceil_div(A->n, min_rows));
     const int64_t rows = (int64_t)round_up((size_t)ceil_div(A->n, want), 32);
