@@ -27,7 +27,8 @@ struct spx_batch {
     spx_ctx *ctx = nullptr;
     int dtype = SPX_F64;
     int64_t nsys = 0, nrows = 0, nnz = 0, max_n = 0;
-    bool wide = false;  // some system's rows are long (krylov_rows.cuh: product_rows_wide)
+    int64_t wide_max_n = 0;  // rows of the largest system whose rows are long (krylov_rows.cuh: product_rows_wide)
+    bool own_size = false;   // a system's product goes by its own size only (the server's batches, the batch of one)
     std::vector<int64_t> row_off, nnz_off;
     spx::DBuf d_row_off, d_nnz_off, rp, col, val, val32, order;
     spx::DBuf work;      // 4 vectors of nrows doubles
@@ -68,7 +69,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
             const int *__restrict__ rp_all, const int *__restrict__ col_all, const T *__restrict__ val_all,
             const float *__restrict__ val32_all, const int *__restrict__ order, const T *__restrict__ b_all,
             T *__restrict__ x_all, T *__restrict__ work, int64_t nrows, T tol, long long maxit, unsigned *queue,
-            BOut out, int smem_vec)
+            BOut out, int smem_vec, int wide_rows)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_sys;
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
         if (q >= nsys) break;
         const int s = order[q];
         const int64_t ro = row_off[s];
-        BlockRows<BLOCK, WIDE> g((int)(row_off[s + 1] - ro));
+        BlockRows<BLOCK, WIDE> g((int)(row_off[s + 1] - ro), wide_rows);
         const SysOut o = solve_rows<T, BLOCK, SOLVER, MIXED>(
             g, rp_all + ro + s, col_all + nnz_off[s], val_all + nnz_off[s], MIXED ? val32_all + nnz_off[s] : nullptr,
             b_all + ro, x_all + ro, work, nrows, ro, smem_vec ? smem : nullptr, tol, maxit);
@@ -94,6 +95,19 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
 }
 
 namespace {
+
+// Rows from which a system of long rows takes several lanes per row.  With one system per SM
+// or less its latency counts, and the shuffles lengthen it: us, a thread per row / several lanes,
+// rows of 20 entries, BiCGSTAB on one system of 200 rows FP64 258 / 309, 600 rows FP64 1144 / 988,
+// mixed 438 / 563, FP32 143 / 181, 1100 rows mixed 1424 / 1367; 150 systems of 600 rows mixed
+// 608 / 721.  With many systems the loads count: 300 of 450 rows FP64 1281 / 1092, mixed 890 / 856,
+// FP32 363 / 356; 1000 of 260 rows FP64 1785 / 1606, mixed 1343 / 1187.
+int wide_rows(const spx_ctx *ctx, const spx_batch *B, bool fp64)
+{
+    if (!B->own_size && B->nsys >= 4 * (int64_t)ctx->sm_count) return 256;
+    if (!B->own_size && 2 * B->nsys >= 3 * (int64_t)ctx->sm_count) return 448;
+    return fp64 ? 576 : 1024;
+}
 
 template <class T, int BLOCK, int SOLVER, bool MIXED, bool WIDE>
 int launch_batch_t(spx_ctx *ctx, spx_batch *B, const T *b, T *x, double tol, int64_t maxit, BOut out,
@@ -123,7 +137,8 @@ int launch_batch_t(spx_ctx *ctx, spx_batch *B, const T *b, T *x, double tol, int
                                 (const int64_t *)B->d_nnz_off.as<int64_t>(), (const int *)B->rp.as<int>(),
                                 (const int *)B->col.as<int>(), (const T *)B->val.as<T>(),
                                 (const float *)B->val32.as<float>(), (const int *)B->order.as<int>(), b, x,
-                                B->work.as<T>(), B->nrows, (T)tol, (long long)maxit, queue, out, smem_vec));
+                                B->work.as<T>(), B->nrows, (T)tol, (long long)maxit, queue, out, smem_vec,
+                                wide_rows(ctx, B, sizeof(T) == 8 && !MIXED)));
     return SPX_OK;
 }
 
@@ -132,8 +147,9 @@ int launch_batch_b(spx_ctx *ctx, spx_batch *B, int block, const T *b, T *x, doub
                    unsigned *queue)
 {
 #define SPX_BATCH(B_)                                                                                     \
-    B->wide ? launch_batch_t<T, B_, SOLVER, MIXED, true>(ctx, B, b, x, tol, maxit, out, queue)            \
-            : launch_batch_t<T, B_, SOLVER, MIXED, false>(ctx, B, b, x, tol, maxit, out, queue)
+    B->wide_max_n >= wide_rows(ctx, B, sizeof(T) == 8 && !MIXED)                                         \
+        ? launch_batch_t<T, B_, SOLVER, MIXED, true>(ctx, B, b, x, tol, maxit, out, queue)               \
+        : launch_batch_t<T, B_, SOLVER, MIXED, false>(ctx, B, b, x, tol, maxit, out, queue)
     switch (block) {
     case 128: return SPX_BATCH(128);
     case 256: return SPX_BATCH(256);
@@ -242,9 +258,9 @@ extern "C" int spx_batch_create(spx_ctx *ctx, spx_batch **out, int dtype, int64_
     B->nrows = nrows;
     B->nnz = nnz;
     B->max_n = max_n;
-    for (int64_t s = 0; s < nsys && !B->wide; ++s) {
+    for (int64_t s = 0; s < nsys; ++s) {
         const int64_t n = row_off[s + 1] - row_off[s];
-        B->wide = n > 0 && nnz_off[s + 1] - nnz_off[s] >= kGroupWideRow * n;
+        if (n > B->wide_max_n && nnz_off[s + 1] - nnz_off[s] >= kGroupWideRow * n) B->wide_max_n = n;
     }
     B->row_off.assign(row_off, row_off + nsys + 1);
     B->nnz_off.assign(nnz_off, nnz_off + nsys + 1);
@@ -396,6 +412,7 @@ int batch_solve_direct(spx_ctx *ctx, spx_batch *B, const void *b, void *x, int s
                        int precision, int block, spx_solve_info *infos)
 {
     if (B->nsys == 0) return SPX_OK;
+    B->own_size = true;
     return batch_solve_impl(ctx, B, b, x, solver, tol, max_iter, precision, infos, block, false);
 }
 

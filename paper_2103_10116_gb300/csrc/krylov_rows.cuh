@@ -32,7 +32,7 @@ constexpr int kGroupMaxRestarts = 3;
 constexpr int kGroupWideRow = 12;  // mean entries per row from which a product takes several lanes per row
 
 // One thread block owns rows [0, n).  WIDE: the kernel also holds the product for long
-// rows (product_rows_wide), which a system takes by its own mean row length; kept out of the
+// rows (product_rows_wide), which a system takes by its own mean row length and size; kept out of the
 // kernels that meet no such system, whose registers it would take (a batch of 4096 2D
 // Laplacians 30.8 ms, 31.3 with it).
 template <int BLOCK, bool WIDE> struct BlockRows {
@@ -40,7 +40,8 @@ template <int BLOCK, bool WIDE> struct BlockRows {
     static constexpr bool kWide = WIDE;
     int lo, hi;
     bool wide = false;
-    __device__ explicit BlockRows(int n) : lo(0), hi(n) {}
+    int wide_rows;  // rows from which a system takes it
+    __device__ BlockRows(int n, int wide_rows) : lo(0), hi(n), wide_rows(wide_rows) {}
     __device__ __forceinline__ void sync() { __syncthreads(); }
     template <class T> __device__ __forceinline__ T sum(T v) { return block_sum<T, BLOCK>(v); }
     template <class T> __device__ __forceinline__ void sum2(T &a, T &b)
@@ -758,7 +759,8 @@ __device__ SysOut solve_rows(G &g, const int *__restrict__ rp, const int *__rest
     T relres = T(0);
     int status;
     int outer = 0;
-    if constexpr (G::kWide) g.wide = rp[g.hi] - rp[g.lo] >= kGroupWideRow * (g.hi - g.lo);
+    if constexpr (G::kWide)
+        g.wide = g.hi - g.lo >= g.wide_rows && rp[g.hi] - rp[g.lo] >= kGroupWideRow * (g.hi - g.lo);
     if constexpr (!MIXED) {
         T *ps = smem_vec ? reinterpret_cast<T *>(smem_vec) : work + 6 * nrows + ro;
         T *w[6];
