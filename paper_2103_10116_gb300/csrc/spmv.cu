@@ -2389,19 +2389,28 @@ template <class T> int64_t rows_smem(const spx_matrix *A, int stages)
     return RowsShape<T, kRowsTile>::smem((int)std::min<int64_t>(A->rows_cap, 1 << 24), stages);
 }
 
-// Whether a matrix is read evict-first: when L2 does not hold it beside the vectors from one product to the next.  Read
-// so, it leaves the vectors in L2; read plainly where all fits, it stays there itself.  Vectors: x and y of a product; x,
-// r, p, q of CG (p.q: mode 4 with w = x) and of a residual (7); seven in the other solvers (r^.v, t.s and t.t; GMRES: mode
-// 1 with skip).  us, hint / no hint, by MB of matrix and vectors together (L2: 135.5): products FP32 27-point 64^3 (58) 12.3 / 10.3, 76^3 (98)
-// 18.5 / 16.4, 79^3 (110) 20.5 / 18.6, 82^3 (123) 20.9 / 23.0; FP64 7-point 100^3 (103) 20.5 / 18.5, 105^3 (120) 22.6 /
-// 23.8; ms, CG FP64 7-point 95^3 (102) 10.05 / 9.66, 100^3 (119) 9.22 / 9.58, 27-point 65^3 (96) 4.55 / 4.26, 70^3
-// (120) 5.36 / 5.48; mixed 7-point 105^3 (88) 8.22 / 7.58, 118^3 (124) 10.97 / 12.56; BiCGSTAB FP64 90^3 (104) 13.7 /
-// 13.2, 95^3 (123) 13.1 / 13.4.
+// Whether a matrix is read evict-first.  Read so, it leaves the vectors in L2; read plainly, it stays there itself from one
+// product to the next, if all fits and nothing else comes between.
+// A solver's products (solver_share: what matrix and vectors may take of L2): the vectors are x, r, p, q of CG (p.q:
+// mode 4 with w = x) and of a residual (7), seven in the other solvers (r^.v, t.s and t.t; GMRES: mode 1 with skip).  ms,
+// hint / no hint, row-block CSR, by MB of all (L2: 135.5): CG FP64 7-point 95^3 (102) 10.05 / 9.66, 100^3 (119) 9.22 / 9.58,
+// 27-point 65^3 (96) 4.55 / 4.26, 70^3 (120) 5.36 / 5.48; mixed 7-point 105^3 (88) 8.22 / 7.58, 118^3 (124) 10.97 / 12.56;
+// BiCGSTAB FP64 90^3 (104) 13.7 / 13.2, 95^3 (123) 13.1 / 13.4; ELL: CG FP64 7-point 85^3 (71) 7.31 / 7.23, 95^3 (99)
+// 10.25 / 10.44, 27-point 68^3 (112) 4.71 / 4.91, 7-point 101^3 (119) 10.98 / 11.83.
+// Products alone (product_share: what the matrix may take): repeated with one matrix the line would lie where L2 is full,
+// with several in turn at L2 over their number; it is taken between.  us, hint / no hint, one matrix and three in turn: CSR
+// FP32 27-point 73^3 (80 MB) 16.4 / 14.4 and 18.0 / 18.6, 79^3 (104) 20.5 / 18.6 and 20.7 / 22.5, FP64 7-point 95^3 (71)
+// 18.5 / 16.4 and 18.5 / 20.0; ELL FP32 27-point 65^3 (59) 12.4 / 8.2 and 14.2 / 16.2, 7-point 95^3 (48) 10.3 / 8.2 and 13.7
+// / 14.3, FP64 5-point 800^2 (38) 11.2 / 10.3 and 13.0 / 14.4, 849^2 (43) 18.9 / 22.2 in turn, 7-point 95^3 (72) 19.5 / 18.5
+// and 18.6 / 20.1.
 template <class T, int MODE>
-bool past_l2(const spx_ctx *ctx, int64_t n, int64_t matrix_bytes, const T *x, const Epi<T> &e, double share = 5.0 / 6)
+bool past_l2(const spx_ctx *ctx, int64_t n, int64_t matrix_bytes, const T *x, const Epi<T> &e, double solver_share,
+             double product_share)
 {
-    const int64_t k = MODE == 7 || (MODE == 4 && e.w == x) ? 4 : MODE >= 4 || (MODE == 1 && e.skip) ? 7 : 2;
-    return (double)(matrix_bytes + k * n * (int64_t)sizeof(T)) > share * (double)ctx->l2_bytes;
+    const bool product = MODE == 0 || (MODE == 1 && !e.skip);
+    const int64_t k = product ? 0 : MODE == 7 || (MODE == 4 && e.w == x) ? 4 : 7;
+    return (double)(matrix_bytes + k * n * (int64_t)sizeof(T)) >
+           (product ? product_share : solver_share) * (double)ctx->l2_bytes;
 }
 
 template <class T, int STAGES, int MODE, int TPR>
@@ -2411,7 +2420,7 @@ int launch_rows_m(spx_ctx *ctx, spx_matrix *A, const T *val, const T *x, const E
     // (two kernels: with both kinds of copies in one, small products were slower; per launch in a graph, FP32 27-point
     // 11^3 2.54 / 2.47, 55^3 6.74 / 6.63, FP64 10^4 rows of 20 random columns 4.25 / 4.18)
     auto kern = k_csr_rows<T, rows, STAGES, MODE, TPR, false>;
-    if (past_l2<T, MODE>(ctx, A->n, A->nnz * (int64_t)(sizeof(T) + 4) + 4 * A->n, x, e))
+    if (past_l2<T, MODE>(ctx, A->n, A->nnz * (int64_t)(sizeof(T) + 4), x, e, 5.0 / 6, 0.5))
         kern = k_csr_rows<T, rows, STAGES, MODE, TPR, true>;
     constexpr int block = rows * TPR;
     SPX_TRY(ensure_rows_cap(ctx, A));
@@ -2788,14 +2797,14 @@ int launch_vector(spx_ctx *ctx, spx_matrix *A, const T *val, const T *x, const E
     return SPX_OK;
 }
 
-// Evict-first loads (k_ell's STREAM): past_l2's rule, from 0.72 of L2 (97.6 MB).  us, with / without, by MB of matrix and
-// vectors (HYB: with its COO part): FP32 27-point 50^3 (28) 8.2 / 6.2, 70^3 (77) 16.4 / 10.3, 7-point 115^3 (97) 16.4 /
-// 14.6, 128^3 (134) 20.7 / 26.7; FP64 95^3 (86) 19.5 / 18.5, 101^3 (103) 20.8 / 21.3, 110^3 (133) 25.0 / 28.7; ms, CG FP64
-// 85^3 (71) 7.31 / 7.23, 95^3 (99) 10.25 / 10.44, 27-point 68^3 (112) 4.71 / 4.91, 7-point 101^3 (119) 10.98 / 11.83.
-template <class T, int MODE> bool ell_past_l2(const spx_ctx *ctx, const spx_matrix *A, const T *x, const Epi<T> &e)
+// Evict-first loads (k_ell's STREAM); HYB counts its COO part.
+template <class T, int MODE>
+bool ell_past_l2(const spx_ctx *ctx, const spx_matrix *A, const T *x, const Epi<T> &e,
+                 double product_share = sizeof(T) == 8 ? 0.27 : 0.5)
 {
     return past_l2<T, MODE>(
-        ctx, A->n, A->ell_w * A->ell_ld * (int64_t)(sizeof(T) + 4) + A->coo_nnz * (int64_t)(sizeof(T) + 8), x, e, 0.72);
+        ctx, A->n, A->ell_w * A->ell_ld * (int64_t)(sizeof(T) + 4) + A->coo_nnz * (int64_t)(sizeof(T) + 8), x, e, 0.72,
+        product_share);
 }
 
 template <class T, int R, int MODE>
@@ -2935,7 +2944,7 @@ int dispatch_ell(spx_ctx *ctx, spx_matrix *A, const T *eval, const T *x, const E
     int p = A->kernel == SPX_KERNEL_ELL ? A->kparam : 0;
     if (p <= 0) {  // see k_ell
         const bool two = sizeof(T) == 4 && A->n >= 2LL * kEllBlock * ctx->sm_count;
-        p = two && !(epi_mode(e) <= 1 && ell_past_l2<T, 1>(ctx, A, x, e)) ? 2 : 1;
+        p = two && !(epi_mode(e) <= 1 && ell_past_l2<T, 1>(ctx, A, x, e, 0.68)) ? 2 : 1;
     }
     if constexpr (sizeof(T) == 8) {
         if (p == 1) return launch_ell<T, 1>(ctx, A, eval, x, e);

@@ -99,7 +99,8 @@ def test_ell_several_rows_per_thread(spx, ctx, width, dt, rows):
     _check(spx, ctx, _random(lens, n), "ell", dt, rows)
 
 
-@pytest.mark.parametrize("m,dt", [(66, torch.float64), (70, torch.float64), (74, torch.float32), (80, torch.float32)])
+@pytest.mark.parametrize("m,dt", [(46, torch.float64), (50, torch.float64), (67, torch.float32), (70, torch.float32),
+                                  (80, torch.float32)])
 def test_ell_matrix_loads(spx, ctx, m, dt):
-    """Matrices of 93, 111, 88 and 111 MB: plain loads, and evict-first ones."""
+    """Matrices of 32, 41, 65, 74 and 111 MB: plain loads; evict-first ones; those at one row per thread in FP32."""
     _check(spx, ctx, synth.stencil3d_27pt(m), "ell", dt)
