@@ -28,7 +28,6 @@ struct spx_batch {
     int dtype = SPX_F64;
     int64_t nsys = 0, nrows = 0, nnz = 0, max_n = 0;
     int64_t wide_max_n = 0;  // rows of the largest system whose rows are long (krylov_rows.cuh: product_rows_wide)
-    bool own_size = false;   // a system's product goes by its own size only (the server's batches, the batch of one)
     std::vector<int64_t> row_off, nnz_off;
     spx::DBuf d_row_off, d_nnz_off, rp, col, val, val32, order;
     spx::DBuf work;      // 4 vectors of nrows doubles
@@ -96,18 +95,15 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK)
 
 namespace {
 
-// Rows from which a system of long rows takes several lanes per row.  With one system per SM
-// or less its latency counts, and the shuffles lengthen it: us, a thread per row / several lanes,
-// rows of 20 entries, BiCGSTAB on one system of 200 rows FP64 258 / 309, 600 rows FP64 1144 / 988,
-// mixed 438 / 563, FP32 143 / 181, 1100 rows mixed 1424 / 1367; 150 systems of 600 rows mixed
-// 608 / 721.  With many systems the loads count: 300 of 450 rows FP64 1281 / 1092, mixed 890 / 856,
-// FP32 363 / 356; 1000 of 260 rows FP64 1785 / 1606, mixed 1343 / 1187.
-int wide_rows(const spx_ctx *ctx, const spx_batch *B, bool fp64)
-{
-    if (!B->own_size && B->nsys >= 4 * (int64_t)ctx->sm_count) return 256;
-    if (!B->own_size && 2 * B->nsys >= 3 * (int64_t)ctx->sm_count) return 448;
-    return fp64 ? 576 : 1024;
-}
+// Rows from which a system of long rows takes several lanes per row (by its own size, so that its
+// result does not depend on its batch).  With one system per SM or less its latency counts, and the
+// shuffles lengthen it: us, a thread per row / several lanes, rows of 20 entries, BiCGSTAB on one
+// system of 200 rows FP64 258 / 309, 600 rows FP64 1144 / 988, mixed 438 / 563, FP32 143 / 181, 1100
+// rows mixed 1424 / 1367; 150 systems of 600 rows mixed 608 / 721.  With many systems the loads count
+// at smaller sizes too: 300 of 450 rows FP64 1281 / 1092, mixed 890 / 856, FP32 363 / 356; 1000 of 260
+// rows FP64 1785 / 1606, mixed 1343 / 1187.  The lines lie between.
+constexpr int kWideRows64 = 512, kWideRows32 = 768;  // FP64 products; FP32 ones, mixed precision among them
+template <class T, bool MIXED> constexpr int wide_rows = sizeof(T) == 8 && !MIXED ? kWideRows64 : kWideRows32;
 
 template <class T, int BLOCK, int SOLVER, bool MIXED, bool WIDE>
 int launch_batch_t(spx_ctx *ctx, spx_batch *B, const T *b, T *x, double tol, int64_t maxit, BOut out,
@@ -138,7 +134,7 @@ int launch_batch_t(spx_ctx *ctx, spx_batch *B, const T *b, T *x, double tol, int
                                 (const int *)B->col.as<int>(), (const T *)B->val.as<T>(),
                                 (const float *)B->val32.as<float>(), (const int *)B->order.as<int>(), b, x,
                                 B->work.as<T>(), B->nrows, (T)tol, (long long)maxit, queue, out, smem_vec,
-                                wide_rows(ctx, B, sizeof(T) == 8 && !MIXED)));
+                                wide_rows<T, MIXED>));
     return SPX_OK;
 }
 
@@ -147,7 +143,7 @@ int launch_batch_b(spx_ctx *ctx, spx_batch *B, int block, const T *b, T *x, doub
                    unsigned *queue)
 {
 #define SPX_BATCH(B_)                                                                                     \
-    B->wide_max_n >= wide_rows(ctx, B, sizeof(T) == 8 && !MIXED)                                         \
+    B->wide_max_n >= wide_rows<T, MIXED>                                                                  \
         ? launch_batch_t<T, B_, SOLVER, MIXED, true>(ctx, B, b, x, tol, maxit, out, queue)               \
         : launch_batch_t<T, B_, SOLVER, MIXED, false>(ctx, B, b, x, tol, maxit, out, queue)
     switch (block) {
@@ -412,7 +408,6 @@ int batch_solve_direct(spx_ctx *ctx, spx_batch *B, const void *b, void *x, int s
                        int precision, int block, spx_solve_info *infos)
 {
     if (B->nsys == 0) return SPX_OK;
-    B->own_size = true;
     return batch_solve_impl(ctx, B, b, x, solver, tol, max_iter, precision, infos, block, false);
 }
 

@@ -94,3 +94,19 @@ def test_wide_systems(spx, ctx, big, solver, precision):
         assert np.array_equal(alone[0], got[0]) and alone_infos[0].iterations == infos[0].iterations
         _, alone = _solve(spx, ctx, mats[-1:], bs[-1:], solver, precision, tol)  # short rows, without the others
         assert np.array_equal(alone[0], got[-1])
+
+
+@pytest.mark.parametrize("precision,line", [("f64", 512), ("f32", 768), ("mixed", 768)])
+@pytest.mark.parametrize("solver", ["cg", "bicgstab"])
+def test_size_line(spx, ctx, solver, precision, line):
+    """Systems of long rows around the size from which they take several lanes per row, beside each other."""
+    mats = [_dominant(n, 14, 70, n, solver == "cg") for n in (line - 1, line, line + 1, line + 33)]
+    tol = 1e-4 if precision == "f32" else 1e-10
+    bs = [oracle.spmv_csr(*m, synth.uniform_vector(m[0].shape[0] - 1, seed=k)) for k, m in enumerate(mats)]
+    infos, got = _solve(spx, ctx, mats, bs, solver, precision, tol)
+    for k, (m, b, i, x) in enumerate(zip(mats, bs, infos, got)):
+        assert i.status == spx.SPX_CONVERGED, i
+        r = np.linalg.norm(b - oracle.spmv_csr(*m, x)) / np.linalg.norm(b)
+        assert r <= tol * 1.001 + (16 * 2.0 ** -24 if precision == "f32" else 0.0), (r, i)  # (as above)
+        _, alone = _solve(spx, ctx, mats[k:k + 1], bs[k:k + 1], solver, precision, tol)
+        assert np.array_equal(alone[0], x)
