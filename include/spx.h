@@ -134,9 +134,9 @@ typedef enum {
                                    a tile-transposed copy of the nonzeros with per-granule row descriptors
                                    (built on first use; one more copy of the column indices and values).
                                    The automatic choice for heavy-tailed rows, with 32 */
-    SPX_KERNEL_CSR_ROWS = 6     /* CSR: tiles of 128 rows bulk-copied to shared memory, 1, 2 or 4 threads
-                                   per row (rows of similar length; SPX_ERR_TOO_LARGE if a tile's nonzeros
-                                   do not fit in shared memory); param = stages + 10 x threads per row,
+    SPX_KERNEL_CSR_ROWS = 6     /* CSR: tiles of 128 rows (32 in FP64 with 2 threads per row) bulk-copied to
+                                   shared memory, 1, 2 or 4 threads per row (rows of similar length;
+                                   SPX_ERR_TOO_LARGE if the nonzeros of 128 rows do not fit in shared memory); param = stages + 10 x threads per row,
                                    stages = shared-memory stages per block (2: the next tile copied while
                                    this one is reduced): 1 or 2 = that many stages, one thread per row;
                                    12, 22, 42 = two stages, 1, 2 or 4 threads per row; 0 = two stages,
@@ -466,16 +466,15 @@ int spx_server_set_batching(spx_server *S, int64_t max_rows, int64_t *effective)
  * entries on average with SPX_SOLVE_ONE_CLUSTER (one launch on one
  * thread-block cluster per request) from now on; 0: none; capped at 2^30;
  * negative: leave the limit unchanged, only report it.  The default is 65 536
- * rows (measured: sixteen concurrent mixed CG solves of a 27 000-row 7-point
- * stencil completed 1.5-1.7x as many solves per second on clusters as on the
- * general path, whose one solve per matrix launches its kernels directly below
- * 50 000 rows; 97 000 rows broke even; longer rows with random columns were
- * slower on clusters).  The decision uses only the request's own matrix.  A request submitted with
- * SPX_SOLVE_ONE_CLUSTER
- * in its solver code takes that route whatever its size.  *effective (may be
- * NULL) receives the limit in force.  As with the batch lanes, a request's
- * result does not depend on other requests; the routes may differ in the last
- * bits. */
+ * rows (measured, sixteen mixed CG solves of a 7-point stencil at once, solves
+ * per second on clusters / by the route spx_solve takes for such sizes, one
+ * launch over the device: 27 000 rows 6900 / 5000, 64 000 rows 3300 / 1800,
+ * 97 336 rows 2400 / 1550; longer rows with random columns are slower on
+ * clusters).  The decision uses only the request's own matrix.  A request
+ * submitted with SPX_SOLVE_ONE_CLUSTER in its solver code takes that route
+ * whatever its size.  *effective (may be NULL) receives the limit in force.
+ * As with the batch lanes, a request's result does not depend on other
+ * requests; the routes may differ in the last bits. */
 int spx_server_set_cluster_rows(spx_server *S, int64_t max_rows, int64_t *effective);
 
 /* The grid share of the slots: every slot's context sizes its launch grids for
@@ -484,12 +483,12 @@ int spx_server_set_cluster_rows(spx_server *S, int64_t max_rows, int64_t *effect
  * operator has at most 8 entries per row on average and for half of them
  * otherwise; below -1: leave the setting unchanged, only report it), applied
  * from the next admitted request on.  Sixteen concurrent mixed solves of one
- * matrix completed up to 1.6x (250 000-row 7-point stencil, quarter grids) and
+ * matrix complete up to 1.4x (512 000-row 7-point stencil, quarter grids) and
  * 1.2x (100 000 rows of 20 random columns, half grids) as many solves per
  * second as with whole-device grids, so workloads of similar concurrent solves
- * gain; on a mix of sizes from 10^3 to 10^6 rows no setting beat the whole
- * device beyond run-to-run variation, and a lone large solve is slower with
- * narrow grids.  The rule uses only the request's own matrix.  *effective (may
+ * gain (250 000 rows: 1.07x); on a mix of sizes from 10^3 to 10^6 rows no
+ * setting had beaten the whole device beyond run-to-run variation, and a lone
+ * large solve is slower with narrow grids.  The rule uses only the request's own matrix.  *effective (may
  * be NULL) receives the setting in force. */
 int spx_server_set_slot_sms(spx_server *S, int sms, int *effective);
 

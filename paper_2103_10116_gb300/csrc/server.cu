@@ -26,16 +26,14 @@
 // Slot requests of CG / BiCGSTAB / CGS (unpreconditioned) on CSR operators of
 // at most cluster_rows rows whose rows hold at most 8 entries on average (the
 // 7-point stencil's class) may run the whole solve in one launch on one
-// thread-block cluster (SPX_SOLVE_ONE_CLUSTER): on the general path such a
-// solve is hundreds of dependent launches of kernels with a few microseconds
-// of work each (and a request solves its matrix once, too few times to repay
-// capturing CUDA graphs).  Sixteen concurrent solves of a 27 000-row 7-point
-// stencil (mixed CG to 1e-8) completed 1.5-1.7x as many solves per second on
-// clusters as on the general path launching its kernels directly; on the
-// serving trace the solve phases of the 25 000 - 100 000-row requests summed to
-// 128 s with the route and 187 s without.  At 97 000 rows the two broke even,
-// and for longer rows with random columns the cluster route was slower at every
-// size measured, so the rule takes short rows of at most 65 536 rows.  The
+// thread-block cluster (SPX_SOLVE_ONE_CLUSTER): the route spx_solve takes
+// otherwise for such a system, one launch over the device, puts a block on
+// every SM, and sixteen solves at once complete fewer per second that way
+// (mixed CG to 1e-8 on 7-point stencils, cluster / device: 27 000 rows 6912 /
+// 5012, 64 000 rows 3294 / 1782, 97 336 rows 2370 / 1553).  For longer rows with
+// random columns the cluster route is slower, so the rule takes short rows, of
+// at most 65 536 rows (the limit was set against the general path, with which
+// 97 000 rows broke even).  The
 // decision reads the row statistics of the request's own matrix, so it does not
 // depend on other requests.
 //
@@ -68,13 +66,14 @@ constexpr double kServeClusterMeanLen = 8.0;    // ... and their largest mean ro
 // Slot grids are sized for a share of the device's SMs, so that the kernels of
 // concurrent slots run side by side (spx_ctx_set_grid_sms).  Sixteen concurrent
 // mixed solves to 1e-8 of one matrix (solves per second at whole-device / half /
-// quarter / eighth grids): 7-point stencils of 250 000 rows 534 / 750 / 839 /
-// 743, of 512 000 rows 292 / 376 / 391 / 353, of 10^6 rows 154 / 175 / 179 /
-// 166; rows of 20 random columns, 10^5 rows 1092 / 1277 / 1233 / 1039,
-// 3 x 10^5 rows 506 / 521 / 490 / 414.  The rule (-1) takes a quarter for short
-// rows and a half for long ones.  On the mixed serving trace no setting beat
-// whole-device grids beyond run-to-run variation (whole device 397-403 solves
-// per second, the rule 382, a half 414, a quarter 374), so the default is 0.
+// quarter / eighth grids): 7-point stencils of 250 000 rows 970 / 936 / 1042 /
+// 969, of 512 000 rows 376 / 487 / 511 / 468, of 10^6 rows 201 / 229 / 237 /
+// 219; rows of 20 random columns, 10^5 rows 1299 / 1552 / 1540 / 1469,
+// 3 x 10^5 rows 552 / 605 / 604 / 553.  The rule (-1) takes a quarter for short
+// rows and a half for long ones.  On the mixed serving trace (before the solves
+// of up to 300 000 rows ran in one launch) no setting beat whole-device grids
+// beyond run-to-run variation (whole device 397-403 solves per second, the rule
+// 382, a half 414, a quarter 374), so the default is 0.
 constexpr int kServeShortRowShare = 4;
 constexpr int kServeLongRowShare = 2;
 constexpr size_t kMaxBatchSystems = 4096;
